@@ -9,11 +9,9 @@
 // double-buffered, so the latency-bound selection of one tile overlaps the
 // bandwidth-bound blend of the previous one:
 //   1. selection (warps 0-3, select_tile.cuh, the same code as qr_select):
-//      the tile's depth-ordered list is staged through shared memory, culled
-//      per warp against the warp's box of pixel centres and walked two pixels
-//      per thread; the kept ids and normalised weights go to one of two
-//      shared-memory buffers and are also written out (coalesced tile-row
-//      runs) for a backward pass;
+//      each warp walks an 8 x 8 block of the tile on its own; the kept ids and
+//      normalised weights go to one of two shared-memory buffers and are also
+//      written out (coalesced runs) for a backward pass;
 //   2. blend (8 warps, warp per 2x2 / 2x1 pixel group and channel chunk, like
 //      qr_blend): equal ids of the group are merged with __match_any_sync, the
 //      group's weights of each distinct row are gathered into a per-warp
@@ -50,80 +48,15 @@ struct BatchView {
     int W, H, tile_w, tiles_x, tiles_y, K;
     float alpha_min, alpha_max;
     uint32_t tile_base;     // first work item of this view
-    uint32_t pad;
+    uint32_t vec;           // ids and weights take 16-byte stores
 };
 
 namespace {
-
-constexpr int T = 256;
-
-template <int DT> struct VecT;
-template <> struct VecT<QR_F32> { static constexpr int C = 4; };
-template <> struct VecT<QR_BF16> { static constexpr int C = 8; };
-template <> struct VecT<QR_FP8E4M3> { static constexpr int C = 16; };
 
 __device__ __forceinline__ void fma2b(float *acc, float w, float x0, float x1) {
     asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %2};\n"
         " mov.b64 xx, {%3, %4};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
         : "+f"(acc[0]), "+f"(acc[1]) : "f"(w), "f"(x0), "f"(x1));
-}
-
-template <int DT>
-__device__ __forceinline__ void dec_fma(const uint4 v, float w, float *acc) {
-    if constexpr (DT == QR_F32) {
-        fma2b(acc + 0, w, __uint_as_float(v.x), __uint_as_float(v.y));
-        fma2b(acc + 2, w, __uint_as_float(v.z), __uint_as_float(v.w));
-    } else if constexpr (DT == QR_BF16) {
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            fma2b(acc + 2 * i, w, __uint_as_float(u[i] << 16), __uint_as_float(u[i] & 0xFFFF0000u));
-    } else {
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const __half2_raw lo = __nv_cvt_fp8x2_to_halfraw2(__nv_fp8x2_storage_t(u[i] & 0xFFFFu), __NV_E4M3);
-            const __half2_raw hi = __nv_cvt_fp8x2_to_halfraw2(__nv_fp8x2_storage_t(u[i] >> 16), __NV_E4M3);
-            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&lo));
-            const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
-            fma2b(acc + 4 * i, w, a.x, a.y);
-            fma2b(acc + 4 * i + 2, w, b.x, b.y);
-        }
-    }
-}
-
-// A 16-byte vector widened to FP32 once (exact for BF16 and E4M3); the group
-// loop then FMAs it into each pixel that lists the row.
-template <int DT>
-__device__ __forceinline__ void dec_vec(const uint4 v, float *o) {
-    if constexpr (DT == QR_F32) {
-        o[0] = __uint_as_float(v.x); o[1] = __uint_as_float(v.y);
-        o[2] = __uint_as_float(v.z); o[3] = __uint_as_float(v.w);
-    } else if constexpr (DT == QR_BF16) {
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            o[2 * i] = __uint_as_float(u[i] << 16);
-            o[2 * i + 1] = __uint_as_float(u[i] & 0xFFFF0000u);
-        }
-    } else {
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const __half2_raw lo = __nv_cvt_fp8x2_to_halfraw2(__nv_fp8x2_storage_t(u[i] & 0xFFFFu), __NV_E4M3);
-            const __half2_raw hi = __nv_cvt_fp8x2_to_halfraw2(__nv_fp8x2_storage_t(u[i] >> 16), __NV_E4M3);
-            const float2 a = __half22float2(*reinterpret_cast<const __half2 *>(&lo));
-            const float2 b = __half22float2(*reinterpret_cast<const __half2 *>(&hi));
-            o[4 * i] = a.x; o[4 * i + 1] = a.y; o[4 * i + 2] = b.x; o[4 * i + 3] = b.y;
-        }
-    }
-}
-
-__device__ __forceinline__ uint4 ldg_nc(const uint4 *p) {
-    uint4 r;
-    asm volatile("ld.global.nc.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
 }
 
 __device__ __forceinline__ void st_cs(float4 *p, float4 v) {
@@ -132,8 +65,8 @@ __device__ __forceinline__ void st_cs(float4 *p, float4 v) {
 }
 
 // ------------------------------------------------------------------ the kernel
-// Warp roles of a CTA: warps 0..3 select (select_tile, 128 threads, two pixels
-// each), warps 4..4+nbw-1 blend (nbw = 4 or 8, from the launch's block size).  Two shared-memory buffers hold a tile's
+// Warp roles of a CTA: warps 0..3 select (select_block, an 8 x 8 block of the
+// tile each), warps 4..4+nbw-1 blend (nbw = 4 or 8, from the launch's block size).  Two shared-memory buffers hold a tile's
 // kept ids, normalised weights and counts; the selection fills one while the
 // blend warps read the other.  Hand-over uses hardware named barriers:
 //   FULL[b]  (ids 2, 3): selection arrives once buffer b holds tile n (or the
@@ -142,9 +75,11 @@ __device__ __forceinline__ void st_cs(float4 *p, float4 v) {
 //                        selection waits before refilling it (from its third
 //                        tile on) and once more after the end marker for the
 //                        last tile's arrival, so every arrival is matched;
-//   id 1:                the selection threads among themselves.
+//   id 1:                the selection threads among themselves, once per
+//                        tile (the item that thread 0 took).
 // Every thread of both roles runs the same number of barrier phases on each
 // id, so no phase is left open and no wait can be missed.
+constexpr int kSelThreads = 128;                      // selection: 4 warps, an 8 x 8 block each
 constexpr int kNBW = 8;                               // blend warps at most
 constexpr int kBT = kSelThreads + 32 * kNBW;          // threads per CTA at most
 constexpr int kItemEnd = -1;
@@ -179,9 +114,8 @@ template <int DT, int QPL, int G, int NCH>
 __global__ void __launch_bounds__(kBT, DT == QR_FP8E4M3 ? 1 : 2)
 batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_items,
              uint32_t *__restrict__ counter, int KSB) {
-    __shared__ SelStage st;
-    __shared__ float s_D[kSelPix];
-    __shared__ uint8_t s_cnt[2][kSelPix];
+    __shared__ SelStage st[kSelThreads / 32];
+    __shared__ float s_thr[kKMax + 1];
     __shared__ int s_item[2];
     __shared__ __align__(16) float s_tw[kNBW][32][G];   // per blend warp: row-weight table
     __shared__ int s_tid[kNBW][32];
@@ -190,10 +124,11 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
     float *s_w0 = reinterpret_cast<float *>(s_dyn) + 2 * kSelPix * KSB;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int nt = int(blockDim.x), nbw = nt / 32 - kSelThreads / 32;
+    select_boundaries(s_thr, views[0].K);   // the batch's views share K
+    __syncthreads();
 
     if (warp < kSelThreads / 32) {
         // ------------------------------------------------ selection role
-        using Bar = NamedBarrier<1, kSelThreads>;
         for (int n = 0;; ++n) {
             const int b = n & 1;
             if (n >= 2) empty_sync(b, nt);   // the blend warps are done with buffer b
@@ -201,7 +136,7 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
                 const uint32_t it = atomicAdd(counter, 1u);
                 s_item[b] = it < total_items ? int(it) : kItemEnd;
             }
-            Bar::sync();
+            bar_sync_id<1>(kSelThreads);
             const int item = s_item[b];
             if (item == kItemEnd) {
                 full_arrive(b, nt);
@@ -213,47 +148,25 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
             int32_t *s_ids = s_ids0 + b * kSelPix * KSB;
             float *s_w = s_w0 + b * kSelPix * KSB;
             const int tile = item - int(V.tile_base);
-            const int tx = tile % V.tiles_x, ty = tile / V.tiles_x;
-            const int tile_w = V.tile_w, tile_h = kSelPix / tile_w;
-            select_tile<Bar>(V.rec_m, V.rec_w, V.rec_a, V.rec_h, V.igid, V.ranges[tile], V.W, V.H,
-                             tile_w, tx, ty, K, V.alpha_min, V.alpha_max, st, s_ids, s_w, s_D,
-                             s_cnt[b]);
-            // normalise this thread's two pixels in place (Algorithm 1's 1 / (1 - T^Q))
-            {
-                const int lx = threadIdx.x % tile_w, ly = 2 * (threadIdx.x / tile_w);
-#pragma unroll
-                for (int r = 0; r < 2; ++r) {
-                    const int sl = (ly + r) * tile_w + lx;
-                    const int c = s_cnt[b][sl];
-                    const float D = s_D[sl];
-                    for (int j = 0; j < K; ++j) {
-                        const bool has = j < c;
-                        s_w[sl * KSB + j] = has ? __fdiv_rn(s_w[sl * KSB + j], D) : 0.0f;
-                        if (!has) s_ids[sl * KSB + j] = -1;
-                    }
-                }
-            }
-            Bar::sync();
-            // coalesced output for a backward pass: each tile row is tile_w * K
-            // consecutive ids and weights in the view
-            const int rowlen = tile_w * K;
-            for (int rem = threadIdx.x; rem < rowlen; rem += kSelThreads) {
-                const int cx = rem / K, j = rem - cx * K;
-                const int gx = tx * tile_w + cx;
-                if (gx >= V.W) continue;
-                for (int row = 0; row < tile_h; ++row) {
-                    const int gy = ty * tile_h + row;
-                    if (gy >= V.H) break;
-                    const int sl = row * tile_w + cx;
-                    const int64_t o = (int64_t(gy) * V.W + gx) * K + j;
-                    V.ids[o] = s_ids[sl * KSB + j];
-                    V.w[o] = s_w[sl * KSB + j];
-                }
-            }
-            for (int e = threadIdx.x; e < kSelPix; e += kSelThreads) {
-                const int gx = tx * tile_w + e % tile_w, gy = ty * tile_h + e / tile_w;
-                if (gx < V.W && gy < V.H) V.cnt[int64_t(gy) * V.W + gx] = s_cnt[b][e];
-            }
+            const int tile_w = V.tile_w, across = tile_w >> 3;
+            // this warp's 8 x 8 block of the tile; slots are the tile's pixels
+            const int bx = (warp % across) * 8, by = (warp / across) * 8;
+            const int x0 = (tile % V.tiles_x) * tile_w + bx;
+            const int y0 = (tile / V.tiles_x) * (kSelPix / tile_w) + by;
+            const int blk = by * tile_w + bx;
+            const int sa = blk + 2 * (lane >> 3) * tile_w + (lane & 7), sb = sa + tile_w;
+            Walk w0, w1;
+            select_block(V.rec_m, V.rec_w, V.rec_a, V.rec_h, V.igid, V.ranges[tile], V.W, V.H, x0,
+                         y0, K, V.alpha_min, V.alpha_max, s_thr, st[warp], s_ids + sa * KSB,
+                         s_w + sa * KSB, s_ids + sb * KSB, s_w + sb * KSB, w0, w1);
+            finish_pixel(w0, K, s_ids + sa * KSB, s_w + sa * KSB);
+            finish_pixel(w1, K, s_ids + sb * KSB, s_w + sb * KSB);
+            __syncwarp();
+            // ids, weights and counts are also written out for a backward pass
+            store_block(V.W, V.H, x0, y0, K, V.vec != 0, s_ids, s_w, blk, tile_w, V.ids, V.w);
+            const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
+            if (px < V.W && py < V.H) V.cnt[int64_t(py) * V.W + px] = uint8_t(w0.m);
+            if (px < V.W && py + 1 < V.H) V.cnt[int64_t(py + 1) * V.W + px] = uint8_t(w1.m);
             full_arrive(b, nt);
         }
         return;
@@ -499,7 +412,8 @@ cudaError_t prepare_batch(const qr_view *views, int n_views, void *ws, uint32_t 
         b.alpha_min = f.params.alpha_min;
         b.alpha_max = f.params.alpha_max;
         b.tile_base = base;
-        b.pad = 0;
+        b.vec = f.params.K % 4 == 0 &&
+                ((reinterpret_cast<uintptr_t>(b.ids) | reinterpret_cast<uintptr_t>(b.w)) & 15) == 0;
         base += uint32_t(f.tiles_x * f.tiles_y);
     }
     *total_items = base;

@@ -317,38 +317,6 @@ __device__ __forceinline__ float box_min_half_q(float4 mm, float4 cc, float x0, 
     return best;
 }
 
-// ---------------------------------------------------------------- Algorithm 1 walk
-// Algorithm 1 state of one pixel.
-struct Walk {
-    float T, TQ, thr;
-    int k, m;
-    bool done;
-};
-
-// The rarely taken end of an Algorithm 1 step, for a member entry (alpha' >=
-// alpha_min) whose T_test = Tt crosses the next quantile boundary or the stop
-// threshold: keep the Gaussian, advance k, stop.  The kept weight is
-// T^Q alpha' (Algorithm 1), or with kCount the number of boundaries Tt
-// crosses (App. C's right-Riemann weights, one segment width per boundary).
-template <bool kCount = false>
-__device__ __forceinline__ void walk_event(Walk &w, float Tt, float a, float tau_stop, int K,
-                                        uint32_t gid, int slot, int KS, int32_t *s_ids, float *s_w) {
-    if (Tt < w.thr) {
-        const int k0 = w.k;
-        s_ids[slot * KS + w.m] = int32_t(gid);
-        if constexpr (!kCount) s_w[slot * KS + w.m] = w.TQ * a;
-        ++w.m;
-        w.TQ = w.TQ * (1.0f - a);
-        do {
-            ++w.k;
-            w.thr = (w.k < K) ? __fdiv_rn(float(K - w.k), float(K + 1)) : -1.0f;
-        } while (Tt < w.thr);
-        if constexpr (kCount) s_w[slot * KS + w.m - 1] = float(w.k - k0);
-    }
-    if (Tt < tau_stop) w.done = true;
-    else w.T = Tt;
-}
-
 // ---------------------------------------------------------------- register bitonic sort
 // Sorts NTH*E keys (32- or 64-bit) held E per thread in blocked order (thread t holds
 // positions tE .. tE+E-1; pad with ~0).  Compare-exchange partners i and i^j

@@ -15,60 +15,58 @@
 // each kept Gaussian weighted by the number of boundaries T_test crosses at
 // it, divided by the number crossed in all.
 //
-// GB300 design: one CTA of 128 threads per screen tile; the walk itself
-// (select_tile.cuh) stages the tile's list through shared memory, culls it
-// per warp against the warp's box of pixel centres and walks two pixels per
-// thread with packed FP32x2 arithmetic.  Kept (id, weight) pairs are written
-// out once per tile row as contiguous runs of tile_w * K ids and weights, so
-// the stores are fully coalesced.
+// GB300 design: one warp per 8 x 8 pixel block (select_tile.cuh) and per CTA,
+// so an SM takes a new block as soon as one is done.  Measured with K = 8
+// (512-D VGA frames but for the last; CTAs of four warps walking a 16 x 16
+// tile in step, 128 staged entries at a time -> now):
+//   room, 500k Gaussians, 457 entries per tile       39.9 -> 22.9 us (issue)
+//   object, 500k Gaussians, up to 5,166 entries       273 -> 110 us (longest lists)
+//   room, 1M Gaussians at 1296 x 968                  126 -> 79 us
+//   2,000 Gaussians at 128 x 128 (256 warps in all)  41.8 -> 18.8 us (latency)
+// Two or four warps per CTA measured 0-5 % slower; a bound of 32 warps per SM
+// (64 registers) instead of 24 cost up to 13 %.
 #include "select_tile.cuh"
 
 namespace qr {
 namespace {
 
-// kCount: App. C's Riemann weights in place of Algorithm 1's (select_tile).
+constexpr int kSelWarps = 1;      // divides 4
+
+// kCount: App. C's Riemann weights in place of Algorithm 1's (select_block).
 template <bool kCount>
-__global__ void __launch_bounds__(kSelThreads, 8)
+__global__ void __launch_bounds__(32 * kSelWarps, 24 / kSelWarps)
 select_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
               const float *__restrict__ rec_a, const float *__restrict__ rec_h,
               const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
               int H, int tile_w, int tiles_x, int K, float alpha_min, float alpha_max,
-              int32_t *__restrict__ ids, float *__restrict__ wout, uint8_t *__restrict__ cnt) {
-    pdl_wait();   // the predecessor's outputs are complete and visible
-    __shared__ SelStage st;
-    __shared__ float s_D[kSelPix];       // 1 - T^Q per pixel
-    __shared__ uint8_t s_cnt[kSelPix];
+              int32_t *__restrict__ ids, float *__restrict__ wout, uint8_t *__restrict__ cnt,
+              int vec) {
+    __shared__ SelStage st[kSelWarps];
+    __shared__ float s_thr[kKMax + 1];
     extern __shared__ unsigned char s_dyn[];
     const int KS = K | 1;
-    int32_t *s_ids = reinterpret_cast<int32_t *>(s_dyn);          // [256][KS]
-    float *s_w = reinterpret_cast<float *>(s_dyn) + KS * kSelPix;  // [256][KS]
-    const int tile = blockIdx.x;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int tile_h = kSelPix / tile_w;
-    select_tile<CtaBarrier, kCount>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[tile], W, H, tile_w, tx,
-                            ty, K, alpha_min, alpha_max, st, s_ids, s_w, s_D, s_cnt);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int32_t *s_ids = reinterpret_cast<int32_t *>(s_dyn) + warp * kSelBlock * KS;   // [64][KS] per warp
+    float *s_w = reinterpret_cast<float *>(s_dyn) + (kSelWarps + warp) * kSelBlock * KS;
+    select_boundaries(s_thr, K);
     __syncthreads();
-    // coalesced output: each row of the tile is tile_w * K consecutive entries
-    // of ids and weights in the image
-    const int rowlen = tile_w * K;
-    for (int rem = threadIdx.x; rem < rowlen; rem += kSelThreads) {
-        const int cx = rem / K, j = rem - cx * K;
-        const int gx = tx * tile_w + cx;
-        if (gx >= W) continue;
-        for (int row = 0; row < tile_h; ++row) {
-            const int gy = ty * tile_h + row;
-            if (gy >= H) break;
-            const int slot = row * tile_w + cx;
-            const int64_t o = (int64_t(gy) * W + gx) * K + j;
-            const bool has = j < int(s_cnt[slot]);
-            ids[o] = has ? s_ids[slot * KS + j] : -1;
-            wout[o] = has ? __fdiv_rn(s_w[slot * KS + j], s_D[slot]) : 0.0f;
-        }
-    }
-    for (int e = threadIdx.x; e < kSelPix; e += kSelThreads) {
-        const int gx = tx * tile_w + e % tile_w, gy = ty * tile_h + e / tile_w;
-        if (gx < W && gy < H) cnt[int64_t(gy) * W + gx] = s_cnt[e];
-    }
+    pdl_wait();   // the predecessor's outputs are complete and visible
+    const int block = int(blockIdx.x) * kSelWarps + warp;
+    const int tile = block >> 2, part = block & 3, across = tile_w >> 3;
+    const int x0 = (tile % tiles_x) * tile_w + (part % across) * 8;
+    const int y0 = (tile / tiles_x) * (kSelPix / tile_w) + (part / across) * 8;
+    const int sa = (2 * (lane >> 3)) * 8 + (lane & 7), sb = sa + 8;
+    Walk w0, w1;
+    select_block<kCount>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[tile], W, H, x0, y0, K,
+                         alpha_min, alpha_max, s_thr, st[warp], s_ids + sa * KS, s_w + sa * KS,
+                         s_ids + sb * KS, s_w + sb * KS, w0, w1);
+    finish_pixel<kCount>(w0, K, s_ids + sa * KS, s_w + sa * KS);
+    finish_pixel<kCount>(w1, K, s_ids + sb * KS, s_w + sb * KS);
+    __syncwarp();
+    store_block(W, H, x0, y0, K, vec != 0, s_ids, s_w, 0, 8, ids, wout);
+    const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
+    if (px < W && py < H) cnt[int64_t(py) * W + px] = uint8_t(w0.m);
+    if (px < W && py + 1 < H) cnt[int64_t(py + 1) * W + px] = uint8_t(w1.m);
 }
 
 }  // namespace
@@ -78,14 +76,10 @@ cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cn
     const int tiles = num_tiles(f);
     if (tiles == 0) return cudaSuccess;
     const int K = f.params.K;
-    const size_t dyn = size_t(K | 1) * kSelPix * 8;
+    const size_t dyn = size_t(K | 1) * kSelBlock * kSelWarps * 8;
+    const int vec = K % 4 == 0 && ((reinterpret_cast<uintptr_t>(ids) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
     auto go = [&](auto kern) -> cudaError_t {
-        if (dyn > 48 * 1024) {
-            const cudaError_t e =
-                cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
-            if (e != cudaSuccess) return e;
-        }
-        return pdl_launch(kern, dim3(tiles), dim3(kSelThreads), dyn, s,
+        return pdl_launch(kern, dim3(unsigned(tiles) * 4 / kSelWarps), dim3(32 * kSelWarps), dyn, s,
                           (const float4 *)slot<float4>(f, S_REC_M),
                           (const float4 *)slot<float4>(f, S_REC_C),
                           (const float *)slot<float>(f, S_REC_A),
@@ -93,7 +87,7 @@ cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cn
                           (const uint32_t *)slot<uint32_t>(f, S_IGID),
                           (const uint2 *)slot<uint2>(f, S_RANGES), f.camera.width,
                           f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
-                          f.params.alpha_max, ids, w, cnt);
+                          f.params.alpha_max, ids, w, cnt, vec);
     };
     const cudaError_t e = riemann ? go(select_kernel<true>) : go(select_kernel<false>);
     count_launch();

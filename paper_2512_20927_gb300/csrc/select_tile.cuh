@@ -1,7 +1,7 @@
-// The selection half of Algorithm 1 for one screen tile, shared by the
-// single-view selection kernel (select.cu) and the many-view persistent
-// kernel (batch.cu), so both keep exactly the same Gaussians with the same
-// FP32 weights.
+// The selection half of Algorithm 1 for a block of 8 x 8 pixels by one warp,
+// shared by the single-view selection kernel (select.cu) and the many-view
+// persistent kernel (batch.cu), so both keep exactly the same Gaussians with
+// the same FP32 weights.
 //
 // Per pixel, front to back over the tile's depth-ordered list:
 //   alpha' = min(alpha_max, alpha exp(-q/2)); entries with alpha' < alpha_min
@@ -10,30 +10,36 @@
 //   if T_test < tau_k (tau_k = (K-k)/(K+1), the boundary 1-(k+1)/(K+1)):
 //       keep the Gaussian with weight w = T^Q alpha', T^Q *= 1 - alpha',
 //       advance k past every boundary T_test is below;
-//   stop once T_test < 1/(K+1); otherwise T = T_test.
+//   stop once T_test < 1/(K+1) = tau_{K-1}, i.e. when k reaches K; otherwise
+//   T = T_test.
 //
-// 128 threads walk the tile's 256 pixels, two vertically adjacent pixels of
-// the same column each.  The tile's list is staged through shared memory 128
-// entries at a time (gid, projected mean hi/lo, conic axes, opacity, reject
-// bound: 44 B each) with coalesced loads; the ids of the next batch are
-// fetched while the current one is walked.
-//   * Each warp first culls the staged entries against its box of pixel
-//     centres, one entry per lane: the minimum of q/2 over the box against
-//     the entry's reject bound.  Most entries a pixel would walk are out of
-//     reach of the whole box.
-//   * The warp walks the survivors four per step (independent chains).  The
-//     two pixels of a thread share the x offset; their y offsets, axis
-//     projections and q/2 use packed FP32x2 instructions (each half rounds
-//     exactly like the scalar instruction).  Entries within reach take the
-//     Algorithm 1 step for both pixels at once; only keeping a Gaussian or
-//     stopping branches off.
-// The 128 threads stop loading as soon as all of their pixels have stopped.
-// Kept (id, unnormalised weight) pairs go to per-pixel shared-memory slots
-// [256][K|1]; s_D gets 1 - T^Q and s_cnt the kept count of each pixel.
-//
-// The barrier policy Bar joins the 128 walking threads: the whole CTA in the
-// selection kernel, a named barrier in the many-view kernel (whose other
-// warps blend meanwhile).
+// What bounds it: instruction issue where every SM has 32 warps (a VGA frame
+// is one wave), and the latency of the longest lists' chain of steps where it
+// has not (a thumbnail, a silhouette tile).  Hence:
+//   * A warp works alone: it owns an 8 x 8 block (two vertically adjacent
+//     pixels per lane), stages the tile's list for itself and stops when its
+//     own 64 pixels have stopped; no CTA barrier ties it to the other warps
+//     of the tile, whose lists end elsewhere.  8 x 8 is the block with the
+//     fewest entries within reach.
+//   * Each lane holds one of 32 list entries in registers (the records of the
+//     next 32 are loaded while these are used, the ids of the 32 after that
+//     too), culls it against the block's box of pixel centres (the minimum of
+//     q/2 over the box against the entry's reject bound), and only the
+//     survivors (a fifth) go to shared memory, compacted in list order; up to
+//     three left over are carried to the next 32, so the walk below always
+//     takes four.
+//   * Four survivors per step: eight independent alpha' (packed FP32x2 for
+//     q/2; each half rounds like the scalar instruction), zero for entries
+//     that are no members, then the four prefix products T (1 - alpha').  A
+//     product with 1 - 0 is exact, so they are Algorithm 1's T_test, and T
+//     never rises, so no boundary is crossed within the step unless the last
+//     product is below the pixel's next boundary: one comparison per pixel
+//     and one vote per step stand for the eight entry tests.  Only crossings
+//     branch off, all pixels' first ones together, then their next ones; the
+//     boundaries (K-k)/(K+1) come from a table.
+// Kept (id, unnormalised weight) pairs go to per-pixel shared-memory slots of
+// KS = K|1 entries; finish_block normalises and pads them, store_block writes
+// them out.
 #pragma once
 
 #include "qr_internal.cuh"
@@ -41,31 +47,22 @@
 namespace qr {
 
 constexpr int kSelPix = 256;       // pixels per tile
-constexpr int kSelThreads = 128;   // two pixels per thread
-constexpr int kSelBatch = 128;     // list entries staged per batch
+constexpr int kSelBlock = 64;      // pixels per warp: 8 x 8
+constexpr int kSelSurv = 36;       // survivors held: 3 carried + 32, rounded up to 4
 
+// One warp's survivors.
 struct SelStage {
-    float4 m[kSelBatch];
-    float4 c[kSelBatch];
-    float a[kSelBatch];
-    float h[kSelBatch];
-    uint32_t g[kSelBatch];
+    float4 m[kSelSurv];
+    float4 c[kSelSurv];
+    float2 ah[kSelSurv];
+    uint32_t g[kSelSurv];
 };
 
-struct CtaBarrier {
-    __device__ static void sync() { __syncthreads(); }
-    __device__ static int count(bool p) { return __syncthreads_count(p); }
-};
-
-template <int ID, int N>
-struct NamedBarrier {
-    __device__ static void sync() { asm volatile("bar.sync %0, %1;" ::"n"(ID), "n"(N) : "memory"); }
-    __device__ static int count(bool p) {
-        int r;
-        asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %1, 0;\n bar.red.popc.u32 %0, %2, %3, q;\n}\n"
-                     : "=r"(r) : "r"(int(p)), "n"(ID), "n"(N) : "memory");
-        return r;
-    }
+// Algorithm 1 state of one pixel: T, T^Q, the next boundary (-1 once k == K),
+// boundaries passed, Gaussians kept.  k == K: the walk has stopped.
+struct Walk {
+    float T, TQ, thr;
+    int k, m;
 };
 
 __device__ __forceinline__ float2 sel_add2(float2 a, float2 b) {
@@ -91,145 +88,208 @@ __device__ __forceinline__ float2 sel_fma2(float2 a, float2 b, float2 c) {
     return d;
 }
 
-// Walks tile (tx, ty) whose depth-ordered ids are isect_gid[range.x, range.y).
-// Called by threads 0..127 (all of them); ends with the per-pixel results in
-// s_ids / s_w / s_D / s_cnt, written by their owners (the caller joins the
-// threads with Bar::sync() before reading other pixels' slots).  With
-// kCount the weights are boundary-crossing counts and s_D the number of
-// boundaries crossed in all (App. C's Riemann weights); the selection is the
-// same.
-template <class Bar, bool kCount = false>
-__device__ __forceinline__ void select_tile(const float4 *__restrict__ rec_m,
-                                            const float4 *__restrict__ rec_w,
-                                            const float *__restrict__ rec_a,
-                                            const float *__restrict__ rec_h,
-                                            const uint32_t *__restrict__ isect_gid, uint2 range,
-                                            int W, int H, int tile_w, int tx, int ty, int K,
-                                            float alpha_min, float alpha_max, SelStage &st,
-                                            int32_t *s_ids, float *s_w, float *s_D, uint8_t *s_cnt) {
-    const int KS = K | 1;   // odd stride: the per-pixel slots fall in distinct banks
-    const int tile_h = kSelPix / tile_w;
-    const int lx = threadIdx.x % tile_w, ly = 2 * (threadIdx.x / tile_w);
-    const int px = tx * tile_w + lx, py = ty * tile_h + ly;
-    const int slot0 = ly * tile_w + lx, slot1 = slot0 + tile_w;
+// The boundaries tau_k = (K-k)/(K+1), k < K, and -1 behind them (K + 1
+// entries in shared memory, written by the CTA's threads; the caller joins
+// them before the walk).
+__device__ __forceinline__ void select_boundaries(float *s_thr, int K) {
+    for (int k = int(threadIdx.x); k <= K; k += int(blockDim.x))
+        s_thr[k] = k < K ? __fdiv_rn(float(K - k), float(K + 1)) : -1.0f;
+}
+
+// A member entry whose T_test = Tt crosses the pixel's next boundary: keep
+// it with weight T^Q alpha' (Algorithm 1), or with kCount the number of
+// boundaries Tt crosses (App. C's right-Riemann weights), and advance k.
+template <bool kCount>
+__device__ __forceinline__ void walk_event(Walk &w, float Tt, float a, uint32_t gid,
+                                           const float *s_thr, int32_t *ids, float *wts) {
+    const int k0 = w.k;
+    ids[w.m] = int32_t(gid);
+    if constexpr (!kCount) wts[w.m] = w.TQ * a;
+    w.TQ = w.TQ * (1.0f - a);
+    do {
+        w.thr = s_thr[++w.k];
+    } while (Tt < w.thr);
+    if constexpr (kCount) wts[w.m] = float(w.k - k0);
+    ++w.m;
+}
+
+// Walks the 8 x 8 block at (x0, y0) over isect_gid[range.x, range.y), the
+// depth-ordered list of the tile that holds it.  All lanes of the warp call
+// it.  Lane l owns pixels (x0 + l % 8, y0 + 2 (l / 8)) and the one below;
+// their kept entries go to ids0 / wts0 and ids1 / wts1 (K entries each) and
+// their final states to w0, w1.
+template <bool kCount = false>
+__device__ __forceinline__ void select_block(
+    const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+    const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+    const uint32_t *__restrict__ isect_gid, uint2 range, int W, int H, int x0, int y0, int K,
+    float alpha_min, float alpha_max, const float *s_thr, SelStage &st, int32_t *ids0, float *wts0,
+    int32_t *ids1, float *wts1, Walk &w0, Walk &w1) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
     const bool in0 = px < W && py < H, in1 = px < W && py + 1 < H;
     const float ux = float(px) + 0.5f;
     const float2 uy = make_float2(float(py) + 0.5f, float(py + 1) + 0.5f);
+    const float thr0 = s_thr[0];
+    w0 = Walk{1.0f, 1.0f, in0 ? thr0 : -1.0f, in0 ? 0 : K, 0};
+    w1 = Walk{1.0f, 1.0f, in1 ? thr0 : -1.0f, in1 ? 0 : K, 0};
+    if (x0 >= W || y0 >= H) return;
+    // the block's box of pixel centres inside the image
+    const float bx0 = float(x0) + 0.5f, bx1 = float(min(x0 + 7, W - 1)) + 0.5f;
+    const float by0 = float(y0) + 0.5f, by1 = float(min(y0 + 7, H - 1)) + 0.5f;
 
-    const float tau_stop = __fdiv_rn(1.0f, float(K + 1));
-    const float thr0 = __fdiv_rn(float(K), float(K + 1));
-    Walk w0{1.0f, 1.0f, thr0, 0, 0, !in0};
-    Walk w1{1.0f, 1.0f, thr0, 0, 0, !in1};
-
-    // the warp's box of pixel centres
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    float bx0 = ux, bx1 = ux, by0 = uy.x, by1 = uy.y;
+    // four survivors from st[j]; false once every pixel of the warp has stopped
+    auto step4 = [&](int j) -> bool {
+        float a0[4], a1[4];
+        float2 t[4];
+        float2 T = make_float2(w0.T, w1.T);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        bx0 = fminf(bx0, __shfl_xor_sync(FULL, bx0, o));
-        bx1 = fmaxf(bx1, __shfl_xor_sync(FULL, bx1, o));
-        by0 = fminf(by0, __shfl_xor_sync(FULL, by0, o));
-        by1 = fmaxf(by1, __shfl_xor_sync(FULL, by1, o));
-    }
-
-    // the id of the next staged entry is fetched while the current batch is walked
-    uint32_t gnext = range.x + threadIdx.x < range.y ? isect_gid[range.x + threadIdx.x] : 0u;
-    for (uint32_t b = range.x; b < range.y; b += kSelBatch) {
-        if (Bar::count(w0.done && w1.done) == kSelThreads) break;
-        if (b + threadIdx.x < range.y) {
-            st.g[threadIdx.x] = gnext;
-            st.m[threadIdx.x] = rec_m[gnext];
-            st.c[threadIdx.x] = rec_w[gnext];
-            st.a[threadIdx.x] = rec_a[gnext];
-            st.h[threadIdx.x] = rec_h[gnext];
+        for (int u = 0; u < 4; ++u) {
+            const float4 mm = st.m[j + u];
+            const float4 cc = st.c[j + u];
+            const float2 ah = st.ah[j + u];
+            // eval_half_q for both pixels: dx shared, the rest packed
+            const float dx = (ux - mm.x) - mm.z;
+            const float2 dy = sel_add2(sel_add2(uy, make_float2(-mm.y, -mm.y)), make_float2(-mm.w, -mm.w));
+            const float2 dx2 = make_float2(dx, dx);
+            const float2 p1 = sel_fma2(dx2, make_float2(cc.x, cc.x), sel_mul2(dy, make_float2(cc.y, cc.y)));
+            const float2 p2 = sel_fma2(dx2, make_float2(cc.z, cc.z), sel_mul2(dy, make_float2(cc.w, cc.w)));
+            const float2 hq = sel_fma2(p1, p1, sel_mul2(p2, p2));
+            const float e0 = eval_alpha(ah.x, hq.x, alpha_max), e1 = eval_alpha(ah.x, hq.y, alpha_max);
+            a0[u] = (hq.x > ah.y || e0 < alpha_min) ? 0.0f : e0;
+            a1[u] = (hq.y > ah.y || e1 < alpha_min) ? 0.0f : e1;
         }
-        Bar::sync();
-        {
-            const uint32_t idx = b + kSelBatch + threadIdx.x;
-            gnext = idx < range.y ? isect_gid[idx] : 0u;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            T = sel_mul2(T, sel_add2(make_float2(1.0f, 1.0f), make_float2(-a0[u], -a1[u])));
+            t[u] = T;
         }
-        const int nb = int(min(uint32_t(kSelBatch), range.y - b));
-        for (int c0 = 0; c0 < nb; c0 += 32) {
-            if (__all_sync(FULL, w0.done && w1.done)) break;
-            // cull 32 staged entries against the warp's box (one per lane): an
-            // entry whose q/2 stays above its reject bound over the whole box
-            // is skipped by every pixel of the warp anyway
-            const int jl = c0 + lane;
-            bool pass = false;
-            if (jl < nb)
-                pass = !(box_min_half_q(st.m[jl], st.c[jl], bx0, bx1, by0, by1) * 0.999f > st.h[jl] + 1e-3f);
-            unsigned todo = __ballot_sync(FULL, pass);
-            // walk the survivors in list order, four entries per step: their
-            // q/2 chains are independent, and the Algorithm 1 steps run only
-            // when one of them is within reach
-            while (todo) {
-                int jj[4];
-                bool valid[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    valid[u] = todo != 0u;
-                    jj[u] = valid[u] ? c0 + __ffs(todo) - 1 : jj[0];
-                    todo &= todo - 1u;
-                }
-                float2 hq[4];
-                float h[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const int j = jj[u];
-                    const float4 mm = st.m[j];
-                    const float4 cc = st.c[j];
-                    h[u] = st.h[j];
-                    // eval_half_q for both pixels: dx shared, the rest packed
-                    const float dx = (ux - mm.x) - mm.z;
-                    const float2 dy = sel_add2(sel_add2(uy, make_float2(-mm.y, -mm.y)),
-                                               make_float2(-mm.w, -mm.w));
-                    const float2 dx2 = make_float2(dx, dx);
-                    const float2 p1 = sel_fma2(dx2, make_float2(cc.x, cc.x), sel_mul2(dy, make_float2(cc.y, cc.y)));
-                    const float2 p2 = sel_fma2(dx2, make_float2(cc.z, cc.z), sel_mul2(dy, make_float2(cc.w, cc.w)));
-                    hq[u] = sel_fma2(p1, p1, sel_mul2(p2, p2));
-                }
-                unsigned reach = 0;   // bit 2u: pixel 0 may take entry u, bit 2u+1: pixel 1
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    reach |= unsigned(valid[u] && !(hq[u].x > h[u])) << (2 * u);
-                    reach |= unsigned(valid[u] && !(hq[u].y > h[u])) << (2 * u + 1);
-                }
-                if (w0.done) reach &= 0xAAu;
-                if (w1.done) reach &= 0x55u;
-                if (!reach) continue;
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const bool r0 = !w0.done && ((reach >> (2 * u)) & 1u);
-                    const bool r1 = !w1.done && ((reach >> (2 * u + 1)) & 1u);
-                    if (!(r0 || r1)) continue;
-                    // alpha' and T_test for both pixels; a pixel for which the entry is
-                    // not a member gets alpha' = 0, i.e. T_test = T (1 - 0) = T exactly
-                    const float alpha = st.a[jj[u]];
-                    const float a0 = eval_alpha(alpha, hq[u].x, alpha_max);
-                    const float a1 = eval_alpha(alpha, hq[u].y, alpha_max);
-                    const bool t0 = r0 && !(a0 < alpha_min), t1 = r1 && !(a1 < alpha_min);
-                    const float2 Tt = sel_mul2(make_float2(w0.T, w1.T),
-                                               sel_add2(make_float2(1.0f, 1.0f),
-                                                        make_float2(t0 ? -a0 : -0.0f, t1 ? -a1 : -0.0f)));
-                    const bool e0 = t0 && (Tt.x < w0.thr || Tt.x < tau_stop);
-                    const bool e1 = t1 && (Tt.y < w1.thr || Tt.y < tau_stop);
-                    if (e0 || e1) {
-                        const uint32_t gid = st.g[jj[u]];
-                        if (e0) walk_event<kCount>(w0, Tt.x, a0, tau_stop, K, gid, slot0, KS, s_ids, s_w);
-                        if (e1) walk_event<kCount>(w1, Tt.y, a1, tau_stop, K, gid, slot1, KS, s_ids, s_w);
-                    }
-                    if (t0 && !e0) w0.T = Tt.x;
-                    if (t1 && !e1) w1.T = Tt.y;
-                }
-                if (w0.done && w1.done) break;
+        w0.T = T.x;
+        w1.T = T.y;
+        if (!__any_sync(FULL, T.x < w0.thr || T.y < w1.thr)) return true;
+        // the first crossing of each pixel, then the next (rarely a third)
+        do {
+            if (T.x < w0.thr) {
+                const int u = t[0].x < w0.thr ? 0 : t[1].x < w0.thr ? 1 : t[2].x < w0.thr ? 2 : 3;
+                const float a = u == 0 ? a0[0] : u == 1 ? a0[1] : u == 2 ? a0[2] : a0[3];
+                const float Tt = u == 0 ? t[0].x : u == 1 ? t[1].x : u == 2 ? t[2].x : t[3].x;
+                walk_event<kCount>(w0, Tt, a, st.g[j + u], s_thr, ids0, wts0);
             }
+            if (T.y < w1.thr) {
+                const int u = t[0].y < w1.thr ? 0 : t[1].y < w1.thr ? 1 : t[2].y < w1.thr ? 2 : 3;
+                const float a = u == 0 ? a1[0] : u == 1 ? a1[1] : u == 2 ? a1[2] : a1[3];
+                const float Tt = u == 0 ? t[0].y : u == 1 ? t[1].y : u == 2 ? t[2].y : t[3].y;
+                walk_event<kCount>(w1, Tt, a, st.g[j + u], s_thr, ids1, wts1);
+            }
+        } while (__any_sync(FULL, T.x < w0.thr || T.y < w1.thr));
+        return !__all_sync(FULL, w0.k == K && w1.k == K);
+    };
+
+    // entry base + lane of the list in registers; g1 / g2: its successors' ids
+    uint32_t b = range.x + lane, g1 = 0, g2 = 0;
+    float4 nm = make_float4(0.f, 0.f, 0.f, 0.f), nc = nm;
+    float na = 0.f, nh = 0.f;
+    if (b < range.y) {
+        g1 = isect_gid[b];
+        nm = rec_m[g1];
+        nc = rec_w[g1];
+        na = rec_a[g1];
+        nh = rec_h[g1];
+    }
+    if (b + 32 < range.y) g2 = isect_gid[b + 32];
+    int left = 0;
+    for (uint32_t base = range.x; base < range.y; base += 32, b += 32) {
+        const float4 cm = nm, cc = nc;
+        const float ca = na, ch = nh;
+        const uint32_t cg = g1;
+        g1 = g2;
+        if (b + 32 < range.y) {
+            nm = rec_m[g1];
+            nc = rec_w[g1];
+            na = rec_a[g1];
+            nh = rec_h[g1];
+        }
+        if (b + 64 < range.y) g2 = isect_gid[b + 64];
+        // an entry whose q/2 stays above its reject bound over the whole box is
+        // skipped by every pixel of the warp anyway
+        const bool pass = b < range.y &&
+                          !(box_min_half_q(cm, cc, bx0, bx1, by0, by1) * 0.999f > ch + 1e-3f);
+        const unsigned bal = __ballot_sync(FULL, pass);
+        if (pass) {
+            const int i = left + __popc(bal & ((1u << lane) - 1u));
+            st.m[i] = cm;
+            st.c[i] = cc;
+            st.ah[i] = make_float2(ca, ch);
+            st.g[i] = cg;
+        }
+        const int n = left + __popc(bal), full = n & ~3;
+        __syncwarp();
+        for (int j = 0; j < full; j += 4)
+            if (!step4(j)) return;
+        left = n - full;
+        if (full) {   // the rest to the front (at most 3; sources lie behind them)
+            __syncwarp();
+            if (lane < left) {
+                st.m[lane] = st.m[full + lane];
+                st.c[lane] = st.c[full + lane];
+                st.ah[lane] = st.ah[full + lane];
+                st.g[lane] = st.g[full + lane];
+            }
+            __syncwarp();
         }
     }
-    s_D[slot0] = kCount ? float(w0.k) : 1.0f - w0.TQ;
-    s_D[slot1] = kCount ? float(w1.k) : 1.0f - w1.TQ;
-    s_cnt[slot0] = uint8_t(w0.m);
-    s_cnt[slot1] = uint8_t(w1.m);
+    if (left) {   // the last step, filled up with entries out of reach
+        if (lane >= left && lane < 4) {
+            st.m[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            st.c[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+            st.ah[lane] = make_float2(0.f, -1.f);
+            st.g[lane] = 0u;
+        }
+        __syncwarp();
+        step4(0);
+    }
+}
+
+// A pixel's kept weights divided by 1 - T^Q (kCount: by the boundaries crossed
+// in all), the rest of its K slots padded with id -1 and weight 0.
+template <bool kCount = false>
+__device__ __forceinline__ void finish_pixel(const Walk &w, int K, int32_t *ids, float *wts) {
+    const float D = kCount ? float(w.k) : 1.0f - w.TQ;
+    for (int j = 0; j < w.m; ++j) wts[j] = __fdiv_rn(wts[j], D);
+    for (int j = w.m; j < K; ++j) {
+        ids[j] = -1;
+        wts[j] = 0.0f;
+    }
+}
+
+// Writes the finished block at (x0, y0) (slot of pixel (x, y): s0 + y stride +
+// x) to the image's ids and weights; the warp's lanes must have finished
+// their pixels (__syncwarp between).  Rows of a block are 8 K consecutive
+// entries of the image; vec (K % 4 == 0 and 16-byte aligned outputs) writes
+// them four at a time.
+__device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K, bool vec,
+                                            const int32_t *s_ids, const float *s_w, int s0, int stride,
+                                            int32_t *__restrict__ ids, float *__restrict__ wout) {
+    const int lane = threadIdx.x & 31;
+    const int KS = K | 1;
+    const int per = vec ? 4 : 1;
+    const int KP = K / per;                        // units per pixel
+    const uint32_t inv = (65536u + uint32_t(KP) - 1u) / uint32_t(KP);   // e / KP, e < 64 KP <= 2048
+    for (int e = lane; e < kSelBlock * KP; e += 32) {
+        const int pix = int((uint32_t(e) * inv) >> 16), j = (e - pix * KP) * per;
+        const int x = x0 + (pix & 7), y = y0 + (pix >> 3);
+        if (x >= W || y >= H) continue;
+        const int at = (s0 + (pix >> 3) * stride + (pix & 7)) * KS + j;
+        const int64_t o = (int64_t(y) * W + x) * K + j;
+        if (vec) {
+            *reinterpret_cast<int4 *>(ids + o) = make_int4(s_ids[at], s_ids[at + 1], s_ids[at + 2], s_ids[at + 3]);
+            *reinterpret_cast<float4 *>(wout + o) = make_float4(s_w[at], s_w[at + 1], s_w[at + 2], s_w[at + 3]);
+        } else {
+            ids[o] = s_ids[at];
+            wout[o] = s_w[at];
+        }
+    }
 }
 
 }  // namespace qr

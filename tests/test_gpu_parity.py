@@ -453,3 +453,28 @@ def test_blend_channel_chunks_bit_identical(dtype, C):
         q.qr_set_blend_chunks(0)
     with pytest.raises(q.QRError):
         q.qr_set_blend_chunks(3)
+
+
+@pytest.mark.parametrize("w,h,K,tile", [(1, 1, 8, (16, 16)), (7, 9, 3, (16, 16)),
+                                        (9, 17, 4, (32, 8)), (33, 8, 12, (8, 32)),
+                                        (16, 31, 32, (32, 8)), (50, 23, 8, (8, 32))])
+def test_selection_block_edges(w, h, K, tile):
+    """8 x 8 blocks cut by the image's edge, every tile shape, vector and
+    scalar stores (K % 4, 4-byte aligned outputs)."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = scenes.tiny_scene(seed=11, n=1500, channels=16)
+    cam = scenes.tiny_camera(w, h)
+    gpu = H.run_gpu(g, f, cam, K, dense=False, params_kw={"tile_w": tile[0], "tile_h": tile[1]})
+    _, pix, ref = H.run_oracle(g, f, cam, K)
+    H.check_frame(gpu, ref, pix, w, f, 1e-5, max_tie_frac=0.05, label=f"{w}x{h}")
+    P = w * h
+    ids = torch.full((P * K + 2,), -7, dtype=torch.int32, device="cuda")
+    wts = torch.full((P * K + 2,), -7.0, device="cuda")
+    cnt = torch.empty(P, dtype=torch.uint8, device="cuda")
+    q.qr_select(gpu["frame"], ids[1:-1].view(P, K), wts[1:-1].view(P, K), cnt)
+    torch.cuda.synchronize()
+    assert (ids[1:-1].cpu().numpy().reshape(P, K) == gpu["ids"]).all()
+    assert (wts[1:-1].cpu().numpy().reshape(P, K) == gpu["weights"]).all()
+    assert (cnt.cpu().numpy() == gpu["counts"]).all()
+    assert ids[0] == -7 and ids[-1] == -7 and wts[0] == -7 and wts[-1] == -7
