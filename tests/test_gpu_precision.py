@@ -64,6 +64,36 @@ def test_fp8_encoder_bit_exact():
     np.testing.assert_array_equal(codes.cpu().numpy(), rc)
 
 
+@pytest.mark.parametrize("rows,C", [(1, 4), (9, 12), (257, 16), (5, 129), (33, 132), (100, 256),
+                                    (64, 260), (70, 512), (17, 516), (9, 1024), (5, 1028)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fp8_encoder_at_code_boundaries(rows, C, shift):
+    """Values at and one ulp around the midpoints between codes, signed zeros,
+    subnormal and huge scales; aligned and unaligned tables."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    rng = np.random.default_rng(rows * 7 + C)
+    scale = (10.0 ** rng.uniform(-3, 3, (rows, 1))).astype(np.float32)
+    scale[::7] = (2.0 ** rng.uniform(-130, 118, scale[::7].shape)).astype(np.float32)
+    mid = (16 + rng.integers(0, 16, (rows, C)) + 0.5) * 2.0 ** rng.integers(-14, 4, (rows, C))
+    f = (np.minimum(mid, 447) * scale.astype(np.float64)).astype(np.float32)
+    step = rng.integers(-1, 2, (rows, C))
+    f = np.where(step < 0, np.nextafter(f, np.float32(0)), np.where(step > 0, np.nextafter(f, np.float32(np.inf)), f))
+    f = f * rng.choice(np.array([-1, 1], np.float32), (rows, C))
+    f[:, C // 2] = -0.0
+    f[:, 0] = 448 * scale[:, 0]
+    f[rows // 2, :] = 0.0
+    buf = torch.zeros(rows * C + shift, device="cuda")
+    x = buf[shift:].view(rows, C)
+    x.copy_(torch.from_numpy(f))
+    codes, s = q.qr_quantize_fp8(x)
+    rc, rs = oracle.fp8_quantize_rows(f)
+    np.testing.assert_array_equal(s.cpu().numpy(), rs)
+    np.testing.assert_array_equal(codes.cpu().numpy(), rc)
+    got = q.qr_quantize_bf16(x).view(torch.int16).cpu().numpy().view(np.uint16)
+    np.testing.assert_array_equal(got, oracle.bf16_encode(f))
+
+
 @pytest.mark.parametrize("dtype", ["bf16", "fp8"])
 def test_low_precision_tables_match_oracle_on_decoded_features(dtype):
     import torch
