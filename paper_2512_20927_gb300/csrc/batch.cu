@@ -163,7 +163,8 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
             finish_pixel(w1, K, s_ids + sb * KSB, s_w + sb * KSB);
             __syncwarp();
             // ids, weights and counts are also written out for a backward pass
-            store_block(V.W, V.H, x0, y0, K, V.vec != 0, s_ids, s_w, blk, tile_w, V.ids, V.w);
+            store_block(V.W, V.H, x0, y0, K, V.vec != 0, s_ids, s_w,
+                        [&](int x, int y) { return blk + y * tile_w + x; }, V.ids, V.w);
             const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
             if (px < V.W && py < V.H) V.cnt[int64_t(py) * V.W + px] = uint8_t(w0.m);
             if (px < V.W && py + 1 < V.H) V.cnt[int64_t(py + 1) * V.W + px] = uint8_t(w1.m);

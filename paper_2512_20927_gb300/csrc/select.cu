@@ -63,7 +63,7 @@ select_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w
     finish_pixel<kCount>(w0, K, s_ids + sa * KS, s_w + sa * KS);
     finish_pixel<kCount>(w1, K, s_ids + sb * KS, s_w + sb * KS);
     __syncwarp();
-    store_block(W, H, x0, y0, K, vec != 0, s_ids, s_w, 0, 8, ids, wout);
+    store_block(W, H, x0, y0, K, vec != 0, s_ids, s_w, [](int x, int y) { return y * 8 + x; }, ids, wout);
     const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
     if (px < W && py < H) cnt[int64_t(py) * W + px] = uint8_t(w0.m);
     if (px < W && py + 1 < H) cnt[int64_t(py + 1) * W + px] = uint8_t(w1.m);

@@ -115,35 +115,31 @@ __device__ __forceinline__ void walk_event(Walk &w, float Tt, float a, uint32_t 
 
 // Walks the 8 x 8 block at (x0, y0) over isect_gid[range.x, range.y), the
 // depth-ordered list of the tile that holds it.  All lanes of the warp call
-// it.  Lane l owns pixels (x0 + l % 8, y0 + 2 (l / 8)) and the one below;
-// their kept entries go to ids0 / wts0 and ids1 / wts1 (K entries each) and
-// their final states to w0, w1.
-template <bool kCount = false>
-__device__ __forceinline__ void select_block(
+// it.  Lane l owns pixels (x0 + l % 8, y0 + 2 (l / 8)) and the one below.  The
+// survivors of the cull come four at a time, in list order: visit(j, a0, a1)
+// with the alpha' of entries st.g[j .. j + 3] at the two pixels, 0 where an
+// entry is no member (alpha' < alpha_min; alpha_min > 0), returns false once
+// every pixel of the warp has stopped.  st.g holds Gaussian ids, or with kPos
+// positions in isect_gid.
+template <bool kPos, typename Visit>
+__device__ __forceinline__ void walk_block(
     const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
     const float *__restrict__ rec_a, const float *__restrict__ rec_h,
-    const uint32_t *__restrict__ isect_gid, uint2 range, int W, int H, int x0, int y0, int K,
-    float alpha_min, float alpha_max, const float *s_thr, SelStage &st, int32_t *ids0, float *wts0,
-    int32_t *ids1, float *wts1, Walk &w0, Walk &w1) {
+    const uint32_t *__restrict__ isect_gid, uint2 range, int W, int H, int x0, int y0,
+    float alpha_min, float alpha_max, SelStage &st, Visit visit) {
     constexpr unsigned FULL = 0xffffffffu;
+    if (x0 >= W || y0 >= H) return;
     const int lane = threadIdx.x & 31;
     const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
-    const bool in0 = px < W && py < H, in1 = px < W && py + 1 < H;
     const float ux = float(px) + 0.5f;
     const float2 uy = make_float2(float(py) + 0.5f, float(py + 1) + 0.5f);
-    const float thr0 = s_thr[0];
-    w0 = Walk{1.0f, 1.0f, in0 ? thr0 : -1.0f, in0 ? 0 : K, 0};
-    w1 = Walk{1.0f, 1.0f, in1 ? thr0 : -1.0f, in1 ? 0 : K, 0};
-    if (x0 >= W || y0 >= H) return;
     // the block's box of pixel centres inside the image
     const float bx0 = float(x0) + 0.5f, bx1 = float(min(x0 + 7, W - 1)) + 0.5f;
     const float by0 = float(y0) + 0.5f, by1 = float(min(y0 + 7, H - 1)) + 0.5f;
 
-    // four survivors from st[j]; false once every pixel of the warp has stopped
+    // four survivors from st[j]
     auto step4 = [&](int j) -> bool {
         float a0[4], a1[4];
-        float2 t[4];
-        float2 T = make_float2(w0.T, w1.T);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const float4 mm = st.m[j + u];
@@ -160,30 +156,7 @@ __device__ __forceinline__ void select_block(
             a0[u] = (hq.x > ah.y || e0 < alpha_min) ? 0.0f : e0;
             a1[u] = (hq.y > ah.y || e1 < alpha_min) ? 0.0f : e1;
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            T = sel_mul2(T, sel_add2(make_float2(1.0f, 1.0f), make_float2(-a0[u], -a1[u])));
-            t[u] = T;
-        }
-        w0.T = T.x;
-        w1.T = T.y;
-        if (!__any_sync(FULL, T.x < w0.thr || T.y < w1.thr)) return true;
-        // the first crossing of each pixel, then the next (rarely a third)
-        do {
-            if (T.x < w0.thr) {
-                const int u = t[0].x < w0.thr ? 0 : t[1].x < w0.thr ? 1 : t[2].x < w0.thr ? 2 : 3;
-                const float a = u == 0 ? a0[0] : u == 1 ? a0[1] : u == 2 ? a0[2] : a0[3];
-                const float Tt = u == 0 ? t[0].x : u == 1 ? t[1].x : u == 2 ? t[2].x : t[3].x;
-                walk_event<kCount>(w0, Tt, a, st.g[j + u], s_thr, ids0, wts0);
-            }
-            if (T.y < w1.thr) {
-                const int u = t[0].y < w1.thr ? 0 : t[1].y < w1.thr ? 1 : t[2].y < w1.thr ? 2 : 3;
-                const float a = u == 0 ? a1[0] : u == 1 ? a1[1] : u == 2 ? a1[2] : a1[3];
-                const float Tt = u == 0 ? t[0].y : u == 1 ? t[1].y : u == 2 ? t[2].y : t[3].y;
-                walk_event<kCount>(w1, Tt, a, st.g[j + u], s_thr, ids1, wts1);
-            }
-        } while (__any_sync(FULL, T.x < w0.thr || T.y < w1.thr));
-        return !__all_sync(FULL, w0.k == K && w1.k == K);
+        return visit(j, a0, a1);
     };
 
     // entry base + lane of the list in registers; g1 / g2: its successors' ids
@@ -221,7 +194,7 @@ __device__ __forceinline__ void select_block(
             st.m[i] = cm;
             st.c[i] = cc;
             st.ah[i] = make_float2(ca, ch);
-            st.g[i] = cg;
+            st.g[i] = kPos ? b : cg;
         }
         const int n = left + __popc(bal), full = n & ~3;
         __syncwarp();
@@ -251,6 +224,55 @@ __device__ __forceinline__ void select_block(
     }
 }
 
+// Algorithm 1 over the block (walk_block): the kept entries of a lane's two
+// pixels go to ids0 / wts0 and ids1 / wts1 (K entries each) and their final
+// states to w0, w1.
+template <bool kCount = false>
+__device__ __forceinline__ void select_block(
+    const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+    const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+    const uint32_t *__restrict__ isect_gid, uint2 range, int W, int H, int x0, int y0, int K,
+    float alpha_min, float alpha_max, const float *s_thr, SelStage &st, int32_t *ids0, float *wts0,
+    int32_t *ids1, float *wts1, Walk &w0, Walk &w1) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
+    const bool in0 = px < W && py < H, in1 = px < W && py + 1 < H;
+    const float thr0 = s_thr[0];
+    w0 = Walk{1.0f, 1.0f, in0 ? thr0 : -1.0f, in0 ? 0 : K, 0};
+    w1 = Walk{1.0f, 1.0f, in1 ? thr0 : -1.0f, in1 ? 0 : K, 0};
+    auto visit = [&](int j, const float (&a0)[4], const float (&a1)[4]) -> bool {
+        float2 t[4];
+        float2 T = make_float2(w0.T, w1.T);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            T = sel_mul2(T, sel_add2(make_float2(1.0f, 1.0f), make_float2(-a0[u], -a1[u])));
+            t[u] = T;
+        }
+        w0.T = T.x;
+        w1.T = T.y;
+        if (!__any_sync(FULL, T.x < w0.thr || T.y < w1.thr)) return true;
+        // the first crossing of each pixel, then the next (rarely a third)
+        do {
+            if (T.x < w0.thr) {
+                const int u = t[0].x < w0.thr ? 0 : t[1].x < w0.thr ? 1 : t[2].x < w0.thr ? 2 : 3;
+                const float a = u == 0 ? a0[0] : u == 1 ? a0[1] : u == 2 ? a0[2] : a0[3];
+                const float Tt = u == 0 ? t[0].x : u == 1 ? t[1].x : u == 2 ? t[2].x : t[3].x;
+                walk_event<kCount>(w0, Tt, a, st.g[j + u], s_thr, ids0, wts0);
+            }
+            if (T.y < w1.thr) {
+                const int u = t[0].y < w1.thr ? 0 : t[1].y < w1.thr ? 1 : t[2].y < w1.thr ? 2 : 3;
+                const float a = u == 0 ? a1[0] : u == 1 ? a1[1] : u == 2 ? a1[2] : a1[3];
+                const float Tt = u == 0 ? t[0].y : u == 1 ? t[1].y : u == 2 ? t[2].y : t[3].y;
+                walk_event<kCount>(w1, Tt, a, st.g[j + u], s_thr, ids1, wts1);
+            }
+        } while (__any_sync(FULL, T.x < w0.thr || T.y < w1.thr));
+        return !__all_sync(FULL, w0.k == K && w1.k == K);
+    };
+    walk_block<false>(rec_m, rec_w, rec_a, rec_h, isect_gid, range, W, H, x0, y0, alpha_min, alpha_max,
+                      st, visit);
+}
+
 // A pixel's kept weights divided by 1 - T^Q (kCount: by the boundaries crossed
 // in all), the rest of its K slots padded with id -1 and weight 0.
 template <bool kCount = false>
@@ -263,14 +285,14 @@ __device__ __forceinline__ void finish_pixel(const Walk &w, int K, int32_t *ids,
     }
 }
 
-// Writes the finished block at (x0, y0) (slot of pixel (x, y): s0 + y stride +
-// x) to the image's ids and weights; the warp's lanes must have finished
-// their pixels (__syncwarp between).  Rows of a block are 8 K consecutive
-// entries of the image; vec (K % 4 == 0 and 16-byte aligned outputs) writes
-// them four at a time.
-__device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K, bool vec,
-                                            const int32_t *s_ids, const float *s_w, int s0, int stride,
-                                            int32_t *__restrict__ ids, float *__restrict__ wout) {
+// Writes a finished array of the block at (x0, y0) (K entries per pixel, of
+// pixel (x, y) at slot_of(x, y) KS in shared memory) to the image's array; the
+// warp's lanes must have finished their pixels (__syncwarp between).  Rows of
+// a block are 8 K consecutive entries of the image; vec (K % 4 == 0 and
+// 16-byte aligned outputs) writes them four at a time.
+template <typename SlotOf, typename Put>
+__device__ __forceinline__ void for_block(int W, int H, int x0, int y0, int K, bool vec,
+                                          SlotOf slot_of, Put put) {
     const int lane = threadIdx.x & 31;
     const int KS = K | 1;
     const int per = vec ? 4 : 1;
@@ -280,8 +302,14 @@ __device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K,
         const int pix = int((uint32_t(e) * inv) >> 16), j = (e - pix * KP) * per;
         const int x = x0 + (pix & 7), y = y0 + (pix >> 3);
         if (x >= W || y >= H) continue;
-        const int at = (s0 + (pix >> 3) * stride + (pix & 7)) * KS + j;
-        const int64_t o = (int64_t(y) * W + x) * K + j;
+        put(slot_of(pix & 7, pix >> 3) * KS + j, (int64_t(y) * W + x) * K + j);
+    }
+}
+template <typename SlotOf>
+__device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K, bool vec,
+                                            const int32_t *s_ids, const float *s_w, SlotOf slot_of,
+                                            int32_t *__restrict__ ids, float *__restrict__ wout) {
+    for_block(W, H, x0, y0, K, vec, slot_of, [&](int at, int64_t o) {
         if (vec) {
             *reinterpret_cast<int4 *>(ids + o) = make_int4(s_ids[at], s_ids[at + 1], s_ids[at + 2], s_ids[at + 3]);
             *reinterpret_cast<float4 *>(wout + o) = make_float4(s_w[at], s_w[at + 1], s_w[at + 2], s_w[at + 3]);
@@ -289,7 +317,7 @@ __device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K,
             ids[o] = s_ids[at];
             wout[o] = s_w[at];
         }
-    }
+    });
 }
 
 }  // namespace qr

@@ -89,6 +89,17 @@ def test_room_small_ragged(rule, tile):
     print(f"room-small {NAMES[rule]} tile {tile}", rep)
 
 
+@pytest.mark.parametrize("rule", [oracle.RULE_TOPK, oracle.RULE_STRATIFIED])
+@pytest.mark.parametrize("K,tile", [(2, (32, 8)), (5, (16, 16)), (16, (32, 8)), (31, (16, 16))])
+def test_rule_blocks_ragged(rule, K, tile):
+    """Slot counts that fill, partly fill and overflow groups of four, and
+    images whose last 8 x 8 blocks are cut (or empty) in both directions."""
+    g, f = H.small_room(n=20000, channels=16)
+    cam = scenes.room_camera(113, 67)
+    _run(g, None, cam, rule, K, params_kw={"tile_w": tile[0], "tile_h": tile[1]},
+         label=f"blocks {NAMES[rule]} K={K} {tile}")
+
+
 @pytest.mark.parametrize("rule", RULES)
 def test_indoor_full_size_sampled(rule):
     """The 500k-Gaussian 640x480 512-D workload, on sampled pixels."""
