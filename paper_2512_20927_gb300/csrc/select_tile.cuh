@@ -113,15 +113,18 @@ __device__ __forceinline__ void walk_event(Walk &w, float Tt, float a, uint32_t 
     ++w.m;
 }
 
-// Walks the 8 x 8 block at (x0, y0) over isect_gid[range.x, range.y), the
-// depth-ordered list of the tile that holds it.  All lanes of the warp call
-// it.  Lane l owns pixels (x0 + l % 8, y0 + 2 (l / 8)) and the one below.  The
-// survivors of the cull come four at a time, in list order: visit(j, a0, a1)
-// with the alpha' of entries st.g[j .. j + 3] at the two pixels, 0 where an
-// entry is no member (alpha' < alpha_min; alpha_min > 0), returns false once
-// every pixel of the warp has stopped.  st.g holds Gaussian ids, or with kPos
-// positions in isect_gid.
-template <bool kPos, typename Visit>
+// Walks the block at (x0, y0) -- 8 x 8 pixels, or 8 x 4 with PX = 1 -- over
+// isect_gid[range.x, range.y), the depth-ordered list of the tile that holds
+// it.  All lanes of the warp call it.  Lane l owns the PX pixels from
+// (x0 + l % 8, y0 + PX (l / 8)) down.  The survivors of the cull come four at
+// a time, in list order: visit(j, a) with the alpha' of entries st.g[j .. j +
+// 3] at the lane's pixels, a[u][i], 0 where an entry is no member (alpha' <
+// alpha_min; alpha_min > 0), returns false once every pixel of the warp has
+// stopped.  st.g holds Gaussian ids, or with kPos positions in isect_gid.
+// The last step is filled up with entries out of reach, so the step's code
+// stands in the kernel once (twice, its misses in the instruction cache
+// bounded the larger callers).
+template <bool kPos, int PX, typename Visit>
 __device__ __forceinline__ void walk_block(
     const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
     const float *__restrict__ rec_a, const float *__restrict__ rec_h,
@@ -130,33 +133,39 @@ __device__ __forceinline__ void walk_block(
     constexpr unsigned FULL = 0xffffffffu;
     if (x0 >= W || y0 >= H) return;
     const int lane = threadIdx.x & 31;
-    const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
+    const int px = x0 + (lane & 7), py = y0 + PX * (lane >> 3);
     const float ux = float(px) + 0.5f;
     const float2 uy = make_float2(float(py) + 0.5f, float(py + 1) + 0.5f);
     // the block's box of pixel centres inside the image
     const float bx0 = float(x0) + 0.5f, bx1 = float(min(x0 + 7, W - 1)) + 0.5f;
-    const float by0 = float(y0) + 0.5f, by1 = float(min(y0 + 7, H - 1)) + 0.5f;
+    const float by0 = float(y0) + 0.5f, by1 = float(min(y0 + 4 * PX - 1, H - 1)) + 0.5f;
 
     // four survivors from st[j]
     auto step4 = [&](int j) -> bool {
-        float a0[4], a1[4];
+        float a[4][PX];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             const float4 mm = st.m[j + u];
             const float4 cc = st.c[j + u];
             const float2 ah = st.ah[j + u];
-            // eval_half_q for both pixels: dx shared, the rest packed
-            const float dx = (ux - mm.x) - mm.z;
-            const float2 dy = sel_add2(sel_add2(uy, make_float2(-mm.y, -mm.y)), make_float2(-mm.w, -mm.w));
-            const float2 dx2 = make_float2(dx, dx);
-            const float2 p1 = sel_fma2(dx2, make_float2(cc.x, cc.x), sel_mul2(dy, make_float2(cc.y, cc.y)));
-            const float2 p2 = sel_fma2(dx2, make_float2(cc.z, cc.z), sel_mul2(dy, make_float2(cc.w, cc.w)));
-            const float2 hq = sel_fma2(p1, p1, sel_mul2(p2, p2));
-            const float e0 = eval_alpha(ah.x, hq.x, alpha_max), e1 = eval_alpha(ah.x, hq.y, alpha_max);
-            a0[u] = (hq.x > ah.y || e0 < alpha_min) ? 0.0f : e0;
-            a1[u] = (hq.y > ah.y || e1 < alpha_min) ? 0.0f : e1;
+            if constexpr (PX == 1) {
+                const float hq = eval_half_q(ux, uy.x, mm, cc).half_q;
+                const float e = eval_alpha(ah.x, hq, alpha_max);
+                a[u][0] = (hq > ah.y || e < alpha_min) ? 0.0f : e;
+            } else {
+                // eval_half_q for both pixels: dx shared, the rest packed
+                const float dx = (ux - mm.x) - mm.z;
+                const float2 dy = sel_add2(sel_add2(uy, make_float2(-mm.y, -mm.y)), make_float2(-mm.w, -mm.w));
+                const float2 dx2 = make_float2(dx, dx);
+                const float2 p1 = sel_fma2(dx2, make_float2(cc.x, cc.x), sel_mul2(dy, make_float2(cc.y, cc.y)));
+                const float2 p2 = sel_fma2(dx2, make_float2(cc.z, cc.z), sel_mul2(dy, make_float2(cc.w, cc.w)));
+                const float2 hq = sel_fma2(p1, p1, sel_mul2(p2, p2));
+                const float e0 = eval_alpha(ah.x, hq.x, alpha_max), e1 = eval_alpha(ah.x, hq.y, alpha_max);
+                a[u][0] = (hq.x > ah.y || e0 < alpha_min) ? 0.0f : e0;
+                a[u][1] = (hq.y > ah.y || e1 < alpha_min) ? 0.0f : e1;
+            }
         }
-        return visit(j, a0, a1);
+        return visit(j, a);
     };
 
     // entry base + lane of the list in registers; g1 / g2: its successors' ids
@@ -196,7 +205,17 @@ __device__ __forceinline__ void walk_block(
             st.ah[i] = make_float2(ca, ch);
             st.g[i] = kPos ? b : cg;
         }
-        const int n = left + __popc(bal), full = n & ~3;
+        int n = left + __popc(bal);
+        if (range.y - base <= 32) {   // the end of the list: fill up to a whole step
+            if (lane < ((4 - n) & 3)) {
+                st.m[n + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+                st.c[n + lane] = make_float4(0.f, 0.f, 0.f, 0.f);
+                st.ah[n + lane] = make_float2(0.f, -1.f);
+                st.g[n + lane] = 0u;
+            }
+            n = (n + 3) & ~3;
+        }
+        const int full = n & ~3;
         __syncwarp();
         for (int j = 0; j < full; j += 4)
             if (!step4(j)) return;
@@ -211,16 +230,6 @@ __device__ __forceinline__ void walk_block(
             }
             __syncwarp();
         }
-    }
-    if (left) {   // the last step, filled up with entries out of reach
-        if (lane >= left && lane < 4) {
-            st.m[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-            st.c[lane] = make_float4(0.f, 0.f, 0.f, 0.f);
-            st.ah[lane] = make_float2(0.f, -1.f);
-            st.g[lane] = 0u;
-        }
-        __syncwarp();
-        step4(0);
     }
 }
 
@@ -241,12 +250,12 @@ __device__ __forceinline__ void select_block(
     const float thr0 = s_thr[0];
     w0 = Walk{1.0f, 1.0f, in0 ? thr0 : -1.0f, in0 ? 0 : K, 0};
     w1 = Walk{1.0f, 1.0f, in1 ? thr0 : -1.0f, in1 ? 0 : K, 0};
-    auto visit = [&](int j, const float (&a0)[4], const float (&a1)[4]) -> bool {
+    auto visit = [&](int j, const float (&a)[4][2]) -> bool {
         float2 t[4];
         float2 T = make_float2(w0.T, w1.T);
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            T = sel_mul2(T, sel_add2(make_float2(1.0f, 1.0f), make_float2(-a0[u], -a1[u])));
+            T = sel_mul2(T, sel_add2(make_float2(1.0f, 1.0f), make_float2(-a[u][0], -a[u][1])));
             t[u] = T;
         }
         w0.T = T.x;
@@ -256,20 +265,20 @@ __device__ __forceinline__ void select_block(
         do {
             if (T.x < w0.thr) {
                 const int u = t[0].x < w0.thr ? 0 : t[1].x < w0.thr ? 1 : t[2].x < w0.thr ? 2 : 3;
-                const float a = u == 0 ? a0[0] : u == 1 ? a0[1] : u == 2 ? a0[2] : a0[3];
+                const float e = u == 0 ? a[0][0] : u == 1 ? a[1][0] : u == 2 ? a[2][0] : a[3][0];
                 const float Tt = u == 0 ? t[0].x : u == 1 ? t[1].x : u == 2 ? t[2].x : t[3].x;
-                walk_event<kCount>(w0, Tt, a, st.g[j + u], s_thr, ids0, wts0);
+                walk_event<kCount>(w0, Tt, e, st.g[j + u], s_thr, ids0, wts0);
             }
             if (T.y < w1.thr) {
                 const int u = t[0].y < w1.thr ? 0 : t[1].y < w1.thr ? 1 : t[2].y < w1.thr ? 2 : 3;
-                const float a = u == 0 ? a1[0] : u == 1 ? a1[1] : u == 2 ? a1[2] : a1[3];
+                const float e = u == 0 ? a[0][1] : u == 1 ? a[1][1] : u == 2 ? a[2][1] : a[3][1];
                 const float Tt = u == 0 ? t[0].y : u == 1 ? t[1].y : u == 2 ? t[2].y : t[3].y;
-                walk_event<kCount>(w1, Tt, a, st.g[j + u], s_thr, ids1, wts1);
+                walk_event<kCount>(w1, Tt, e, st.g[j + u], s_thr, ids1, wts1);
             }
         } while (__any_sync(FULL, T.x < w0.thr || T.y < w1.thr));
         return !__all_sync(FULL, w0.k == K && w1.k == K);
     };
-    walk_block<false>(rec_m, rec_w, rec_a, rec_h, isect_gid, range, W, H, x0, y0, alpha_min, alpha_max,
+    walk_block<false, 2>(rec_m, rec_w, rec_a, rec_h, isect_gid, range, W, H, x0, y0, alpha_min, alpha_max,
                       st, visit);
 }
 
