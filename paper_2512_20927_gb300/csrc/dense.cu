@@ -6,11 +6,11 @@
 // fall below T_min.
 //
 // GB300 design: every pixel of a tile walks the same list, so the blend is a
-// dense product W (pixels x batch) * F (batch x channels) per batch of 32
-// list entries.  Rows of 128, 256 or 512 channels go to dense_sub_kernel
-// (below: one CTA per 64-pixel sub-tile over all channels, warp-specialised
-// walk and accumulation).  Other widths use dense_kernel, where one CTA owns
-// a screen tile and a 16/32/64-channel slice:
+// dense product W (pixels x entries) * F (entries x channels).  Rows of 128,
+// 256 or 512 channels go to dense_block_kernel (below: warp-specialised walk,
+// row copies and accumulation over 8 x 8 pixel blocks).  Other widths use
+// dense_kernel, 32 list entries at a time, where one CTA owns a screen tile
+// and a 16/32/64-channel slice:
 //   1. the batch's Gaussian records and feature-row slices are staged in
 //      shared memory (coalesced 16-byte loads; BF16/FP8 widened here),
 //   2. each thread walks its own pixel over the batch (scalar FP32, the exact
@@ -20,10 +20,9 @@
 //      load feeds 8 FMAs.
 // FP32 is kept on purpose: Eq. 1 is compared element by element with an FP64
 // oracle, which a TF32/BF16 tensor-core product would not meet.
-#include <cuda_bf16.h>
-#include <cuda_fp8.h>
-
-#include "qr_internal.cuh"
+#include "quad.cuh"
+#include "select_tile.cuh"
+#include "tma.cuh"
 
 namespace qr {
 namespace {
@@ -197,326 +196,396 @@ dense_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
     if (T_final && blockIdx.y == 0 && inside) T_final[int64_t(py) * W + px] = T;
 }
 
-// ------------------------------------------------------------------ sub-tile kernel
-// One CTA renders a 64-pixel sub-tile of a screen tile (16x4, 8x8 or 32x2)
-// over all C channels (C = 64 CH, CH = 2, 4 or 8), so each pixel's alpha' / T
-// walk runs once.  The CTA is warp-specialised and double-buffered, so the
-// serial walk of one batch of list entries overlaps the accumulation of the
-// previous one:
-//   producers (warps 16, 17: one thread per pixel), per batch of 32 entries:
-//     1. cull the batch's records (loaded into registers while the previous
-//        batch was walked) against the sub-tile's box of pixel centres (the
-//        conservative test of the selection);
-//     2. walk every pixel over the survivors in list order (the scalar FP32
-//        recurrence of dense_kernel) and write w = T alpha' into W[slot];
-//     3. list, in list order, the survivors with a nonzero weight anywhere in
-//        the sub-tile (and their ids);
-//   consumers (warps 0-15: warps 2g and 2g+1 own pixel group g, a 4x2 block
-//   of 8 pixels): stage the kept entries' feature rows in shared memory
-//   (FP32 rows by 16-byte cp.async, BF16 / FP8 rows widened), then per kept
-//   entry 8 weights and CH features per thread, 8 CH FMAs; an entry whose 8
-//   weights are all zero is skipped by the warp.
-// Hand-over through hardware named barriers: FULL[slot] (producers arrive
-// once the slot is written, consumers wait) and EMPTY[slot] (consumers arrive
-// once the slot is read, producers wait before writing it again and, at the
-// end, for every slot still unread), so every barrier phase is matched.  A
-// slot whose kept count is -1 ends the consumers' loop.  Zero weights add
-// nothing (fmaf(0, f, acc) == acc), so the result equals dense_kernel's.
+// ------------------------------------------------------------------ block kernel
+// Rows of 128, 256 or 512 channels.  One persistent CTA per SM; a work item is
+// an 8 x 8 pixel block over all C channels, so each pixel's alpha' / T walk
+// runs once.  The blend itself (8 pixels x C channels per group and kept
+// entry) is bound by the FP32 pipe, so everything else runs beside it in
+// warps of its own, far enough ahead that the consumers never wait for a walk
+// or a row:
+//   consumers (8 pixel groups of 4 x 2 pixels, WPG warps each): per kept entry
+//     of their group 8 weights and 4 QPT channels per lane from shared memory,
+//     8 x 4 QPT multiply-adds in packed FP32x2 instructions; a bit mask per
+//     group and slot holds the entries with a nonzero weight in it;
+//   producers (kProd warps, a block each in turn): walk_block's cull and
+//     alpha', T, and w = T alpha'; the entries with a nonzero weight anywhere
+//     in the block go, in list order, to the producer's ring of kSlots slots
+//     of kEnt entries (weights, ids, group masks), a whole block ahead;
+//   loader (1 warp): in consumption order, copies the rows of a slot's entries
+//     as stored (cp.async.bulk, one copy per row) into a ring of kRows row
+//     slots; BF16 / FP8 are widened in the consumers' registers.
+// A producer that takes a block asks for the next one, which goes to the next
+// producer: the launch of a CTA that has not begun is cancelled and its work
+// taken over (clusterlaunchcontrol), so lists of very different lengths
+// balance without a counter in memory.
+// Every hand-over is an mbarrier with a bounded wait; a wait that runs out
+// sets a flag that ends every role, the copies in flight are waited for, and
+// the frame's status reports QR_ERR_DEVICE_TIMEOUT.
+// Zero weights add nothing (fmaf(0, f, acc) == acc) and the entries are summed
+// in list order, so the result equals dense_kernel's bit for bit.
 // stats (nullable): [0] += blended (pixel, Gaussian) pairs, [1] += executed
 // multiply-adds.
-constexpr int S_CONS = 512;                  // consumer threads (16 warps)
-constexpr int S_PROD = 64;                   // producer threads (2 warps, one per pixel)
-constexpr int S_THREADS = S_CONS + S_PROD;
-constexpr int S_PIX = 64;
-constexpr int S_BATCH = 32;
-// named barriers (0 is __syncthreads)
-constexpr int kBarFull = 1;                  // + slot
-constexpr int kBarEmpty = 3;                 // + slot
-constexpr int kBarProd = 5;
-constexpr int kBarCons = 6;
+// Room VGA, 500k Gaussians, 512 FP32 channels (21.5 GFLOP useful, 1.1 times
+// that executed): 1379 us with one CTA per 16 x 4 pixels that walked, staged
+// rows and accumulated 32 list entries (9 survivors) at a time behind named
+// barriers; 566 us now.  The roles alone: consumers 320 us at the FP32 peak,
+// walk and copies without the multiply-adds 326 us.  Five warps per scheduler
+// (20 in all) leave a consumer 96 registers; a 21st warp cost 80 and spills
+// (1096 us), two producers 585 us.
+constexpr int kProd = 3;                     // producer warps
+constexpr int kSlots = 6;                    // weight slots per producer
+constexpr int kEnt = 16;                     // entries per slot
+constexpr int kRows = 4;                     // row slots
+constexpr int kItemEnd = -1;
+constexpr unsigned kDenseSpin = 1u << 26;    // polls before a wait gives up
 
-__device__ __forceinline__ void nbar_sync(int id, int n) {
-    asm volatile("bar.sync %0, %1;" :: "r"(id), "r"(n) : "memory");
+struct DenseSlot {
+    float w[kEnt][kSelBlock];                // pixel slot 8 g + i of group g
+    uint32_t gid[kEnt];
+    uint32_t mask[8];                        // per group: entries with a nonzero weight
+    int n, last, block;                      // entries; last slot of its block; block or kItemEnd
+    int pad;
+};
+struct DenseRow {                            // what a row slot holds
+    int slot, n, last, block;                // slot: producer * kSlots + weight slot
+    float scale[kEnt];
+};
+struct DenseShared {
+    DenseSlot slot[kProd][kSlots];
+    DenseRow row[kRows];
+    SelStage st[kProd];
+    uint64_t w_full[kProd][kSlots], w_empty[kProd][kSlots];
+    uint64_t r_full[kRows], r_empty[kRows];
+    uint64_t mail_full[kProd], mail_empty[kProd], clc;
+    alignas(16) uint4 response;
+    int mail[kProd];
+    int abort;
+};
+constexpr size_t kDenseShared = (sizeof(DenseShared) + 127) / 128 * 128;
+
+__device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tma_smem_addr(bar)) : "memory");
 }
-__device__ __forceinline__ void nbar_arrive(int id, int n) {
-    asm volatile("bar.arrive %0, %1;" :: "r"(id), "r"(n) : "memory");
+// Bounded wait; false when it ran out or another role has given up.
+__device__ __forceinline__ bool dense_wait(uint64_t *bar, uint32_t parity, volatile int *abort) {
+    for (unsigned i = 0; i < kDenseSpin; i += 1024) {
+        if (tma_mbar_wait(bar, parity, 1024)) return true;
+        if (*abort) return false;
+    }
+    *abort = 1;
+    return false;
 }
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
-                 :: "r"(uint32_t(__cvta_generic_to_shared(smem))), "l"(gmem) : "memory");
+__device__ __forceinline__ void bulk_row(void *dst, const void *src, uint32_t bytes, uint64_t *bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 :: "r"(tma_smem_addr(dst)), "l"(src), "r"(bytes), "r"(tma_smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ void try_cancel(uint4 *response, uint64_t *bar) {
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 :: "r"(tma_smem_addr(response)), "r"(tma_smem_addr(bar)) : "memory");
+}
+// The CTA whose launch was cancelled, or -1 when none was left.
+__device__ __forceinline__ int cancelled_cta(const uint4 *response) {
+    int got, x;
+    asm volatile("{\n .reg .b128 r;\n .reg .pred p;\n ld.shared.b128 r, [%2];\n"
+                 " clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n"
+                 " selp.s32 %0, 1, 0, p;\n mov.s32 %1, 0;\n"
+                 " @p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, r;\n}\n"
+                 : "=r"(got), "=r"(x) : "r"(tma_smem_addr(response)) : "memory");
+    return got ? x : -1;
 }
 
-template <int DT, int CH>
-__global__ void __launch_bounds__(S_THREADS, 1)
-dense_sub_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
-                 const float *__restrict__ rec_a, const float *__restrict__ rec_h,
-                 const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges,
-                 const unsigned char *__restrict__ feat, const float *__restrict__ fscale, int C,
-                 int W, int H, int tile_w, int tiles_x, float alpha_min, float alpha_max,
-                 float T_min, float *__restrict__ out, float *__restrict__ T_final,
-                 unsigned long long *__restrict__ stats) {
-    constexpr int CPV = Cpv<DT>::v;
-    constexpr int ESZ = DT == QR_F32 ? 4 : DT == QR_BF16 ? 2 : 1;
+__device__ __forceinline__ void fma2d(float *acc, float w, float x0, float x1) {
+    asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %2};\n"
+        " mov.b64 xx, {%3, %4};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
+        : "+f"(acc[0]), "+f"(acc[1]) : "f"(w), "f"(x0), "f"(x1));
+}
+
+struct BlockPos {
+    int tile, x0, y0;
+};
+__device__ __forceinline__ BlockPos dense_block(int block, int tile_w, int tiles_x) {
+    const int tile = block >> 2, part = block & 3, across = tile_w >> 3;
+    return {tile, (tile % tiles_x) * tile_w + (part % across) * 8,
+            (tile / tiles_x) * (kSelPix / tile_w) + (part / across) * 8};
+}
+
+template <int WPG>
+constexpr int dense_threads() { return 32 * (8 * WPG + kProd + 1); }
+
+// C = 128 WPG QPT
+template <int DT, int QPT, int WPG>
+__global__ void __launch_bounds__(dense_threads<WPG>(), 1)
+dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+                   const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+                   const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges,
+                   const unsigned char *__restrict__ feat, const float *__restrict__ fscale, int W,
+                   int H, int tile_w, int tiles_x, float alpha_min, float alpha_max, float T_min,
+                   float *__restrict__ out, float *__restrict__ T_final,
+                   unsigned long long *__restrict__ stats, uint32_t *__restrict__ counters) {
     constexpr unsigned FULL = 0xffffffffu;
-    // producer state
-    __shared__ float4 s_m[S_BATCH];
-    __shared__ float4 s_c[S_BATCH];
-    __shared__ float s_a[S_BATCH];
-    __shared__ float s_h[S_BATCH];
-    __shared__ uint32_t s_g[S_BATCH];
-    __shared__ int s_surv[S_BATCH];          // survivor -> staged entry
-    __shared__ int s_ns;
-    __shared__ int s_done[2];
-    __shared__ float s_box[4];
-    // double-buffered hand-over
-    __shared__ __align__(16) float s_W[2][S_BATCH][S_PIX];
-    __shared__ int s_used[2][S_BATCH];       // kept -> survivor
-    __shared__ uint32_t s_kg[2][S_BATCH];    // kept -> Gaussian id
-    __shared__ int s_nu[2];                  // kept entries, -1 = end
-    extern __shared__ __align__(16) float s_F[];     // [S_BATCH][C], the consumers' rows
-
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tile = blockIdx.x >> 2, sub = blockIdx.x & 3;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int tile_h = 256 / tile_w, sub_h = S_PIX / tile_w;
-    const int gx_n = tile_w / 4;                       // pixel groups across
-    // pixel slot ps = 8 g + i  ->  (lx, ly) in the sub-tile
-    auto slot_xy = [&](int ps, int &x, int &y) {       // groups of 4 x 2 pixels
-        const int g = ps >> 3, i = ps & 7;
-        x = tx * tile_w + (g % gx_n) * 4 + (i & 3);
-        y = ty * tile_h + sub * sub_h + (g / gx_n) * 2 + (i >> 2);
-    };
-    const uint2 range = ranges[tile];
-    const bool producer = tid >= S_CONS;
-    if (tid >= S_CONS && tid < S_CONS + 32) {
-        // the sub-tile's box of pixel centres (clipped to the image)
-        float bx0 = 1e30f, bx1 = -1e30f, by0 = 1e30f, by1 = -1e30f;
-        for (int ps = lane; ps < S_PIX; ps += 32) {
-            int x, y;
-            slot_xy(ps, x, y);
-            const float cx = float(x) + 0.5f, cy = float(y) + 0.5f;
-            bx0 = fminf(bx0, cx); bx1 = fmaxf(bx1, cx); by0 = fminf(by0, cy); by1 = fmaxf(by1, cy);
+    constexpr int QB = Quad<DT>::B;
+    constexpr int C = 128 * WPG * QPT;
+    constexpr uint32_t ROW = uint32_t(C / 4) * QB;           // bytes of a row
+    constexpr int NCW = 8 * WPG;                             // consumer warps
+    extern __shared__ __align__(128) unsigned char s_dyn[];
+    DenseShared &sh = *reinterpret_cast<DenseShared *>(s_dyn);
+    unsigned char *s_rows = s_dyn + kDenseShared;            // [kRows][kEnt][ROW]
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) {
+        for (int p = 0; p < kProd; ++p) {
+            for (int s = 0; s < kSlots; ++s) {
+                tma_mbar_init(&sh.w_full[p][s], 1);
+                tma_mbar_init(&sh.w_empty[p][s], NCW);
+            }
+            tma_mbar_init(&sh.mail_full[p], 1);
+            tma_mbar_init(&sh.mail_empty[p], 1);
         }
-        for (int o = 16; o > 0; o >>= 1) {
-            bx0 = fminf(bx0, __shfl_xor_sync(FULL, bx0, o));
-            bx1 = fmaxf(bx1, __shfl_xor_sync(FULL, bx1, o));
-            by0 = fminf(by0, __shfl_xor_sync(FULL, by0, o));
-            by1 = fmaxf(by1, __shfl_xor_sync(FULL, by1, o));
+        for (int r = 0; r < kRows; ++r) {
+            tma_mbar_init(&sh.r_full[r], 1);
+            tma_mbar_init(&sh.r_empty[r], NCW);
         }
-        if (lane == 0) { s_box[0] = bx0; s_box[1] = bx1; s_box[2] = by0; s_box[3] = by1; }
+        tma_mbar_init(&sh.clc, 1);
+        sh.abort = 0;
+        sh.mail[0] = int(blockIdx.x);      // the first block, already delivered
+        mbar_arrive(&sh.mail_full[0]);
+        tma_fence_init();
     }
     __syncthreads();
-    const size_t row_bytes = size_t(C) * ESZ;
+    volatile int *abort = &sh.abort;
 
-    if (producer) {
-        // ---------------------------------------------------------- producers
-        const int pt = tid - S_CONS, pw = pt >> 5;     // pixel slot, producer warp
-        int px, py;
-        slot_xy(pt, px, py);
-        const bool inside = px < W && py < H;
-        const float ux = float(px) + 0.5f, uy = float(py) + 0.5f;
-        float T = 1.0f;
-        bool done = !inside;
-        unsigned long long n_blend = 0;
-        bool pending[2] = {false, false};
-        int sl = 0;
-        // producer warp 0 holds the next batch's records in registers: their
-        // loads (the list ids, then the records) run while the current batch
-        // is walked
-        uint32_t n_gid = 0;
-        float4 n_m = make_float4(0.f, 0.f, 0.f, 0.f), n_c = n_m;
-        float n_a = 0.f, n_h = 0.f;
-        auto prefetch = [&](uint32_t bb) {
-            if (pw == 0 && bb < range.y && uint32_t(lane) < range.y - bb) {
-                n_gid = isect_gid[bb + lane];
-                n_m = rec_m[n_gid];
-                n_c = rec_w[n_gid];
-                n_a = rec_a[n_gid];
-                n_h = rec_h[n_gid];
+    if (warp < NCW) {
+        // ------------------------------------------------------ consumers
+        const int g = warp / WPG;
+        const int q0 = (warp % WPG) * 32 + lane;             // first quad; then + 32 WPG
+        float acc[8][QPT][4];
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+            for (int k = 0; k < QPT; ++k)
+#pragma unroll
+                for (int c = 0; c < 4; ++c) acc[i][k][c] = 0.f;
+        unsigned long long n_exec = 0;
+        for (uint32_t it = 0;; ++it) {
+            const uint32_t r = it % kRows, ph = (it / kRows) & 1u;
+            if (!dense_wait(&sh.r_full[r], ph, abort)) break;
+            const DenseRow &R = sh.row[r];
+            const int block = R.block, last = R.last, at = R.slot;
+            if (block == kItemEnd) break;
+            const DenseSlot &S = sh.slot[0][at];
+            const unsigned char *rows = s_rows + size_t(r) * kEnt * ROW + size_t(q0) * QB;
+            uint32_t mask = S.mask[g];
+            n_exec += __popc(mask);
+            while (mask) {
+                const int e = __ffs(mask) - 1;
+                mask &= mask - 1u;
+                const float4 *wr = reinterpret_cast<const float4 *>(&S.w[e][8 * g]);
+                const float4 wa = wr[0], wb = wr[1];
+                const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                const float sc = DT == QR_FP8E4M3 ? R.scale[e] : 1.f;
+#pragma unroll
+                for (int k = 0; k < QPT; ++k) {
+                    float f[4];
+                    dec_quad<DT>(*reinterpret_cast<const typename Quad<DT>::T *>(rows + uint32_t(e) * ROW +
+                                                                                 uint32_t(32 * WPG * k) * QB), f);
+                    if constexpr (DT == QR_FP8E4M3) {
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) f[c] *= sc;
+                    }
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        fma2d(acc[i][k], wv[i], f[0], f[1]);
+                        fma2d(acc[i][k] + 2, wv[i], f[2], f[3]);
+                    }
+                }
             }
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&sh.r_empty[r]);
+                mbar_arrive(&sh.w_empty[0][at]);
+            }
+            if (last) {
+                const BlockPos b = dense_block(block, tile_w, tiles_x);
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    const int x = b.x0 + (g & 1) * 4 + (i >> 1), y = b.y0 + (g >> 1) * 2 + (i & 1);
+                    float4 *o = reinterpret_cast<float4 *>(out) + (int64_t(y) * W + x) * (C / 4) + q0;
+#pragma unroll
+                    for (int k = 0; k < QPT; ++k) {
+                        if (x < W && y < H)
+                            __stcs(o + 32 * WPG * k, make_float4(acc[i][k][0], acc[i][k][1], acc[i][k][2], acc[i][k][3]));
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) acc[i][k][c] = 0.f;
+                    }
+                }
+            }
+        }
+        if (stats && lane == 0) atomicAdd(&stats[1], n_exec * 32ull * 8ull * 4ull * QPT);
+    } else if (warp < NCW + kProd) {
+        // ------------------------------------------------------ producers
+        const int p = warp - NCW;
+        SelStage &st = sh.st[p];
+        uint32_t sc = 0;                   // slots begun
+        int e = -1;                        // entries of the open slot, -1: none open
+        uint32_t gmask = 0;                // lane g < 8: the open slot's mask of group g
+        bool ok = true;
+        auto open = [&]() {
+            if (e >= 0) return;
+            ok = ok && dense_wait(&sh.w_empty[p][sc % kSlots], ((sc / kSlots) & 1u) ^ 1u, abort);
+            ok = __all_sync(FULL, ok);
+            e = 0;
+            gmask = 0;
         };
-        prefetch(range.x);
-        for (uint32_t b = range.x;; b += S_BATCH) {
-            const unsigned dv = __ballot_sync(FULL, done);
-            if (lane == 0) s_done[pw] = dv == FULL;
-            nbar_sync(kBarProd, S_PROD);
-            const bool all_done = s_done[0] && s_done[1];
-            nbar_sync(kBarProd, S_PROD);               // s_done is read before it is rewritten
-            if (b >= range.y || all_done) break;
-            const int nb = int(min(uint32_t(S_BATCH), range.y - b));
-            // 1. stage and cull (producer warp 0, one entry per lane)
-            if (pw == 0) {
-                bool pass = false;
-                if (lane < nb) {
-                    s_g[lane] = n_gid;
-                    s_m[lane] = n_m;
-                    s_c[lane] = n_c;
-                    s_a[lane] = n_a;
-                    s_h[lane] = n_h;
-                    pass = !(box_min_half_q(n_m, n_c, s_box[0], s_box[1], s_box[2], s_box[3]) * 0.999f >
-                             n_h + 1e-3f);
+        auto commit = [&](int last, int block) {
+            DenseSlot &S = sh.slot[p][sc % kSlots];
+            if (lane < 8) S.mask[lane] = gmask;
+            if (lane == 0) {
+                S.n = e;
+                S.last = last;
+                S.block = block;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.w_full[p][sc % kSlots]);
+            ++sc;
+            e = -1;
+        };
+        for (uint32_t j = 0; ok; ++j) {
+            ok = __all_sync(FULL, dense_wait(&sh.mail_full[p], j & 1u, abort));
+            if (!ok) break;
+            const int block = sh.mail[p];
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&sh.mail_empty[p]);
+                // the next producer's block (none is asked for after a refusal)
+                const uint32_t i = j * kProd + uint32_t(p), p1 = (i + 1) % kProd;
+                int next = kItemEnd;
+                if (block != kItemEnd) {
+                    // the previous response was read through the generic proxy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    tma_expect_tx(&sh.clc, 16);
+                    try_cancel(&sh.response, &sh.clc);
+                    ok = dense_wait(&sh.clc, i & 1u, abort);
+                    if (ok) next = cancelled_cta(&sh.response);
                 }
-                const unsigned bal = __ballot_sync(FULL, pass);
-                if (pass) s_surv[__popc(bal & ((1u << lane) - 1u))] = lane;
-                if (lane == 0) s_ns = __popc(bal);
-                prefetch(b + S_BATCH);
+                ok = ok && dense_wait(&sh.mail_empty[p1], (((i + 1) / kProd) & 1u) ^ 1u, abort);
+                if (ok) {
+                    sh.mail[p1] = next;
+                    mbar_arrive(&sh.mail_full[p1]);
+                }
             }
-            if (pending[sl]) {                        // the consumers are done with this slot
-                nbar_sync(kBarEmpty + sl, S_THREADS);
-                pending[sl] = false;
+            ok = __all_sync(FULL, ok);
+            if (!ok) break;
+            if (block == kItemEnd) {
+                open();
+                if (ok) commit(1, kItemEnd);
+                break;
             }
-            nbar_sync(kBarProd, S_PROD);
-            const int ns = s_ns;
-            // 2. the walk: W[slot][survivor][pixel slot]
-            float(*Wt)[S_PIX] = s_W[sl];
-            for (int sv = 0; sv < ns; ++sv) {
-                const int j = s_surv[sv];
-                float w = 0.f;
-                if (!done) {
-                    const PixelTerm ptm = eval_half_q(ux, uy, s_m[j], s_c[j]);
-                    const float a = ptm.half_q > s_h[j] ? 0.f : eval_alpha(s_a[j], ptm.half_q, alpha_max);
-                    if (a >= alpha_min) {
-                        const float Tt = T * (1.0f - a);
-                        if (T_min > 0.f && Tt < T_min) {
-                            done = true;
-                        } else {
-                            w = T * a;
-                            T = Tt;
-                            ++n_blend;
-                        }
+            const BlockPos b = dense_block(block, tile_w, tiles_x);
+            const int px = b.x0 + (lane & 7), py = b.y0 + 2 * (lane >> 3);
+            const bool in0 = px < W && py < H, in1 = px < W && py + 1 < H;
+            // T over all members (below T_min for good once a pixel has stopped),
+            // and over the blended ones
+            float T0 = 1.0f, T1 = 1.0f, B0 = 1.0f, B1 = 1.0f;
+            uint32_t n_blend = 0;
+            auto visit = [&](int js, const float (&a)[4][2]) -> bool {
+                float2 w[4];
+                unsigned any[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const float t0 = __fmul_rn(T0, __fsub_rn(1.0f, a[u][0])), t1 = __fmul_rn(T1, __fsub_rn(1.0f, a[u][1]));
+                    const bool b0 = in0 && a[u][0] > 0.0f && !(t0 < T_min), b1 = in1 && a[u][1] > 0.0f && !(t1 < T_min);
+                    w[u] = make_float2(b0 ? __fmul_rn(T0, a[u][0]) : 0.0f, b1 ? __fmul_rn(T1, a[u][1]) : 0.0f);
+                    n_blend += uint32_t(b0) + uint32_t(b1);
+                    T0 = t0;
+                    T1 = t1;
+                    B0 = b0 ? t0 : B0;
+                    B1 = b1 ? t1 : B1;
+                    any[u] = __ballot_sync(FULL, w[u].x != 0.0f || w[u].y != 0.0f);
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (any[u] == 0u) continue;
+                    open();
+                    if (!ok) return false;
+                    DenseSlot &S = sh.slot[p][sc % kSlots];
+                    // lanes 4 g .. 4 g + 3 hold the 8 pixels of group g
+                    reinterpret_cast<float2 *>(S.w[e])[lane] = w[u];
+                    if (lane == 0) S.gid[e] = st.g[js + u];
+                    if (lane < 8 && ((any[u] >> (4 * lane)) & 15u)) gmask |= 1u << e;
+                    if (++e == kEnt) commit(0, block);
+                }
+                return !__all_sync(FULL, (T0 < T_min || !in0) && (T1 < T_min || !in1));
+            };
+            walk_block<false, 2>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[b.tile], W, H, b.x0, b.y0,
+                              alpha_min, alpha_max, st, visit);
+            __syncwarp();
+            if (ok) open();
+            if (!ok) break;
+            commit(1, block);
+            if (T_final) {
+                if (in0) T_final[int64_t(py) * W + px] = B0;
+                if (in1) T_final[int64_t(py + 1) * W + px] = B1;
+            }
+            if (stats && n_blend) atomicAdd(&stats[0], (unsigned long long)n_blend);
+        }
+    } else {
+        // ------------------------------------------------------ loader
+        uint32_t rc = 0;                   // row slots filled
+        uint32_t sc[kProd] = {};           // slots taken per producer
+        bool ok = true, end = false;
+        while (ok && !end) {
+#pragma unroll
+            for (int p = 0; p < kProd; ++p) {
+                for (bool last = false; ok && !end && !last;) {
+                    const uint32_t s = sc[p] % kSlots, r = rc % kRows;
+                    ok = __all_sync(FULL, dense_wait(&sh.w_full[p][s], (sc[p] / kSlots) & 1u, abort));
+                    if (ok) ok = __all_sync(FULL, dense_wait(&sh.r_empty[r], ((rc / kRows) & 1u) ^ 1u, abort));
+                    if (!ok) break;
+                    ++sc[p];
+                    ++rc;
+                    const DenseSlot &S = sh.slot[p][s];
+                    DenseRow &R = sh.row[r];
+                    const int n = S.n;
+                    last = S.last != 0;
+                    end = S.block == kItemEnd;
+                    if (lane == 0) {
+                        R.slot = p * kSlots + int(s);
+                        R.n = n;
+                        R.last = S.last;
+                        R.block = S.block;
                     }
+                    const uint32_t gid = lane < n ? S.gid[lane] : 0u;
+                    if (DT == QR_FP8E4M3 && lane < n) R.scale[lane] = fscale[gid];
+                    __syncwarp();
+                    if (lane == 0) tma_expect_tx(&sh.r_full[r], uint32_t(n) * ROW);
+                    __syncwarp();
+                    if (lane < n)
+                        bulk_row(s_rows + (size_t(r) * kEnt + lane) * ROW, feat + size_t(gid) * ROW, ROW, &sh.r_full[r]);
                 }
-                Wt[sv][pt] = w;
             }
-            nbar_sync(kBarProd, S_PROD);
-            // 3. survivors with a nonzero weight, in list order, and their ids
-            // (producer warp 0)
-            if (pw == 0) {
-                bool used = false;
-                if (lane < ns) {
-                    const float4 *wr = reinterpret_cast<const float4 *>(Wt[lane]);
-#pragma unroll
-                    for (int q = 0; q < S_PIX / 4; ++q) {
-                        const float4 t = wr[q];
-                        used |= (t.x != 0.f) | (t.y != 0.f) | (t.z != 0.f) | (t.w != 0.f);
-                    }
-                }
-                const unsigned bal = __ballot_sync(FULL, used);
-                if (used) {
-                    const int u = __popc(bal & ((1u << lane) - 1u));
-                    s_used[sl][u] = lane;
-                    s_kg[sl][u] = s_g[s_surv[lane]];
-                }
-                if (lane == 0) s_nu[sl] = __popc(bal);
-            }
-            nbar_arrive(kBarFull + sl, S_THREADS);
-            pending[sl] = true;
-            sl ^= 1;
         }
-        // the end marker, then wait until every produced slot has been read
-        if (pending[sl]) {
-            nbar_sync(kBarEmpty + sl, S_THREADS);
-            pending[sl] = false;
-        }
-        if (pt == 0) s_nu[sl] = -1;
-        nbar_arrive(kBarFull + sl, S_THREADS);
-        sl ^= 1;
-        if (pending[sl]) nbar_sync(kBarEmpty + sl, S_THREADS);
-        if (T_final && inside) T_final[int64_t(py) * W + px] = T;
-        if (stats) atomicAdd(&stats[0], n_blend);
-        return;
+        // after a timeout: the copies issued last land before the CTA exits
+        if (!ok)
+            for (uint32_t i = rc > kRows ? rc - kRows : 0; i < rc; ++i)
+                tma_mbar_wait(&sh.r_full[i % kRows], (i / kRows) & 1u, kDenseSpin);
     }
-
-    // -------------------------------------------------------------- consumers
-    // thread t of a group's warp pair owns the channel pairs 2 t + 128 k
-    // (k < CH / 2), so a warp's shared-memory reads and global writes are
-    // consecutive 8-byte pairs
-    const int g = warp >> 1;
-    const int c0 = (tid & 63) * 2;
-    float acc[8][CH];
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int c = 0; c < CH; ++c) acc[i][c] = 0.f;
-    unsigned long long n_exec = 0;
-    for (int sl = 0;; sl ^= 1) {
-        nbar_sync(kBarFull + sl, S_THREADS);
-        const int nu = s_nu[sl];
-        if (nu < 0) break;
-        // the kept rows into F (the consumers are all past the previous
-        // batch: the FULL barrier counts every one of them)
-        const int vpr = C / CPV;                       // 16-byte vectors per row
-        for (int i = tid; i < nu * vpr; i += S_CONS) {
-            const int u = i / vpr, v = i - u * vpr;
-            const uint32_t gid = s_kg[sl][u];
-            const unsigned char *src = feat + size_t(gid) * row_bytes + size_t(v) * 16;
-            if constexpr (DT == QR_F32) {
-                cp_async16(s_F + size_t(u) * C + v * CPV, src);
-            } else {
-                const uint4 x = __ldg(reinterpret_cast<const uint4 *>(src));
-                float tmp[CPV];
-                widen16<DT>(x, DT == QR_FP8E4M3 ? fscale[gid] : 1.f, tmp);
-#pragma unroll
-                for (int q = 0; q < CPV; q += 4)
-                    *reinterpret_cast<float4 *>(s_F + size_t(u) * C + v * CPV + q) =
-                        make_float4(tmp[q], tmp[q + 1], tmp[q + 2], tmp[q + 3]);
-            }
-        }
-        if constexpr (DT == QR_F32) asm volatile("cp.async.wait_all;" ::: "memory");
-        nbar_sync(kBarCons, S_CONS);
-        for (int u = 0; u < nu; ++u) {
-            const int sv = s_used[sl][u];
-            const float4 *wr = reinterpret_cast<const float4 *>(&s_W[sl][sv][g * 8]);
-            const float4 wa = wr[0], wb = wr[1];
-            const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-            const bool any = (wa.x != 0.f) | (wa.y != 0.f) | (wa.z != 0.f) | (wa.w != 0.f) |
-                             (wb.x != 0.f) | (wb.y != 0.f) | (wb.z != 0.f) | (wb.w != 0.f);
-            if (!any) continue;
-            ++n_exec;
-            const float *Fr = s_F + size_t(u) * C;
-            float fv[CH];
-#pragma unroll
-            for (int k = 0; k < CH / 2; ++k) {
-                const float2 t = *reinterpret_cast<const float2 *>(Fr + 128 * k + c0);
-                fv[2 * k] = t.x;
-                fv[2 * k + 1] = t.y;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-#pragma unroll
-                for (int c = 0; c < CH; ++c) acc[i][c] = fmaf(wv[i], fv[c], acc[i][c]);
-        }
-        nbar_arrive(kBarEmpty + sl, S_THREADS);
-    }
-    // write the sub-tile
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        int x, y;
-        slot_xy(g * 8 + i, x, y);
-        if (x < W && y < H) {
-            float *o = out + (int64_t(y) * W + x) * C + c0;
-#pragma unroll
-            for (int k = 0; k < CH / 2; ++k)
-                *reinterpret_cast<float2 *>(o + 128 * k) = make_float2(acc[i][2 * k], acc[i][2 * k + 1]);
-        }
-    }
-    // executed FMAs (a warp's entries x 32 lanes x 8 pixels x CH)
-    if (stats && lane == 0) atomicAdd(&stats[1], n_exec * 32ull * 8ull * CH);
+    __syncthreads();
+    if (threadIdx.x == 0 && *abort) atomicExch(&counters[CNT_STATUS], uint32_t(QR_ERR_DEVICE_TIMEOUT));
 }
 
-template <int DT, int CH>
-cudaError_t run_sub(const qr_frame &f, const void *feat, const float *scale, int C, float *out,
-                    float *T_final, unsigned long long *stats, cudaStream_t s) {
-    const size_t dyn = size_t(S_BATCH) * C * 4;
-    cudaError_t e = cudaFuncSetAttribute(dense_sub_kernel<DT, CH>,
+template <int DT, int QPT, int WPG>
+cudaError_t run_block(const qr_frame &f, const void *feat, const float *scale, float *out,
+                      float *T_final, unsigned long long *stats, cudaStream_t s) {
+    constexpr size_t dyn = kDenseShared + size_t(kRows) * kEnt * 32 * WPG * QPT * Quad<DT>::B;
+    static_assert(dyn <= 227 * 1024, "shared memory");
+    cudaError_t e = cudaFuncSetAttribute(dense_block_kernel<DT, QPT, WPG>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
     if (e != cudaSuccess) return e;
-    dense_sub_kernel<DT, CH><<<unsigned(num_tiles(f)) * 4, S_THREADS, dyn, s>>>(
+    dense_block_kernel<DT, QPT, WPG><<<unsigned(num_tiles(f)) * 4, dense_threads<WPG>(), dyn, s>>>(
         slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C), slot<float>(f, S_REC_A),
         slot<float>(f, S_REC_H), slot<uint32_t>(f, S_IGID), slot<uint2>(f, S_RANGES),
-        static_cast<const unsigned char *>(feat), scale, C, f.camera.width, f.camera.height,
+        static_cast<const unsigned char *>(feat), scale, f.camera.width, f.camera.height,
         f.params.tile_w, f.tiles_x, f.params.alpha_min, f.params.alpha_max, f.params.T_min, out,
-        T_final, stats);
+        T_final, stats, slot<uint32_t>(f, S_COUNTERS));
     count_launch();
     return cudaGetLastError();
 }
@@ -539,10 +608,10 @@ template <int DT>
 cudaError_t dispatch(const qr_frame &f, const void *feat, const float *scale, int C, float *out,
                      float *T_final, unsigned long long *stats, cudaStream_t s) {
     constexpr int cpv = Cpv<DT>::v;
-    // wide rows: the sub-tile kernel (one walk per pixel, culled and skipped entries)
-    if (C == 512) return run_sub<DT, 8>(f, feat, scale, C, out, T_final, stats, s);
-    if (C == 256) return run_sub<DT, 4>(f, feat, scale, C, out, T_final, stats, s);
-    if (C == 128 && cpv <= 8) return run_sub<DT, 2>(f, feat, scale, C, out, T_final, stats, s);
+    // wide rows: one walk per pixel, culled and skipped entries
+    if (C == 512) return run_block<DT, 2, 2>(f, feat, scale, out, T_final, stats, s);
+    if (C == 256) return run_block<DT, 1, 2>(f, feat, scale, out, T_final, stats, s);
+    if (C == 128 && cpv <= 8) return run_block<DT, 1, 1>(f, feat, scale, out, T_final, stats, s);
     if (C % 64 == 0) return run<DT, 64, 8, 8>(f, feat, scale, C, out, T_final, s);
     if (C % 32 == 0) return run<DT, 32, 8, 4>(f, feat, scale, C, out, T_final, s);
     if (C % 16 == 0) return run<DT, 16, 4, 4>(f, feat, scale, C, out, T_final, s);
