@@ -221,6 +221,33 @@ def test_tile_sort_size_classes(n, lo, hi):
                   label=f"slab {n}")
 
 
+@pytest.mark.parametrize("n", [1, 2, 256, 300, 1025, 2048, 2049, 5000, 9000])
+@pytest.mark.parametrize("depths", ["equal", "few", "narrow", "clusters"])
+def test_tile_sort_equal_and_narrow_depths(n, depths):
+    """Buckets whose 32-bit sort keys tie: one depth, a few, a range of a few
+    ulps beside a far Gaussian, clusters.  The lists are in (depth, id) order."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, _ = _slab_scene(n)
+    rng = np.random.default_rng(n)
+    z = {"equal": np.zeros(n), "few": rng.integers(0, 7, n) * 0.05, "narrow": rng.integers(0, 40, n) * 2.0 ** -21,
+         "clusters": rng.integers(0, 5, n) * 0.1 + rng.normal(0, 1e-5, n)}[depths]
+    if depths == "narrow" and n > 2:
+        z[n // 2] = -50.0
+    g.mean[:, 2] = z
+    fr = H.run_gpu(g, None, scenes.tiny_camera(48, 48), K=8, dense=False)["frame"]
+    v = q.qr_frame_view_get(fr)
+    tiles = fr.frame.tiles_x * fr.frame.tiles_y
+    rngs = _device_copy(v.tile_range, 2 * tiles, torch.int32).cpu().numpy().reshape(tiles, 2)
+    gkey = _device_copy(v.depth_key, n, torch.int32).cpu().numpy().view(np.uint32)
+    gids = _device_copy(v.isect_gid, int(rngs[-1, 1]), torch.int32).cpu().numpy()
+    assert (rngs[:, 1] - rngs[:, 0]).max() >= 0.9 * n - 1
+    for a, b in rngs:
+        order = np.lexsort((gids[a:b], gkey.view(np.float32)[gids[a:b]]))
+        np.testing.assert_array_equal(order, np.arange(b - a))
+        assert len(set(gids[a:b].tolist())) == b - a
+
+
 @pytest.mark.parametrize("C", [16, 64, 512])
 def test_blend_stage_matches_definition(C):
     import torch
@@ -272,6 +299,28 @@ def test_dense_without_early_stop():
     gpu = H.run_gpu(g, f, cam, K=8, params_kw={"T_min": 0.0})
     pr, pix, ref = H.run_oracle(g, f, cam, 8, T_min=0.0)
     H.check_frame(gpu, ref, pix, cam.width, f, FEAT_TOL, DENSE_TOL, label="T_min=0")
+
+
+@pytest.mark.parametrize("C,T_min,size", [(128, 0.0, (48, 48)), (256, 1e-4, (41, 23)), (512, 0.0, (17, 9))])
+def test_dense_long_lists(C, T_min, size):
+    """Blocks that keep hundreds of entries (every ring of the block kernel
+    wraps around), images smaller than a tile and with cut blocks."""
+    rng = np.random.default_rng(11)
+    n = 2000
+    mean = np.stack([rng.uniform(-0.2, 0.2, n), rng.uniform(-0.2, 0.2, n),
+                     rng.uniform(-1.5, 1.5, n)], 1).astype(np.float32)
+    g = scenes.Gaussians(mean, np.full((n, 3), -2.0, np.float32),
+                         np.tile(np.array([1, 0, 0, 0], np.float32), (n, 1)),
+                         np.full(n, 0.02, np.float32))
+    f = rng.normal(size=(n, C)).astype(np.float32)
+    cam = scenes.tiny_camera(*size)
+    gpu = H.run_gpu(g, f, cam, K=8, dense=True, params_kw={"T_min": T_min})
+    pr, pix, ref = H.run_oracle(g, f, cam, 8, T_min=float(np.float32(T_min)))
+    assert ref.n_dense.max() > 300
+    ok = (ref.tie & compare.DENSE_TIE_BITS) == 0
+    err = compare.feature_error(np.asarray(gpu["dense"]), ref.out_dense, ref.scale_dense)[ok]
+    # every factor of T and every sum rounds once: 2^-23 per entry of the longest walk
+    assert err.max() <= DENSE_TOL + 2.0 ** -23 * ref.n_dense.max(), err.max()
 
 
 def test_indoor_full_size_sampled():
