@@ -9,8 +9,8 @@
 // tiles its support
 // {u : alpha exp(-q(u)/2) >= alpha_min}, q = (u-mu')^T A (u-mu'), can reach.
 //
-// GB300 design: one kernel, one CTA per 1024 consecutive ids.  Stage A (a
-// thread per Gaussian, four coalesced passes) applies a cheap FP32 bound on
+// GB300 design: one kernel, one CTA per 256 to 1024 consecutive ids.  Stage A (a
+// thread per Gaussian, coalesced passes) applies a cheap FP32 bound on
 // the footprint and writes the culled records; the survivors (a tenth of an
 // indoor scene) are compacted in shared memory and the CTA's threads run
 // stage B on them: the exact projection in compensated double-FP32
@@ -26,8 +26,14 @@
 namespace qr {
 namespace {
 
-constexpr int kThreads = kProjectThreads;
-constexpr int kProjPer = 4;   // Gaussians per thread in the cull stage: 4 id blocks per CTA
+constexpr int kBlk = kProjectThreads;   // ids per counter block
+// Ids per CTA, by the number of Gaussians: few Gaussians take small CTAs, so
+// that a CTA's threads do not project several survivors in turn while SMs
+// stand idle; many take large ones, whose compaction fills warps where most
+// are culled.  Measured with 256 / 512 / 1024 ids (us, VGA): 10k object 13 /
+// 19 / 33, 150k object 23 / 25 / 34, 150k room 15 / 15 / 19; 300k room 21 / 17 /
+// 20, object 40 / 40 / 45; 500k room 33 / 27 / 24, object 70 / 63 / 72.
+constexpr int64_t kIds256 = 152 * 1024, kIds512 = 3 * kIds256;
 
 struct CamArgs {
     float R[9], t[3], fx, fy, cx, cy, znear;
@@ -208,14 +214,15 @@ __device__ __forceinline__ void project_one(int64_t gi, int blk, const float *__
     atomicAdd(&dcopy[(ty1 + 1) * stride + tx1 + 1], 1);
 }
 
-// One CTA per kProjPer x 256 consecutive ids (kProjPer id blocks of 256):
-// stage A culls them (coalesced, kProjPer passes) and writes the culled
-// records; the survivors are compacted in shared memory (one shared atomic
+// One CTA of NT threads per IDS consecutive ids (a whole number of id blocks
+// of 256): stage A culls them (coalesced) and writes the culled records; the
+// survivors are compacted in shared memory (one shared atomic
 // per warp) and the CTA's threads run stage B on them.  The per-256-id
 // counts are summed in shared memory and written (not accumulated) for the
 // CTA's own id blocks, so only the difference array needs clearing (a memset
 // before the launch).
-__global__ void __launch_bounds__(kThreads)
+template <int NT, int IDS>
+__global__ void __launch_bounds__(NT)
 project_kernel(int64_t n, const float *__restrict__ mean, const float *__restrict__ log_scale,
                const float *__restrict__ quat, const float *__restrict__ opacity, CamArgs cam,
                float dilation, float alpha_min, int tile_w, int tile_h,
@@ -225,21 +232,23 @@ project_kernel(int64_t n, const float *__restrict__ mean, const float *__restric
                uint32_t *__restrict__ tile_sum, int tiles_x, int tiles_y, int *__restrict__ diff,
                uint32_t *__restrict__ counters) {
     pdl_wait();   // the predecessor's outputs are complete and visible
-    __shared__ uint32_t s_cand[kThreads * kProjPer];
+    constexpr int NB = IDS / kBlk;
+    static_assert(IDS % kBlk == 0 && IDS % NT == 0 && NB <= NT, "whole id blocks");
+    __shared__ uint32_t s_cand[IDS];
     __shared__ uint32_t s_n;
-    __shared__ uint32_t s_vis[kProjPer], s_ts[kProjPer];
-    if (threadIdx.x < kProjPer) {
+    __shared__ uint32_t s_vis[NB], s_ts[NB];
+    if (threadIdx.x < NB) {
         s_vis[threadIdx.x] = 0u;
         s_ts[threadIdx.x] = 0u;
     }
     if (threadIdx.x == 0) s_n = 0u;
     if (blockIdx.x == 0 && threadIdx.x == 0) counters[CNT_N] = uint32_t(n);
     __syncthreads();
-    const int64_t g0 = int64_t(blockIdx.x) * (kThreads * kProjPer);
+    const int64_t g0 = int64_t(blockIdx.x) * IDS;
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int k = 0; k < kProjPer; ++k) {
-        const int64_t g = g0 + k * kThreads + threadIdx.x;
+    for (int k = 0; k < IDS / NT; ++k) {
+        const int64_t g = g0 + k * NT + threadIdx.x;
         bool pass = false;
         if (g < n) {
             pass = cull_pass(g, mean, log_scale, opacity, cam, dilation, alpha_min);
@@ -254,16 +263,16 @@ project_kernel(int64_t n, const float *__restrict__ mean, const float *__restric
     __syncthreads();
     const uint32_t nc = s_n;
     int *dcopy = diff + size_t(blockIdx.x % kDiffCopies) * size_t(tiles_x + 1) * size_t(tiles_y + 1);
-    for (uint32_t i = threadIdx.x; i < nc; i += kThreads) {
+    for (uint32_t i = threadIdx.x; i < nc; i += NT) {
         const uint32_t loc = s_cand[i];
         project_one(g0 + loc, int(loc >> 8), mean, log_scale, quat, opacity, cam, dilation,
                     alpha_min, tile_w, tile_h, rec_m, rec_w, rec_a, rec_h, rect, tcount, dkey,
                     s_vis, s_ts, tiles_x, dcopy);
     }
     __syncthreads();
-    if (threadIdx.x < kProjPer) {
-        const int64_t blk = g0 / kThreads + threadIdx.x;
-        if (blk * kThreads < n) {
+    if (threadIdx.x < NB) {
+        const int64_t blk = g0 / kBlk + threadIdx.x;
+        if (blk * kBlk < n) {
             vis_count[blk] = s_vis[threadIdx.x];
             tile_sum[blk] = s_ts[threadIdx.x];
         }
@@ -287,14 +296,18 @@ cudaError_t launch_project(const qr_frame &f, const float *mean, const float *lo
     for (int i = 0; i < 3; ++i) cam.t[i] = f.camera.t[i];
     cam.fx = f.camera.fx; cam.fy = f.camera.fy; cam.cx = f.camera.cx; cam.cy = f.camera.cy;
     cam.znear = f.camera.near_plane; cam.W = f.camera.width; cam.H = f.camera.height;
-    const unsigned blocks = unsigned((n + kThreads * kProjPer - 1) / (kThreads * kProjPer));
-    e = pdl_launch(project_kernel, dim3(blocks), dim3(kThreads), 0, s, n, mean, log_scale, quat,
-                   opacity, cam, f.params.dilation, f.params.alpha_min, f.params.tile_w,
-                   f.params.tile_h, slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C),
-                   slot<float>(f, S_REC_A), slot<float>(f, S_REC_H), slot<uint2>(f, S_RECT),
-                   slot<uint32_t>(f, S_TCOUNT), slot<uint32_t>(f, S_GKEY),
-                   slot<uint32_t>(f, S_VISCNT), slot<uint32_t>(f, S_BSUM), f.tiles_x, f.tiles_y,
-                   slot<int>(f, S_DIFF), counters);
+    auto go = [&](auto kern, int nt, int ids) -> cudaError_t {
+        return pdl_launch(kern, dim3(unsigned((n + ids - 1) / ids)), dim3(nt), 0, s, n, mean, log_scale,
+                          quat, opacity, cam, f.params.dilation, f.params.alpha_min, f.params.tile_w,
+                          f.params.tile_h, slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C),
+                          slot<float>(f, S_REC_A), slot<float>(f, S_REC_H), slot<uint2>(f, S_RECT),
+                          slot<uint32_t>(f, S_TCOUNT), slot<uint32_t>(f, S_GKEY),
+                          slot<uint32_t>(f, S_VISCNT), slot<uint32_t>(f, S_BSUM), f.tiles_x, f.tiles_y,
+                          slot<int>(f, S_DIFF), counters);
+    };
+    if (n <= kIds256) e = go(project_kernel<256, 256>, 256, 256);
+    else if (n <= kIds512) e = go(project_kernel<256, 512>, 256, 512);
+    else e = go(project_kernel<256, 1024>, 256, 1024);
     count_launch(1);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
