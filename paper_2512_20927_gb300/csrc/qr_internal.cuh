@@ -337,6 +337,10 @@ template <typename KT>
 __device__ __forceinline__ KT key_pick(KT a, KT b, bool take_min) {
     return ((a < b) == take_min) ? a : b;
 }
+template <>
+__device__ __forceinline__ uint32_t key_pick(uint32_t a, uint32_t b, bool take_min) {
+    return take_min ? min(a, b) : max(a, b);
+}
 
 // Position i = base + e of a thread's keys differs from base only below bit
 // log2(E) (base is a multiple of E), so for strides j >= E and blocks k > j

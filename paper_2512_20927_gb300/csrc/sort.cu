@@ -284,19 +284,111 @@ expand_scatter(const uint32_t *__restrict__ koff, const uint32_t *__restrict__ k
 }
 
 // ------------------------------------------------------------------ per-tile sort
-// A bucket of up to NTH*E keys, loaded E per thread in blocked order and
-// padded with ~0, sorted by the register bitonic network, ids written out.
-template <int E, int NTH = T>
+// Buckets are sorted by 32-bit keys first: the leading bits of (depth - the
+// bucket's smallest depth) that 32 - IB bits hold, and the key's position in
+// the bucket (IB bits, below 2^IB keys).  The order of the 64-bit keys is
+// then right but for keys whose leading bits agree (about n^2 / 2^(33 - IB)
+// pairs of evenly spread depths), which exchange places with their
+// neighbours until every pair is in order; buckets that need more than
+// kFixRounds of that (many equal depths) are sorted again by the 64-bit keys.
+// The result is the order of the 64-bit keys in every case.  A 32-bit
+// compare-exchange takes one shuffle and three instructions, a 64-bit one two
+// and seven, and a shared-memory key half the bandwidth.
+// Projected frames (sort stage, 64-bit network and merges -> now): 1M room at
+// 1296 x 968 157 -> 135 us, object VGA with 710 buckets of 2k-5k keys 162 ->
+// 150 us, room VGA 38 -> 37 us, 2,000 Gaussians 14.3 -> 15.4 us (the two
+// barriers of the depth range and the check).
+constexpr int kFixRounds = 16;
+
+// CTA-wide smallest value and bit length of the spread of a thread's (lo, hi).
+template <int NTH>
+__device__ __forceinline__ void depth_span(uint32_t lo, uint32_t hi, uint32_t *s_w, uint32_t &smallest,
+                                           int &bits) {
+    lo = __reduce_min_sync(0xffffffffu, lo);
+    hi = __reduce_max_sync(0xffffffffu, hi);
+    if ((threadIdx.x & 31) == 0) {
+        s_w[threadIdx.x >> 5] = lo;
+        s_w[32 + (threadIdx.x >> 5)] = hi;
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    lo = __reduce_min_sync(0xffffffffu, lane < NTH / 32 ? s_w[lane] : 0xFFFFFFFFu);
+    hi = __reduce_max_sync(0xffffffffu, lane < NTH / 32 ? s_w[32 + lane] : 0u);
+    smallest = lo;
+    bits = hi > lo ? 32 - __clz(hi - lo) : 0;
+}
+
+// Neighbours of the n keys in s exchange places until all are in order; false
+// if kFixRounds did not suffice.  Ends with a barrier.
+template <int NTH>
+__device__ __forceinline__ bool fix_order(unsigned long long *s, int n) {
+    for (int r = 0;; ++r) {
+        bool bad = false;
+        for (int i = threadIdx.x; i + 1 < n; i += NTH) bad |= s[i] > s[i + 1];
+        if (!__syncthreads_or(bad)) return true;
+        if (r == kFixRounds) return false;
+        for (int odd = 0; odd < 2; ++odd) {
+            for (int i = 2 * int(threadIdx.x) + odd; i + 1 < n; i += 2 * NTH) {
+                const unsigned long long x = s[i], y = s[i + 1];
+                if (x > y) {
+                    s[i] = y;
+                    s[i + 1] = x;
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+
+// A bucket of up to T * E keys: E per thread in blocked order, sorted by the
+// register bitonic network, ids written out.  s: T E keys, x: T E words.
+template <int E>
 __device__ void sort_registers(const unsigned long long *__restrict__ src, int n,
-                               unsigned long long *s, uint32_t *__restrict__ dst) {
+                               unsigned long long *s, uint32_t *x, uint32_t *s_w,
+                               uint32_t *__restrict__ dst) {
+    constexpr int IB = 8 + (E == 8 ? 3 : E == 4 ? 2 : E == 2 ? 1 : 0);   // log2(T E)
     const int base = threadIdx.x * E;
-    unsigned long long v[E];
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = base + e < n ? src[base + e] : ~0ull;
-    bitonic_regs<E, NTH, unsigned long long>(v, s);
+    for (int e = 0; e < E; ++e) {
+        const int i = int(threadIdx.x) + e * T;
+        if (i < n) {
+            const unsigned long long k = src[i];
+            s[i] = k;
+            lo = min(lo, uint32_t(k >> 32));
+            hi = max(hi, uint32_t(k >> 32));
+        }
+    }
+    uint32_t smallest;
+    int bits;
+    depth_span<T>(lo, hi, s_w, smallest, bits);   // its barrier also publishes s
+    const int sh = max(0, bits - (32 - IB));
+    uint32_t v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e)
-        if (base + e < n) dst[base + e] = uint32_t(v[e]);
+        v[e] = base + e < n ? (((uint32_t(s[base + e] >> 32) - smallest) >> sh) << IB) | uint32_t(base + e)
+                            : 0xFFFFFFFFu;
+    bitonic_regs<E, T, uint32_t>(v, x);
+    unsigned long long k[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[v[e] & ((1u << IB) - 1u)] : ~0ull;
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (base + e < n) s[base + e] = k[e];
+    __syncthreads();
+    if (!fix_order<T>(s, n)) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[base + e] : ~0ull;
+        __syncthreads();
+        bitonic_regs<E, T, unsigned long long>(k, s);
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            if (base + e < n) s[base + e] = k[e];
+        __syncthreads();
+    }
+    for (int i = threadIdx.x; i < n; i += T) dst[i] = uint32_t(s[i]);
 }
 
 // Merge sorted A[0,na) and B[0,nb) into C with the whole CTA of NT threads
@@ -333,6 +425,8 @@ tile_sort(const uint2 *__restrict__ ranges, unsigned long long *__restrict__ key
           uint32_t *__restrict__ igid, uint32_t *__restrict__ big, uint32_t *__restrict__ counters) {
     pdl_wait();   // the predecessor's outputs are complete and visible
     __shared__ unsigned long long s_k[8 * T];
+    __shared__ uint32_t s_x[8 * T];
+    __shared__ uint32_t s_w[64];
     const uint2 r = ranges[blockIdx.x];
     const int n = int(r.y - r.x);
     if (n > 8 * T) {
@@ -342,12 +436,12 @@ tile_sort(const uint2 *__restrict__ ranges, unsigned long long *__restrict__ key
     if (n == 0) return;
     unsigned long long *src = keys + r.x;
     if (n <= 2 * T) {
-        if (n <= T) sort_registers<1>(src, n, s_k, igid + r.x);
-        else sort_registers<2>(src, n, s_k, igid + r.x);
+        if (n <= T) sort_registers<1>(src, n, s_k, s_x, s_w, igid + r.x);
+        else sort_registers<2>(src, n, s_k, s_x, s_w, igid + r.x);
         return;
     }
-    if (n <= 4 * T) sort_registers<4>(src, n, s_k, igid + r.x);
-    else sort_registers<8>(src, n, s_k, igid + r.x);
+    if (n <= 4 * T) sort_registers<4>(src, n, s_k, s_x, s_w, igid + r.x);
+    else sort_registers<8>(src, n, s_k, s_x, s_w, igid + r.x);
 }
 
 // ------------------------------------------------------------------ big buckets
@@ -429,27 +523,136 @@ __device__ unsigned long long *sort_smem(unsigned long long *s, unsigned long lo
     return s;
 }
 
-__device__ __forceinline__ unsigned long long *sort_smem_any(unsigned long long *s,
-                                                             unsigned long long *t, int n) {
-    if (n <= TB * 2) return sort_smem<2>(s, t, n);
-    if (n <= TB * 4) return sort_smem<4>(s, t, n);
-    return sort_smem<8>(s, t, n);
+// 32-bit keys: eight in registers, and the same merge rounds (a pad word after
+// every 32 keys).  A thread holds the two candidates in registers, so each
+// output costs one read.
+__device__ __forceinline__ void cx(uint32_t &a, uint32_t &b) {
+    const uint32_t lo = min(a, b), hi = max(a, b);
+    a = lo;
+    b = hi;
+}
+__device__ __forceinline__ void sort8(uint32_t (&v)[8]) {
+    cx(v[0], v[1]); cx(v[2], v[3]); cx(v[4], v[5]); cx(v[6], v[7]);
+    cx(v[0], v[2]); cx(v[1], v[3]); cx(v[4], v[6]); cx(v[5], v[7]);
+    cx(v[1], v[2]); cx(v[5], v[6]);
+    cx(v[0], v[4]); cx(v[1], v[5]); cx(v[2], v[6]); cx(v[3], v[7]);
+    cx(v[2], v[4]); cx(v[3], v[5]);
+    cx(v[1], v[2]); cx(v[3], v[4]); cx(v[5], v[6]);
+}
+__device__ __forceinline__ int pad32(int i) { return i + (i >> 5); }
+
+template <int E>
+__device__ uint32_t *merge_words(uint32_t *s, uint32_t *t, int n) {
+    const int d0 = int(threadIdx.x) * E;
+    const int m = max(0, min(E, n - d0));
+    for (int L = 8; L < n; L <<= 1) {
+        if (m > 0) {
+            const int ps = d0 & ~(2 * L - 1);
+            const int na = min(L, n - ps);
+            const int nb = max(0, min(L, n - ps - na));
+            const int pb = ps + na;   // run A is keys [ps, pb), run B [pb, pb + nb)
+            const int diag = d0 - ps;
+            int lo = max(0, diag - nb), hi = min(diag, na);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (s[pad32(ps + mid)] < s[pad32(pb + diag - 1 - mid)]) lo = mid + 1; else hi = mid;
+            }
+            int i = ps + lo, j = pb + diag - lo;
+            const int ie = pb, je = pb + nb;
+            uint32_t ka = i < ie ? s[pad32(i)] : 0xFFFFFFFFu, kb = j < je ? s[pad32(j)] : 0xFFFFFFFFu;
+#pragma unroll
+            for (int e = 0; e < E; ++e) {
+                if (e >= m) break;
+                // an exhausted run reads as the largest word (which no other
+                // key of it equals, or it is the last of all)
+                const bool take_a = ka <= kb;
+                t[pad32(d0 + e)] = take_a ? ka : kb;
+                const int next = take_a ? ++i : ++j;
+                const uint32_t k = next < (take_a ? ie : je) ? s[pad32(next)] : 0xFFFFFFFFu;
+                if (take_a) ka = k; else kb = k;
+            }
+        }
+        // as in sort_smem: warp barriers while a round's reads stay in the
+        // warp's own outputs
+        if (4 * L <= 32 * E && 2 * L < n) __syncwarp();
+        else __syncthreads();
+        uint32_t *x = s;
+        s = t;
+        t = x;
+    }
+    return s;
+}
+
+// Sorts the n <= BIG_CAP keys in a (unpadded; a and b hold BIG_SLOTS 64-bit
+// slots each) and returns the buffer with the sorted keys (unpadded).
+template <int E>
+__device__ unsigned long long *sort_big_bucket(unsigned long long *a, unsigned long long *b, int n,
+                                               uint32_t *s_w) {
+    constexpr int IB = 13;   // BIG_CAP positions
+    uint32_t *x = reinterpret_cast<uint32_t *>(b), *y = x + BIG_CAP + BIG_CAP / 32;
+    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    for (int i = threadIdx.x; i < n; i += TB) {
+        const uint32_t d = uint32_t(a[i] >> 32);
+        lo = min(lo, d);
+        hi = max(hi, d);
+    }
+    uint32_t smallest;
+    int bits;
+    depth_span<TB>(lo, hi, s_w, smallest, bits);
+    const int sh = max(0, bits - (32 - IB));
+    for (int r0 = int(threadIdx.x) * 8; r0 < n; r0 += TB * 8) {
+        uint32_t v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            v[e] = r0 + e < n ? (((uint32_t(a[r0 + e] >> 32) - smallest) >> sh) << IB) | uint32_t(r0 + e)
+                              : 0xFFFFFFFFu;
+        sort8(v);
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            if (r0 + e < n) x[pad32(r0 + e)] = v[e];
+    }
+    __syncthreads();
+    const uint32_t *o = merge_words<E>(x, y, n);
+    unsigned long long k[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = int(threadIdx.x) + e * TB;
+        k[e] = i < n ? a[o[pad32(i)] & ((1u << IB) - 1u)] : 0ull;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int i = int(threadIdx.x) + e * TB;
+        if (i < n) b[i] = k[e];
+    }
+    __syncthreads();
+    if (fix_order<TB>(b, n)) return b;
+    for (int i = threadIdx.x; i < n; i += TB) a[pad(i)] = b[i];
+    __syncthreads();
+    unsigned long long *q = sort_smem<E>(a, b, n), *t = q == a ? b : a;
+    for (int i = threadIdx.x; i < n; i += TB) t[i] = q[pad(i)];
+    __syncthreads();
+    return t;
+}
+__device__ __forceinline__ unsigned long long *sort_big_any(unsigned long long *a, unsigned long long *b,
+                                                            int n, uint32_t *s_w) {
+    if (n <= TB * 4) return sort_big_bucket<4>(a, b, n, s_w);
+    return sort_big_bucket<8>(a, b, n, s_w);
 }
 
 // The buckets of more than 8 T keys, listed by tile_sort: persistent CTAs of
 // TB threads (one per SM: 136 KB of shared memory) take them in turn.  Up to
-// BIG_CAP keys are merge-sorted in shared memory (faster here than the
-// register bitonic network over 1024 threads: 232 vs 365 us for the object
-// frame's sort stage); a larger bucket is sorted in BIG_CAP chunks whose
-// sorted runs are merged in global memory by the same CTA (merge path,
-// ping-ponging between the key buffer and the scratch buffer), so no size is
-// refused.
+// BIG_CAP keys are sorted in shared memory; a larger bucket is sorted in
+// BIG_CAP chunks whose sorted runs are merged in global memory by the same
+// CTA (merge path, ping-ponging between the key buffer and the scratch
+// buffer), so no size is refused.
 __global__ void __launch_bounds__(TB, 1)
 tile_sort_big(const uint2 *__restrict__ ranges, unsigned long long *__restrict__ keys,
               unsigned long long *__restrict__ scratch, uint32_t *__restrict__ igid,
               const uint32_t *__restrict__ big, const uint32_t *__restrict__ counters) {
     pdl_wait();   // the predecessor's outputs are complete and visible
-    extern __shared__ unsigned long long s_k[];   // 2 x BIG_SLOTS (padded slots)
+    extern __shared__ unsigned long long s_k[];   // 2 x BIG_SLOTS
+    __shared__ uint32_t s_w[64];
     unsigned long long *s_t = s_k + BIG_SLOTS;
     const uint32_t nbig = counters[CNT_BIG];
     for (uint32_t bi = blockIdx.x; bi < nbig; bi += gridDim.x) {
@@ -457,19 +660,19 @@ tile_sort_big(const uint2 *__restrict__ ranges, unsigned long long *__restrict__
         const int n = int(r.y - r.x);
         unsigned long long *src = keys + r.x;
         if (n <= BIG_CAP) {
-            for (int i = threadIdx.x; i < n; i += TB) s_k[pad(i)] = src[i];
+            for (int i = threadIdx.x; i < n; i += TB) s_k[i] = src[i];
             __syncthreads();
-            const unsigned long long *o = sort_smem_any(s_k, s_t, n);
-            for (int i = threadIdx.x; i < n; i += TB) igid[r.x + i] = uint32_t(o[pad(i)]);
+            const unsigned long long *o = sort_big_any(s_k, s_t, n, s_w);
+            for (int i = threadIdx.x; i < n; i += TB) igid[r.x + i] = uint32_t(o[i]);
             __syncthreads();
             continue;
         }
         for (int c0 = 0; c0 < n; c0 += BIG_CAP) {
             const int m = min(BIG_CAP, n - c0);
-            for (int i = threadIdx.x; i < m; i += TB) s_k[pad(i)] = src[c0 + i];
+            for (int i = threadIdx.x; i < m; i += TB) s_k[i] = src[c0 + i];
             __syncthreads();
-            const unsigned long long *o = sort_smem_any(s_k, s_t, m);
-            for (int i = threadIdx.x; i < m; i += TB) src[c0 + i] = o[pad(i)];
+            const unsigned long long *o = sort_big_any(s_k, s_t, m, s_w);
+            for (int i = threadIdx.x; i < m; i += TB) src[c0 + i] = o[i];
             __syncthreads();
         }
         unsigned long long *a = src, *dst = scratch + r.x;
