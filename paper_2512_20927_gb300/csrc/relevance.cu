@@ -480,7 +480,7 @@ relevance_tma_kernel(const __grid_constant__ CUtensorMap tmap, const uint16_t *_
 //     distinct rows and each row's four pixel weights in shared memory.  Then,
 //     128 channels at a time, it reads each distinct row once (one warp-wide
 //     512-byte load), accumulates the four pixels in FP32 in entry order per
-//     pixel (eight rows in flight), rounds them to BF16 and writes them into
+//     pixel (four rows in flight), rounds them to BF16 and writes them into
 //     a 128-byte-swizzled K-major stage (two 64-channel slices) of a ring
 //     (2 stages: a deeper ring costs L1 capacity the row reads need) -- the
 //     layout the fallback relevance kernel stages.
@@ -491,11 +491,15 @@ relevance_tma_kernel(const __grid_constant__ CUtensorMap tmap, const uint16_t *_
 // share nothing but the ring.  Long waits back off with __nanosleep so the
 // waiting warps leave issue slots to the producers.  Same bounded waits,
 // abort flag and drain as the other kernels.
+// Bound by the producers' issue and row-load latency.  Room VGA, 512 FP32
+// channels, 64 queries: 247 us with eight rows in flight, a branch after each
+// and scalar multiply-adds; 209 us with four, no branches, packed FP32x2 ones
+// (eight rows with packed ones spill: 234 us).
 constexpr int FB_PRODUCERS = 16;
 constexpr int FB_THREADS = (5 + FB_PRODUCERS) * 32;   // 4 epilogue warps, 1 MMA warp, producers
 constexpr int FB_MAX_STAGES = 2;
 constexpr int FB_GPW = 32 / FB_PRODUCERS;             // 2 x 2 groups per producer warp
-constexpr int FB_ROWS = 8;                            // row loads in flight per lane
+constexpr int FB_ROWS = 4;                            // row loads in flight per lane
 constexpr int FB_CHUNK = 128;                        // channels per stage
 constexpr int FB_STAGE_BYTES = 128 * FB_CHUNK * 2;    // 32 KB (two 64-channel BF16 slices)
 
@@ -530,6 +534,13 @@ __device__ __forceinline__ bool lane_wait_sleep(uint64_t *bar, uint32_t parity,
     }
     *abort_flag = 1;
     return false;
+}
+
+// acc += w * (x0, x1), each half rounded like fmaf
+__device__ __forceinline__ void fb_fma2(float2 &acc, float w, float x0, float x1) {
+    asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %2};\n"
+        " mov.b64 xx, {%3, %4};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(w), "f"(x0), "f"(x1));
 }
 
 // 4 channels of a row at channel c, widened to FP32 (the lane's share of a
@@ -667,26 +678,24 @@ blend_relevance_kernel(const unsigned char *__restrict__ feat, const float *__re
                     const int nr = t_n[gi];
                     const int32_t *tid = t_id + gi * 32;
                     const float4 *tw = t_w + gi * 32;
-                    float4 acc[4];
+                    float2 acc[4][2];
 #pragma unroll
-                    for (int mm = 0; mm < 4; ++mm) acc[mm] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    for (int mm = 0; mm < 4; ++mm) acc[mm][0] = acc[mm][1] = make_float2(0.f, 0.f);
                     for (int r0 = 0; r0 < nr; r0 += FB_ROWS) {
                         float4 f[FB_ROWS];
 #pragma unroll
                         for (int u = 0; u < FB_ROWS; ++u)
                             f[u] = r0 + u < nr ? fb_load4<DT>(feat, row_bytes, tid[r0 + u], c)
                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+                        // no branch between the rows (past nr: zeros with weight zero)
 #pragma unroll
                         for (int u = 0; u < FB_ROWS; ++u) {
-                            if (r0 + u >= nr) break;
                             const float4 wg = tw[r0 + u];
                             const float wv[4] = {wg.x, wg.y, wg.z, wg.w};
 #pragma unroll
                             for (int mm = 0; mm < 4; ++mm) {
-                                acc[mm].x = fmaf(wv[mm], f[u].x, acc[mm].x);
-                                acc[mm].y = fmaf(wv[mm], f[u].y, acc[mm].y);
-                                acc[mm].z = fmaf(wv[mm], f[u].z, acc[mm].z);
-                                acc[mm].w = fmaf(wv[mm], f[u].w, acc[mm].w);
+                                fb_fma2(acc[mm][0], wv[mm], f[u].x, f[u].y);
+                                fb_fma2(acc[mm][1], wv[mm], f[u].z, f[u].w);
                             }
                         }
                     }
@@ -695,8 +704,8 @@ blend_relevance_kernel(const unsigned char *__restrict__ feat, const float *__re
 #pragma unroll
                     for (int mm = 0; mm < 4; ++mm) {
                         const int r = fb_row(gi, mm);
-                        const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[mm].x, acc[mm].y);
-                        const __nv_bfloat162 hi = __floats2bfloat162_rn(acc[mm].z, acc[mm].w);
+                        const __nv_bfloat162 lo = __floats2bfloat162_rn(acc[mm][0].x, acc[mm][0].y);
+                        const __nv_bfloat162 hi = __floats2bfloat162_rn(acc[mm][1].x, acc[mm][1].y);
                         uint2 packed;
                         packed.x = *reinterpret_cast<const uint32_t *>(&lo);
                         packed.y = *reinterpret_cast<const uint32_t *>(&hi);
