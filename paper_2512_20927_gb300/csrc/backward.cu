@@ -289,6 +289,169 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
     }
 }
 
+// acc += (x0, x1) * g for both halves
+__device__ __forceinline__ void fma2x(float2 &acc, float x0, float x1, float2 g) {
+    asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %3};\n"
+        " mov.b64 xx, {%4, %5};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(x0), "f"(x1), "f"(g.x), "f"(g.y));
+}
+
+// The same without the loss, for K <= 8 and rows of up to 512 channels, a warp per 2 x 2 pixels:
+// the four pixels' slices of g stay in registers and each distinct row of
+// their entries (8 of 22 in a room) is read and widened once, its four dot
+// products formed in packed FP32x2 instructions and reduced together; the
+// alpha' terms, prefix and suffix sums of the four pixels run side by side,
+// lane m K + j for entry j of pixel m.
+// Bound by instruction issue and the reads of g.  300k room VGA, 512 BF16
+// channels, K = 8: a warp per pixel 277 us, this 173 us (ncu).  With the loss
+// fused it took 410 us (two maps in registers leave 16 warps per SM) where the
+// warp per pixel takes 375.
+template <int DT, int VPL>
+__global__ void __launch_bounds__(T, 2)
+bwd_group(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+          const float *__restrict__ rec_a, const unsigned char *__restrict__ feat,
+          const float *__restrict__ fscale, int C, const int32_t *__restrict__ ids,
+          const float *__restrict__ wts, const uint8_t *__restrict__ cnt,
+          const float *__restrict__ grad_out, int K, int W, int H, float alpha_max,
+          float4 *__restrict__ E) {
+    constexpr int CPV = VecB<DT>::C, ESZ = VecB<DT>::E;
+    constexpr int NP = VPL * CPV / 2;              // channel pairs per lane
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int NW = T / 32;
+    __shared__ int s_id[NW][32];
+    __shared__ float s_dot[NW][32][4];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const size_t row_bytes = size_t(C) * ESZ;
+    const int strips = (W + 15) >> 4;
+    const int x0 = int(blockIdx.x % strips) * 16, y0 = int(blockIdx.x / strips) * 8;
+    const int m = lane / K, j = lane - m * K;
+    // the lane's channels of a row: vectors lane, lane + 32, ... of CPV channels
+    auto load_row = [&](const float *row, float2 (&v)[NP]) {
+#pragma unroll
+        for (int t = 0; t < VPL; ++t)
+#pragma unroll
+            for (int q = 0; q < CPV / 4; ++q) {
+                const float4 a = reinterpret_cast<const float4 *>(row + (lane + 32 * t) * CPV)[q];
+                v[(t * CPV + 4 * q) / 2] = make_float2(a.x, a.y);
+                v[(t * CPV + 4 * q) / 2 + 1] = make_float2(a.z, a.w);
+            }
+    };
+    for (int q = warp; q < 32; q += NW) {
+        const int gx = x0 + 2 * (q & 7), gy = y0 + 2 * (q >> 3);
+        auto pixel = [&](int mm) -> int64_t {
+            const int x = gx + (mm & 1), y = gy + (mm >> 1);
+            return x < W && y < H ? int64_t(y) * W + x : -1;
+        };
+        if (gx >= W || gy >= H) continue;
+        const int64_t p = m < 4 ? pixel(m) : -1;
+        const int c = p >= 0 ? min(int(cnt[p]), K) : 0;
+        const int id = j < c ? ids[p * K + j] : -1;
+        const float w = j < c ? wts[p * K + j] : 0.f;
+        const unsigned listed = __ballot_sync(FULL, j < c);
+        float2 g[4][NP];
+        if (listed == 0u) continue;
+#pragma unroll
+        for (int mm = 0; mm < 4; ++mm) {
+            if ((listed >> (mm * K)) & 1u) {   // entry 0 of the pixel
+                load_row(grad_out + pixel(mm) * int64_t(C), g[mm]);
+            } else {
+#pragma unroll
+                for (int i = 0; i < NP; ++i) g[mm][i] = make_float2(0.f, 0.f);
+            }
+        }
+        // the distinct rows: slot = rank of the row's first lane
+        const unsigned peers = __match_any_sync(FULL, id);
+        const int leader = __ffs(peers) - 1;
+        const unsigned leaders = __ballot_sync(FULL, j < c && lane == leader);
+        const int slot = __popc(leaders & ((1u << leader) - 1u));
+        const int rows = __popc(leaders);
+        if (j < c && lane == leader) s_id[warp][slot] = id;
+        __syncwarp();
+        // s = g . f for every row and pixel, two rows in flight
+        for (int r = 0; r < rows; r += 2) {
+            uint4 rv[2][VPL];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const unsigned char *row = feat + size_t(s_id[warp][min(r + u, rows - 1)]) * row_bytes;
+#pragma unroll
+                for (int t = 0; t < VPL; ++t)
+                    rv[u][t] = *reinterpret_cast<const uint4 *>(row + size_t(lane + 32 * t) * 16);
+            }
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                float2 part[4];
+#pragma unroll
+                for (int mm = 0; mm < 4; ++mm) part[mm] = make_float2(0.f, 0.f);
+#pragma unroll
+                for (int t = 0; t < VPL; ++t) {
+                    float fv[CPV];
+                    widen<DT>(rv[u][t], fv);
+#pragma unroll
+                    for (int k = 0; k < CPV / 2; ++k)
+#pragma unroll
+                        for (int mm = 0; mm < 4; ++mm)
+                            fma2x(part[mm], fv[2 * k], fv[2 * k + 1], g[mm][t * CPV / 2 + k]);
+                }
+                float v4[4];
+#pragma unroll
+                for (int mm = 0; mm < 4; ++mm) v4[mm] = part[mm].x + part[mm].y;
+                const float x = reduce4(v4, lane);
+                // lane red4_lane(mm) holds pixel mm's dot
+                if ((lane & 7) == 0 && r + u < rows)
+                    s_dot[warp][r + u][2 * ((lane >> 4) & 1) + ((lane >> 3) & 1)] = x;
+            }
+        }
+        __syncwarp();
+        float s_mine = 0.f, a = 0.f, G = 0.f, dx = 0.f, dy = 0.f;
+        bool clamped = false;
+        if (j < c) {
+            s_mine = s_dot[warp][slot][m];
+            if (DT == QR_FP8E4M3) s_mine *= fscale[id];
+            // alpha', G, offsets, recomputed exactly as in the forward
+            const PixelTerm t = eval_half_q(float(gx + (m & 1)) + 0.5f, float(gy + (m >> 1)) + 0.5f,
+                                            rec_m[id], rec_w[id]);
+            const float alpha = rec_a[id];
+            G = __expf(-t.half_q);
+            a = eval_alpha(alpha, t.half_q, alpha_max);
+            clamped = !(alpha * G < alpha_max);
+            dx = t.dx;
+            dy = t.dy;
+        }
+        // prefix products, T^Q, g.F and suffix sums of each pixel (sequential,
+        // like the forward; entries past a pixel's count leave them unchanged)
+        const int first = m < 4 ? m * K : 0;
+        float Pj = 1.f, Pmine = 1.f, gF = 0.f;
+        for (int k = 0; k < K; ++k) {
+            const float ak = __shfl_sync(FULL, a, first + k), wk = __shfl_sync(FULL, w, first + k),
+                        sk = __shfl_sync(FULL, s_mine, first + k);
+            if (j == k) Pmine = Pj;
+            if (k < c) {
+                gF = fmaf(wk, sk, gF);
+                Pj = Pj * (1.f - ak);
+            }
+        }
+        const float TQ = Pj, D = 1.f - TQ;
+        float suffix = 0.f, smine_suffix = 0.f;
+        for (int k = K - 1; k >= 0; --k) {
+            const float ak = __shfl_sync(FULL, a, first + k), pk = __shfl_sync(FULL, Pmine, first + k),
+                        sk = __shfl_sync(FULL, s_mine, first + k);
+            if (j == k) smine_suffix = suffix;
+            if (k < c) suffix = fmaf(ak * pk, sk, suffix);
+        }
+        if (j < c) {
+            const float om = 1.f - a;
+            const float da = (Pmine * s_mine - smine_suffix / om) / D - gF * TQ / (om * D);
+            float4 e = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (!clamped) {
+                const float h = -0.5f * a * da;
+                e = make_float4(da * G, h * dx * dx, h * 2.f * dx * dy, h * dy * dy);
+            }
+            E[p * K + j] = e;
+        }
+        __syncwarp();   // the tables are rewritten by the next group
+    }
+}
+
 // acc += w * g for both halves with one packed FP32x2 FMA (each half rounds
 // exactly like fmaf).
 __device__ __forceinline__ void fma2v(float2 &acc, float w, float2 g) {
@@ -795,6 +958,23 @@ void launch_bwd_pixel(const qr_frame &f, const void *feat, const float *scale, i
             static_cast<const unsigned char *>(feat), scale, C, ids, w, cnt, g, P, f.params.K,
             f.camera.width, f.params.alpha_max, E, pl);
     };
+    // four pixels' rows of up to 16 channels per lane fit a warp's registers
+    auto group = [&](auto kern) {
+        const unsigned strips = unsigned((f.camera.width + 15) / 16) * unsigned((f.camera.height + 7) / 8);
+        kern<<<strips, T, 0, s>>>(
+            slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C), slot<float>(f, S_REC_A),
+            static_cast<const unsigned char *>(feat), scale, C, ids, w, cnt, g, f.params.K,
+            f.camera.width, f.camera.height, f.params.alpha_max, E);
+    };
+    constexpr int CPV = VecB<DT>::C;
+    if (!loss && f.params.K <= 8 && vpl > 0 && vpl * CPV <= 16) {
+        if (vpl == 1) group(bwd_group<DT, 1>);
+        if constexpr (CPV <= 8)
+            if (vpl == 2) group(bwd_group<DT, 2>);
+        if constexpr (CPV <= 4)
+            if (vpl == 4) group(bwd_group<DT, 4>);
+        return;
+    }
     if (loss) {
         switch (vpl) {
             case 1: go(bwd_pixel<DT, 1, true>); break;

@@ -131,6 +131,61 @@ def test_backward_room_matches_oracle(K):
     print(f"room K={K} backward errors in yardstick units", e)
 
 
+@pytest.mark.parametrize("kind,C,K", [("f32", 128, 8), ("f32", 256, 1), ("f32", 512, 3), ("bf16", 256, 5),
+                                      ("bf16", 512, 8), ("fp8", 512, 7)])
+def test_backward_pixel_groups(kind, C, K):
+    """The per-entry terms of 2 x 2 pixels by one warp: every width and dtype it
+    serves, numbers of entries that do not divide a warp, an odd image."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=C)
+    fdev = torch.from_numpy(f).cuda()
+    table, decoded = None, f
+    if kind == "bf16":
+        table, decoded = q.qr_quantize_bf16(fdev), oracle.bf16_decode(oracle.bf16_encode(f))
+    elif kind == "fp8":
+        table, decoded = q.qr_quantize_fp8(fdev), oracle.fp8_dequantize_rows(*oracle.fp8_quantize_rows(f))
+    cam = scenes.room_camera(61, 45)
+    if kind == "fp8":
+        res = q.render_frame(q.gaussians_to_device(g), None, cam, K=K)
+        pr, pix, ref = H.run_oracle(g, decoded, cam, K)
+        gout = np.random.default_rng(C + K).normal(size=(cam.width * cam.height, C)).astype(np.float32)
+        gout[(ref.tie & compare.Q_TIE_BITS) != 0] = 0.0
+        got = q.qr_backward(res["frame"], *table, res["ids"], res["weights"], res["counts"],
+                            torch.from_numpy(gout).cuda())
+        got = tuple(x.cpu().numpy() for x in got)
+        ref = oracle.backward(pr, decoded, K, pix, gout.astype(np.float64), alpha_min=oracle.ALPHA_MIN_F32,
+                              alpha_max=oracle.ALPHA_MAX_F32, with_scales=True)
+    else:
+        got, ref = _run(g, f, cam, K, table=table, decoded=decoded, seed=C + K)
+    _check_all(got, ref)
+
+
+def test_backward_non_finite_gradient_stays_with_its_pixels():
+    """An infinite upstream gradient reaches the Gaussians its pixel lists and
+    no others; the rest is what it is without that pixel."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=512)
+    cam = scenes.room_camera(61, 45)
+    fdev = torch.from_numpy(f).cuda()
+    res = q.render_frame(q.gaussians_to_device(g), fdev, cam, K=8)
+    gout = torch.randn(cam.width * cam.height, 512, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    p = 20 * cam.width + 31
+    gout[p] = 0
+    call = lambda x: q.qr_backward(res["frame"], fdev, None, res["ids"], res["weights"], res["counts"], x)  # noqa: E731
+    want = call(gout)[0].clone()
+    gout[p, 100] = float("inf")
+    got = call(gout)[0]
+    listed = torch.zeros(g.n, dtype=torch.bool, device="cuda")
+    listed[res["ids"][p][:int(res["counts"][p])].long()] = True
+    assert listed.any()
+    assert torch.equal(got[~listed], want[~listed])
+    assert torch.isinf(got[listed][:, 100]).all()
+    other = torch.arange(512, device="cuda") != 100
+    assert torch.equal(got[listed][:, other], want[listed][:, other])
+
+
 def test_backward_bf16_table():
     import torch
     from paper_2512_20927_gb300 import qrender as q
