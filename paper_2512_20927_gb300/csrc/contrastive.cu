@@ -252,9 +252,12 @@ eq2_terms(const float *__restrict__ F, const float *__restrict__ tn, int M, int 
 //      over the eight lanes that share t;
 //   3. G = C T^ (M = pixels, N = channels, K = targets): the c_j fragments
 //      are gathered by shuffles, T^ fragments read from shared memory, and
-//      each 16 x 8 result, (G / nf - (sum_j c_j s_j) F / nf^2) / n, is
+//      each 16 x 16 result, (G / nf - (sum_j c_j s_j) F / nf^2) / n, is
 //      written (streaming stores) with the F values it needs re-read (they
 //      were read moments before and come from L2).
+// Bound by shared-memory reads of T^ (68 %), issue (51 %) and the tensor pipe.
+// Room VGA, 512 channels, 32 patches: 531 us with 8-channel steps, 4-byte
+// fragment reads and the F values loaded one step ahead; 478 us now.
 constexpr int kMmaThreads = 512;
 
 template <int MT>
@@ -438,32 +441,47 @@ eq2_mma(const float *__restrict__ F, const float *__restrict__ tn, int M, int C,
             const int64_t pxa = p0 + pa, pxb = p0 + pb;
             const float a1a = s_a1[warp][pa], a2a = s_a2[warp][pa];
             const float a1b = s_a1[warp][pb], a2b = s_a2[warp][pb];
-            // F values of the F term, one 8-channel step ahead
-            auto load_f2 = [&](int64_t px, int c) {
-                return (px < P && c < C) ? __ldg(reinterpret_cast<const float2 *>(F + px * C + c))
-                                         : make_float2(0.f, 0.f);
+            // 16 channels a step, as two 8-column products: column n of the first
+            // is channel 2 n, of the second 2 n + 1, so a lane's four results
+            // per pixel are channels 4 t .. 4 t + 3 and one 8-byte read serves
+            // both products' T^ fragments.  The F values of the F term are
+            // loaded two steps ahead (they come from L2).
+            auto load_f4 = [&](int64_t px, int c) {
+                return (px < P && c < C) ? __ldg(reinterpret_cast<const float4 *>(F + px * C + c))
+                                         : make_float4(0.f, 0.f, 0.f, 0.f);
             };
-            float2 fa = load_f2(pxa, 2 * t), fb = load_f2(pxb, 2 * t);
-            for (int c0 = 0; c0 < C; c0 += 8) {
-                const float2 fa_n = load_f2(pxa, c0 + 8 + 2 * t), fb_n = load_f2(pxb, c0 + 8 + 2 * t);
-                float d[4] = {0.f, 0.f, 0.f, 0.f};
+            float4 fa = load_f4(pxa, 4 * t), fb = load_f4(pxb, 4 * t);
+            float4 fa1 = load_f4(pxa, 16 + 4 * t), fb1 = load_f4(pxb, 16 + 4 * t);
+            for (int c0 = 0; c0 < C; c0 += 16) {
+                const float4 fa2 = load_f4(pxa, c0 + 32 + 4 * t), fb2 = load_f4(pxb, c0 + 32 + 4 * t);
+                float d[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int kk = 0; kk < 2 * MT; ++kk) {
-                    const int r0 = (8 * kk + t) * S + c0 + g, r1 = r0 + 4 * S;
-                    mma3(d, ch[kk], cl[kk], __float_as_uint(s_hi[r0]), __float_as_uint(s_hi[r1]),
-                         __float_as_uint(s_lo[r0]), __float_as_uint(s_lo[r1]));
+                    const int r0 = (8 * kk + t) * S + c0 + 2 * g, r1 = r0 + 4 * S;
+                    const float2 h0 = *reinterpret_cast<const float2 *>(s_hi + r0);
+                    const float2 h1 = *reinterpret_cast<const float2 *>(s_hi + r1);
+                    const float2 l0 = *reinterpret_cast<const float2 *>(s_lo + r0);
+                    const float2 l1 = *reinterpret_cast<const float2 *>(s_lo + r1);
+                    mma3(d, ch[kk], cl[kk], __float_as_uint(h0.x), __float_as_uint(h1.x),
+                         __float_as_uint(l0.x), __float_as_uint(l1.x));
+                    mma3(e, ch[kk], cl[kk], __float_as_uint(h0.y), __float_as_uint(h1.y),
+                         __float_as_uint(l0.y), __float_as_uint(l1.y));
                 }
-                const int cc = c0 + 2 * t;
+                const int cc = c0 + 4 * t;
                 if (pxa < P)
-                    __stcs(reinterpret_cast<float2 *>(grad + pxa * C + cc),
-                           a1a > 0.f ? make_float2(fmaf(d[0], a1a, -a2a * fa.x), fmaf(d[1], a1a, -a2a * fa.y))
-                                     : make_float2(0.f, 0.f));
+                    __stcs(reinterpret_cast<float4 *>(grad + pxa * C + cc),
+                           a1a > 0.f ? make_float4(fmaf(d[0], a1a, -a2a * fa.x), fmaf(e[0], a1a, -a2a * fa.y),
+                                                   fmaf(d[1], a1a, -a2a * fa.z), fmaf(e[1], a1a, -a2a * fa.w))
+                                     : make_float4(0.f, 0.f, 0.f, 0.f));
                 if (pxb < P)
-                    __stcs(reinterpret_cast<float2 *>(grad + pxb * C + cc),
-                           a1b > 0.f ? make_float2(fmaf(d[2], a1b, -a2b * fb.x), fmaf(d[3], a1b, -a2b * fb.y))
-                                     : make_float2(0.f, 0.f));
-                fa = fa_n;
-                fb = fb_n;
+                    __stcs(reinterpret_cast<float4 *>(grad + pxb * C + cc),
+                           a1b > 0.f ? make_float4(fmaf(d[2], a1b, -a2b * fb.x), fmaf(e[2], a1b, -a2b * fb.y),
+                                                   fmaf(d[3], a1b, -a2b * fb.z), fmaf(e[3], a1b, -a2b * fb.w))
+                                     : make_float4(0.f, 0.f, 0.f, 0.f));
+                fa = fa1;
+                fb = fb1;
+                fa1 = fa2;
+                fb1 = fb2;
             }
         }
         __syncwarp();   // s_a1 / s_a2 are rewritten by the next block
