@@ -738,11 +738,11 @@ cudaError_t launch_sort(const qr_frame &f, cudaStream_t s) {
         e = cudaFuncSetAttribute(expand_scatter<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  int(sizeof(uint32_t) * 2 * kAggTiles));
         if (e != cudaSuccess) return e;
-        e = pdl_launch(expand_scatter<true>, dim3(sms * 4), dim3(T), agg, s, (const uint32_t *)koff,
+        e = pdl_launch(expand_scatter<true>, dim3(min(uint32_t(sms) * 4, nchunk)), dim3(T), agg, s, (const uint32_t *)koff,
                        (const uint32_t *)kid, rect, (const uint32_t *)slot<uint32_t>(f, S_GKEY),
                        (const uint32_t *)chunk_owner, counters, f.tiles_x, tiles, ranges, tcnt, keys);
     } else {
-        e = pdl_launch(expand_scatter<false>, dim3(sms * 6), dim3(T), 0, s, (const uint32_t *)koff,
+        e = pdl_launch(expand_scatter<false>, dim3(min(uint32_t(sms) * 6, nchunk)), dim3(T), 0, s, (const uint32_t *)koff,
                        (const uint32_t *)kid, rect, (const uint32_t *)slot<uint32_t>(f, S_GKEY),
                        (const uint32_t *)chunk_owner, counters, f.tiles_x, tiles, ranges, tcnt, keys);
     }
@@ -751,12 +751,14 @@ cudaError_t launch_sort(const qr_frame &f, cudaStream_t s) {
     // holds the list of big buckets
     e = pdl_launch(tile_sort, dim3(tiles), dim3(T), 0, s, (const uint2 *)ranges, keys,
                    slot<uint32_t>(f, S_IGID), tcnt, counters);
-    if (e != cudaSuccess) return e;
+    count_launch(4);
+    // no bucket holds more keys than there are Gaussians
+    if (e != cudaSuccess || f.n <= 8 * T) return e != cudaSuccess ? e : cudaGetLastError();
     e = pdl_launch(tile_sort_big, dim3(unsigned(min(tiles, sms))), dim3(TB),
                    2 * BIG_SLOTS * sizeof(unsigned long long), s,
                    (const uint2 *)ranges, keys, slot<unsigned long long>(f, S_SCRATCH64),
                    slot<uint32_t>(f, S_IGID), (const uint32_t *)tcnt, (const uint32_t *)counters);
-    count_launch(5);
+    count_launch(1);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
