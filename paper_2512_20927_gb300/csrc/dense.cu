@@ -6,8 +6,8 @@
 // fall below T_min.
 //
 // GB300 design: every pixel of a tile walks the same list, so the blend is a
-// dense product W (pixels x entries) * F (entries x channels).  Rows of 128,
-// 256 or 512 channels go to dense_block_kernel (below: warp-specialised walk,
+// dense product W (pixels x entries) * F (entries x channels).  Rows of 64,
+// 128, 256 or 512 channels go to dense_block_kernel (below: warp-specialised walk,
 // row copies and accumulation over 8 x 8 pixel blocks).  Other widths use
 // dense_kernel, 32 list entries at a time, where one CTA owns a screen tile
 // and a 16/32/64-channel slice:
@@ -197,7 +197,7 @@ dense_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 }
 
 // ------------------------------------------------------------------ block kernel
-// Rows of 128, 256 or 512 channels.  One persistent CTA per SM; a work item is
+// Rows of 64, 128, 256 or 512 channels.  One persistent CTA per SM; a work item is
 // an 8 x 8 pixel block over all C channels, so each pixel's alpha' / T walk
 // runs once.  The blend itself (8 pixels x C channels per group and kept
 // entry) is bound by the FP32 pipe, so everything else runs beside it in
@@ -231,7 +231,11 @@ dense_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 // barriers; 566 us now.  The roles alone: consumers 320 us at the FP32 peak,
 // walk and copies without the multiply-adds 326 us.  Five warps per scheduler
 // (20 in all) leave a consumer 96 registers; a 21st warp cost 80 and spills
-// (1096 us), two producers 585 us.
+// (1096 us), two producers 585 us.  Other rows (slices of 64 channels that walk
+// again, or the 16 x 4 kernel -> now): room VGA C = 64 FP32 401 -> 332 us, C = 128
+// FP8 757 -> 343 us; object VGA C = 256 BF16 1470 -> 813 us, C = 512 FP32 1752 ->
+// 868 us; object 320 x 240 C = 64 BF16 585 -> 327 us; room 160 x 100 C = 64 47 ->
+// 30 us.
 constexpr int kProd = 3;                     // producer warps
 constexpr int kSlots = 6;                    // weight slots per producer
 constexpr int kEnt = 16;                     // entries per slot
@@ -309,12 +313,14 @@ __device__ __forceinline__ BlockPos dense_block(int block, int tile_w, int tiles
             (tile / tiles_x) * (kSelPix / tile_w) + (part / across) * 8};
 }
 
-template <int WPG>
-constexpr int dense_threads() { return 32 * (8 * WPG + kProd + 1); }
+// Warps per pixel group and quads per lane of a row of C channels (64 channels
+// leave half of a warp's lanes without one).
+constexpr int dense_wpg(int C) { return C >= 256 ? 2 : 1; }
+constexpr int dense_qpt(int C) { return C > 128 ? C / 256 : 1; }
+constexpr int dense_threads(int C) { return 32 * (8 * dense_wpg(C) + kProd + 1); }
 
-// C = 128 WPG QPT
-template <int DT, int QPT, int WPG>
-__global__ void __launch_bounds__(dense_threads<WPG>(), 1)
+template <int DT, int C>
+__global__ void __launch_bounds__(dense_threads(C), 1)
 dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
                    const float *__restrict__ rec_a, const float *__restrict__ rec_h,
                    const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges,
@@ -324,7 +330,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                    unsigned long long *__restrict__ stats, uint32_t *__restrict__ counters) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int QB = Quad<DT>::B;
-    constexpr int C = 128 * WPG * QPT;
+    constexpr int WPG = dense_wpg(C), QPT = dense_qpt(C);
     constexpr uint32_t ROW = uint32_t(C / 4) * QB;           // bytes of a row
     constexpr int NCW = 8 * WPG;                             // consumer warps
     extern __shared__ __align__(128) unsigned char s_dyn[];
@@ -356,7 +362,8 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
     if (warp < NCW) {
         // ------------------------------------------------------ consumers
         const int g = warp / WPG;
-        const int q0 = (warp % WPG) * 32 + lane;             // first quad; then + 32 WPG
+        const int q0 = ((warp % WPG) * 32 + lane) % (C / 4);   // first quad; then + 32 WPG
+        const bool spare = C < 128 && lane >= C / 4;         // a lane without a quad of its own
         float acc[8][QPT][4];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -411,7 +418,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                     float4 *o = reinterpret_cast<float4 *>(out) + (int64_t(y) * W + x) * (C / 4) + q0;
 #pragma unroll
                     for (int k = 0; k < QPT; ++k) {
-                        if (x < W && y < H)
+                        if (x < W && y < H && !spare)
                             __stcs(o + 32 * WPG * k, make_float4(acc[i][k][0], acc[i][k][1], acc[i][k][2], acc[i][k][3]));
 #pragma unroll
                         for (int c = 0; c < 4; ++c) acc[i][k][c] = 0.f;
@@ -419,7 +426,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                 }
             }
         }
-        if (stats && lane == 0) atomicAdd(&stats[1], n_exec * 32ull * 8ull * 4ull * QPT);
+        if (stats && lane == 0) atomicAdd(&stats[1], n_exec * 8ull * (C / WPG));
     } else if (warp < NCW + kProd) {
         // ------------------------------------------------------ producers
         const int p = warp - NCW;
@@ -572,15 +579,15 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
     if (threadIdx.x == 0 && *abort) atomicExch(&counters[CNT_STATUS], uint32_t(QR_ERR_DEVICE_TIMEOUT));
 }
 
-template <int DT, int QPT, int WPG>
+template <int DT, int C>
 cudaError_t run_block(const qr_frame &f, const void *feat, const float *scale, float *out,
                       float *T_final, unsigned long long *stats, cudaStream_t s) {
-    constexpr size_t dyn = kDenseShared + size_t(kRows) * kEnt * 32 * WPG * QPT * Quad<DT>::B;
+    constexpr size_t dyn = kDenseShared + size_t(kRows) * kEnt * (C / 4) * Quad<DT>::B;
     static_assert(dyn <= 227 * 1024, "shared memory");
-    cudaError_t e = cudaFuncSetAttribute(dense_block_kernel<DT, QPT, WPG>,
+    cudaError_t e = cudaFuncSetAttribute(dense_block_kernel<DT, C>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
     if (e != cudaSuccess) return e;
-    dense_block_kernel<DT, QPT, WPG><<<unsigned(num_tiles(f)) * 4, dense_threads<WPG>(), dyn, s>>>(
+    dense_block_kernel<DT, C><<<unsigned(num_tiles(f)) * 4, dense_threads(C), dyn, s>>>(
         slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C), slot<float>(f, S_REC_A),
         slot<float>(f, S_REC_H), slot<uint32_t>(f, S_IGID), slot<uint2>(f, S_RANGES),
         static_cast<const unsigned char *>(feat), scale, f.camera.width, f.camera.height,
@@ -609,9 +616,10 @@ cudaError_t dispatch(const qr_frame &f, const void *feat, const float *scale, in
                      float *T_final, unsigned long long *stats, cudaStream_t s) {
     constexpr int cpv = Cpv<DT>::v;
     // wide rows: one walk per pixel, culled and skipped entries
-    if (C == 512) return run_block<DT, 2, 2>(f, feat, scale, out, T_final, stats, s);
-    if (C == 256) return run_block<DT, 1, 2>(f, feat, scale, out, T_final, stats, s);
-    if (C == 128 && cpv <= 8) return run_block<DT, 1, 1>(f, feat, scale, out, T_final, stats, s);
+    if (C == 512) return run_block<DT, 512>(f, feat, scale, out, T_final, stats, s);
+    if (C == 256) return run_block<DT, 256>(f, feat, scale, out, T_final, stats, s);
+    if (C == 128) return run_block<DT, 128>(f, feat, scale, out, T_final, stats, s);
+    if (C == 64) return run_block<DT, 64>(f, feat, scale, out, T_final, stats, s);
     if (C % 64 == 0) return run<DT, 64, 8, 8>(f, feat, scale, C, out, T_final, s);
     if (C % 32 == 0) return run<DT, 32, 8, 4>(f, feat, scale, C, out, T_final, s);
     if (C % 16 == 0) return run<DT, 16, 4, 4>(f, feat, scale, C, out, T_final, s);
