@@ -15,7 +15,7 @@
 // each kept Gaussian weighted by the number of boundaries T_test crosses at
 // it, divided by the number crossed in all.
 //
-// GB300 design: one warp per 8 x 8 pixel block (select_tile.cuh) and per CTA,
+// GB300 design: one warp per 8 x 8 pixel block or half of one (select_tile.cuh) and per CTA,
 // so an SM takes a new block as soon as one is done.  Measured with K = 8
 // (512-D VGA frames but for the last; CTAs of four warps walking a 16 x 16
 // tile in step, 128 staged entries at a time -> now):
@@ -25,48 +25,68 @@
 //   2,000 Gaussians at 128 x 128 (256 warps in all)  41.8 -> 18.8 us (latency)
 // Two or four warps per CTA measured 0-5 % slower; a bound of 32 warps per SM
 // (64 registers) instead of 24 cost up to 13 %.
+// Where latency bounds it, a warp takes half a block (8 x 4 pixels, one per
+// lane): each step of its chain is shorter, the list is culled twice as often.
+// That is so for images of few blocks and where lists are long, for which the
+// capacity of the lists per tile stands (the host does not know their lengths;
+// a caller sizes it by the frame's intersections).  Whole blocks / halves, K =
+// 8 unless stated: 2,000 Gaussians at 128 x 128 25 / 17 us, room at 320 x 240 23 /
+// 19, at 480 x 360 23 / 25, at 640 x 480 31 / 33, 1M room at 1296 x 968 85 / 109;
+// object (2,500 entries per tile at VGA) at 320 x 240 167 / 117, at 640 x 480
+// 130 / 115 (K = 16: 165 / 134, K = 32: 206 / 189), at 1000 x 700 127 / 122.
+// Halving only the blocks of long lists (the second halves' CTAs leave early
+// elsewhere) cost 2-9 us wherever lists are short.
 #include "select_tile.cuh"
 
 namespace qr {
 namespace {
 
-constexpr int kSelWarps = 1;      // divides 4
+// 8 x 8 blocks up to which, and capacity per tile from which, blocks are halved
+constexpr int kSmallBlocks = 152 * 8;
+constexpr int64_t kLongLists = 2048;
 
+// One CTA of one warp per 8 x (4 PX) pixels.
 // kCount: App. C's Riemann weights in place of Algorithm 1's (select_block).
-template <bool kCount>
-__global__ void __launch_bounds__(32 * kSelWarps, 24 / kSelWarps)
+template <bool kCount, int PX>
+__global__ void __launch_bounds__(32, 24)
 select_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
               const float *__restrict__ rec_a, const float *__restrict__ rec_h,
               const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
               int H, int tile_w, int tiles_x, int K, float alpha_min, float alpha_max,
               int32_t *__restrict__ ids, float *__restrict__ wout, uint8_t *__restrict__ cnt,
               int vec) {
-    __shared__ SelStage st[kSelWarps];
+    constexpr int N = 8 / PX;                                     // blocks per tile
+    __shared__ SelStage st;
     __shared__ float s_thr[kKMax + 1];
     extern __shared__ unsigned char s_dyn[];
     const int KS = K | 1;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int32_t *s_ids = reinterpret_cast<int32_t *>(s_dyn) + warp * kSelBlock * KS;   // [64][KS] per warp
-    float *s_w = reinterpret_cast<float *>(s_dyn) + (kSelWarps + warp) * kSelBlock * KS;
+    const int lane = threadIdx.x & 31;
+    int32_t *s_ids = reinterpret_cast<int32_t *>(s_dyn);          // [32 PX][KS]
+    float *s_w = reinterpret_cast<float *>(s_dyn) + 32 * PX * KS;
     select_boundaries(s_thr, K);
     __syncthreads();
     pdl_wait();   // the predecessor's outputs are complete and visible
-    const int block = int(blockIdx.x) * kSelWarps + warp;
-    const int tile = block >> 2, part = block & 3, across = tile_w >> 3;
+    const int tile = int(blockIdx.x) / N, part = int(blockIdx.x) % N, across = tile_w >> 3;
     const int x0 = (tile % tiles_x) * tile_w + (part % across) * 8;
-    const int y0 = (tile / tiles_x) * (kSelPix / tile_w) + (part / across) * 8;
-    const int sa = (2 * (lane >> 3)) * 8 + (lane & 7), sb = sa + 8;
+    const int y0 = (tile / tiles_x) * (kSelPix / tile_w) + (part / across) * 4 * PX;
+    const int px = x0 + (lane & 7), py = y0 + PX * (lane >> 3);
+    const int sa = PX * (lane >> 3) * 8 + (lane & 7), sb = sa + 8;
     Walk w0, w1;
-    select_block<kCount>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[tile], W, H, x0, y0, K,
-                         alpha_min, alpha_max, s_thr, st[warp], s_ids + sa * KS, s_w + sa * KS,
-                         s_ids + sb * KS, s_w + sb * KS, w0, w1);
+    if constexpr (PX == 2) {
+        select_block<kCount>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[tile], W, H, x0, y0, K,
+                             alpha_min, alpha_max, s_thr, st, s_ids + sa * KS, s_w + sa * KS,
+                             s_ids + sb * KS, s_w + sb * KS, w0, w1);
+        finish_pixel<kCount>(w1, K, s_ids + sb * KS, s_w + sb * KS);
+    } else {
+        select_block1<kCount>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[tile], W, H, x0, y0, K,
+                              alpha_min, alpha_max, s_thr, st, s_ids + sa * KS, s_w + sa * KS, w0);
+    }
     finish_pixel<kCount>(w0, K, s_ids + sa * KS, s_w + sa * KS);
-    finish_pixel<kCount>(w1, K, s_ids + sb * KS, s_w + sb * KS);
     __syncwarp();
-    store_block(W, H, x0, y0, K, vec != 0, s_ids, s_w, [](int x, int y) { return y * 8 + x; }, ids, wout);
-    const int px = x0 + (lane & 7), py = y0 + 2 * (lane >> 3);
+    store_block<32 * PX>(W, H, x0, y0, K, vec != 0, s_ids, s_w, [](int x, int y) { return y * 8 + x; }, ids, wout);
     if (px < W && py < H) cnt[int64_t(py) * W + px] = uint8_t(w0.m);
-    if (px < W && py + 1 < H) cnt[int64_t(py + 1) * W + px] = uint8_t(w1.m);
+    if constexpr (PX == 2)
+        if (px < W && py + 1 < H) cnt[int64_t(py + 1) * W + px] = uint8_t(w1.m);
 }
 
 }  // namespace
@@ -76,10 +96,9 @@ cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cn
     const int tiles = num_tiles(f);
     if (tiles == 0) return cudaSuccess;
     const int K = f.params.K;
-    const size_t dyn = size_t(K | 1) * kSelBlock * kSelWarps * 8;
     const int vec = K % 4 == 0 && ((reinterpret_cast<uintptr_t>(ids) | reinterpret_cast<uintptr_t>(w)) & 15) == 0;
-    auto go = [&](auto kern) -> cudaError_t {
-        return pdl_launch(kern, dim3(unsigned(tiles) * 4 / kSelWarps), dim3(32 * kSelWarps), dyn, s,
+    auto go = [&](auto kern, int px) -> cudaError_t {
+        return pdl_launch(kern, dim3(unsigned(tiles) * (8 / px)), dim3(32), size_t(K | 1) * 32 * px * 8, s,
                           (const float4 *)slot<float4>(f, S_REC_M),
                           (const float4 *)slot<float4>(f, S_REC_C),
                           (const float *)slot<float>(f, S_REC_A),
@@ -89,7 +108,11 @@ cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cn
                           f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
                           f.params.alpha_max, ids, w, cnt, vec);
     };
-    const cudaError_t e = riemann ? go(select_kernel<true>) : go(select_kernel<false>);
+    cudaError_t e;
+    if (tiles * 4 <= kSmallBlocks || f.max_isect >= kLongLists * tiles)
+        e = riemann ? go(select_kernel<true, 1>, 1) : go(select_kernel<false, 1>, 1);
+    else
+        e = riemann ? go(select_kernel<true, 2>, 2) : go(select_kernel<false, 2>, 2);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -282,6 +282,36 @@ __device__ __forceinline__ void select_block(
                       st, visit);
 }
 
+// The same over an 8 x 4 block, one pixel per lane.
+template <bool kCount = false>
+__device__ __forceinline__ void select_block1(
+    const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+    const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+    const uint32_t *__restrict__ isect_gid, uint2 range, int W, int H, int x0, int y0, int K,
+    float alpha_min, float alpha_max, const float *s_thr, SelStage &st, int32_t *ids, float *wts, Walk &w) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool inside = x0 + (lane & 7) < W && y0 + (lane >> 3) < H;
+    w = Walk{1.0f, 1.0f, inside ? s_thr[0] : -1.0f, inside ? 0 : K, 0};
+    auto visit = [&](int j, const float (&a)[4][1]) -> bool {
+        float t[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) t[u] = w.T = __fmul_rn(w.T, __fsub_rn(1.0f, a[u][0]));
+        if (!__any_sync(FULL, w.T < w.thr)) return true;
+        do {
+            if (w.T < w.thr) {
+                const int u = t[0] < w.thr ? 0 : t[1] < w.thr ? 1 : t[2] < w.thr ? 2 : 3;
+                const float e = u == 0 ? a[0][0] : u == 1 ? a[1][0] : u == 2 ? a[2][0] : a[3][0];
+                const float Tt = u == 0 ? t[0] : u == 1 ? t[1] : u == 2 ? t[2] : t[3];
+                walk_event<kCount>(w, Tt, e, st.g[j + u], s_thr, ids, wts);
+            }
+        } while (__any_sync(FULL, w.T < w.thr));
+        return !__all_sync(FULL, w.k == K);
+    };
+    walk_block<false, 1>(rec_m, rec_w, rec_a, rec_h, isect_gid, range, W, H, x0, y0, alpha_min, alpha_max,
+                         st, visit);
+}
+
 // A pixel's kept weights divided by 1 - T^Q (kCount: by the boundaries crossed
 // in all), the rest of its K slots padded with id -1 and weight 0.
 template <bool kCount = false>
@@ -299,7 +329,7 @@ __device__ __forceinline__ void finish_pixel(const Walk &w, int K, int32_t *ids,
 // warp's lanes must have finished their pixels (__syncwarp between).  Rows of
 // a block are 8 K consecutive entries of the image; vec (K % 4 == 0 and
 // 16-byte aligned outputs) writes them four at a time.
-template <typename SlotOf, typename Put>
+template <int NPIX, typename SlotOf, typename Put>
 __device__ __forceinline__ void for_block(int W, int H, int x0, int y0, int K, bool vec,
                                           SlotOf slot_of, Put put) {
     const int lane = threadIdx.x & 31;
@@ -307,18 +337,18 @@ __device__ __forceinline__ void for_block(int W, int H, int x0, int y0, int K, b
     const int per = vec ? 4 : 1;
     const int KP = K / per;                        // units per pixel
     const uint32_t inv = (65536u + uint32_t(KP) - 1u) / uint32_t(KP);   // e / KP, e < 64 KP <= 2048
-    for (int e = lane; e < kSelBlock * KP; e += 32) {
+    for (int e = lane; e < NPIX * KP; e += 32) {
         const int pix = int((uint32_t(e) * inv) >> 16), j = (e - pix * KP) * per;
         const int x = x0 + (pix & 7), y = y0 + (pix >> 3);
         if (x >= W || y >= H) continue;
         put(slot_of(pix & 7, pix >> 3) * KS + j, (int64_t(y) * W + x) * K + j);
     }
 }
-template <typename SlotOf>
+template <int NPIX = kSelBlock, typename SlotOf>
 __device__ __forceinline__ void store_block(int W, int H, int x0, int y0, int K, bool vec,
                                             const int32_t *s_ids, const float *s_w, SlotOf slot_of,
                                             int32_t *__restrict__ ids, float *__restrict__ wout) {
-    for_block(W, H, x0, y0, K, vec, slot_of, [&](int at, int64_t o) {
+    for_block<NPIX>(W, H, x0, y0, K, vec, slot_of, [&](int at, int64_t o) {
         if (vec) {
             *reinterpret_cast<int4 *>(ids + o) = make_int4(s_ids[at], s_ids[at + 1], s_ids[at + 2], s_ids[at + 3]);
             *reinterpret_cast<float4 *>(wout + o) = make_float4(s_w[at], s_w[at + 1], s_w[at + 2], s_w[at + 3]);

@@ -301,7 +301,8 @@ def test_dense_without_early_stop():
     H.check_frame(gpu, ref, pix, cam.width, f, FEAT_TOL, DENSE_TOL, label="T_min=0")
 
 
-@pytest.mark.parametrize("C,T_min,size", [(128, 0.0, (48, 48)), (256, 1e-4, (41, 23)), (512, 0.0, (17, 9))])
+@pytest.mark.parametrize("C,T_min,size", [(64, 1e-4, (33, 50)), (128, 0.0, (48, 48)), (256, 1e-4, (41, 23)),
+                                          (512, 0.0, (17, 9))])
 def test_dense_long_lists(C, T_min, size):
     """Blocks that keep hundreds of entries (every ring of the block kernel
     wraps around), images smaller than a tile and with cut blocks."""
@@ -527,3 +528,26 @@ def test_selection_block_edges(w, h, K, tile):
     assert (wts[1:-1].cpu().numpy().reshape(P, K) == gpu["weights"]).all()
     assert (cnt.cpu().numpy() == gpu["counts"]).all()
     assert ids[0] == -7 and ids[-1] == -7 and wts[0] == -7 and wts[-1] == -7
+
+
+@pytest.mark.parametrize("K,tile", [(8, (16, 16)), (5, (32, 8)), (32, (8, 32))])
+def test_selection_whole_and_half_blocks_agree(K, tile):
+    """The two block sizes of the selection (by the capacity of the lists per
+    tile) keep the same Gaussians with the same weights on a ragged image."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=16)
+    cam = scenes.room_camera(517, 389)
+    gdev = q.gaussians_to_device(g)
+    params = q.default_params(K, tile_w=tile[0], tile_h=tile[1])
+    tiles = -(-517 // tile[0]) * -(-389 // tile[1])
+    for rule in (q.QR_RULE_QUANTILE, q.QR_RULE_RIEMANN):
+        outs = []
+        for per_tile in (500, 2048):
+            res = q.render_frame(gdev, None, cam, K=K, params=params, max_isect=per_tile * tiles, rule=rule)
+            torch.cuda.synchronize()
+            assert res["frame"].frame.max_isect == per_tile * tiles and res["n_isect"] > 0
+            outs.append(res)
+        for k in ("ids", "weights", "counts"):
+            assert torch.equal(outs[0][k], outs[1][k]), (rule, k)
+        assert int(outs[0]["counts"].max()) > 1
