@@ -350,6 +350,15 @@ qr_status qr_backward(const qr_frame *frame, const void *feat, const float *feat
                       float *grad_opacity, float *grad_conic, void *ws, size_t ws_bytes,
                       qr_stream stream);
 
+/* qr_backward with grad_feat [n][C] stored as grad_dtype: QR_F32, or QR_BF16
+ * (each element of the float32 gradient rounded to nearest even), which spares
+ * a BF16 table's user the float32 rows and a pass that rounds them. */
+qr_status qr_backward_typed(const qr_frame *frame, const void *feat, const float *feat_scale,
+                            qr_dtype dtype, int32_t C, const int32_t *ids, const float *weights,
+                            const uint8_t *counts, const float *grad_out, void *grad_feat,
+                            qr_dtype grad_dtype, float *grad_opacity, float *grad_conic, void *ws,
+                            size_t ws_bytes, qr_stream stream);
+
 /* Loss of the differentiation workload (the paper trains with the contrastive
  * Eq. 2 on CLIP targets, which are not available): L = mean over pixels with
  * counts > 0 of 1 - cos(F_p, t_p), cos = F.t / (max(|F|, 1e-8) max(|t|, 1e-8)).

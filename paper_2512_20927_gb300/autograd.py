@@ -32,8 +32,10 @@ class QuantileRenderFunction(torch.autograd.Function):
         features, feat_scale, ids, weights, counts = ctx.saved_tensors
         P = ids.shape[0]
         g = grad_out.reshape(P, -1).float().contiguous()
+        # the rows of a BF16 table's gradient are rounded as they are written
         gf, ga, _ = q.qr_backward(ctx.frame, features, feat_scale, ids, weights, counts, g,
-                                  want_conic=False)
+                                  want_conic=False,
+                                  grad_dtype=torch.bfloat16 if features.dtype == torch.bfloat16 else None)
         gfeat = gf.to(features.dtype) if ctx.needs_input_grad[4] else None
         gop = ga if ctx.needs_input_grad[3] else None
         return None, None, None, gop, gfeat, None, None, None, None

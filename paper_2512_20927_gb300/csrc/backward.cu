@@ -799,12 +799,13 @@ isect_offsets(const uint32_t *__restrict__ tcount, const uint32_t *__restrict__ 
 // R = NW / nb, in order, eight rows in flight; the R partial sums are added in
 // subset order at the end.  Warp 0 adds the (dalpha, dA) terms of the found
 // slots in tile order.  Channel blocks beyond NW are taken in further rounds.
-template <int NT>
+// G: float, or uint16_t for gradient rows rounded to BF16 as they are written.
+template <int NT, typename G>
 __global__ void __launch_bounds__(NT)
 bwd_rows(const uint32_t *__restrict__ list, const uint32_t *__restrict__ d_nlist,
          const uint32_t *__restrict__ goff, const uint32_t *__restrict__ tcount,
          const uint32_t *__restrict__ slotmap, int64_t X, const float *__restrict__ partial,
-         const float4 *__restrict__ partial_s, int C, float *__restrict__ grad_feat,
+         const float4 *__restrict__ partial_s, int C, G *__restrict__ grad_feat,
          float *__restrict__ grad_alpha, float *__restrict__ grad_conic) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int NW = NT / 32;
@@ -872,7 +873,13 @@ bwd_rows(const uint32_t *__restrict__ list, const uint32_t *__restrict__ d_nlist
                     const float4 o = s_acc[warp + q * nb][lane];
                     t.x += o.x; t.y += o.y; t.z += o.z; t.w += o.w;
                 }
-                *reinterpret_cast<float4 *>(grad_feat + int64_t(g) * C + c0) = t;
+                if constexpr (sizeof(G) == 4) {
+                    *reinterpret_cast<float4 *>(grad_feat + int64_t(g) * C + c0) = t;
+                } else {
+                    const __nv_bfloat162 lo = __floats2bfloat162_rn(t.x, t.y), hi = __floats2bfloat162_rn(t.z, t.w);
+                    *reinterpret_cast<uint2 *>(grad_feat + int64_t(g) * C + c0) =
+                        make_uint2(*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi));
+                }
             }
             __syncthreads();
         }
@@ -997,7 +1004,7 @@ namespace {
 
 cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scale, qr_dtype dt,
                           int C, const int32_t *ids, const float *w, const uint8_t *cnt,
-                          const float *grad_out, const CosLossArgs *loss, float *grad_feat,
+                          const float *grad_out, const CosLossArgs *loss, void *grad_feat, bool bf16,
                           float *grad_alpha, float *grad_conic, void *ws, cudaStream_t s) {
     const BwdLayout L = bwd_layout(f, C);
     char *b = static_cast<char *>(ws);
@@ -1049,7 +1056,7 @@ cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scal
         }
         zs = side;
     }
-    e = cudaMemsetAsync(grad_feat, 0, size_t(f.n) * size_t(C) * 4, zs);
+    e = cudaMemsetAsync(grad_feat, 0, size_t(f.n) * size_t(C) * (bf16 ? 2 : 4), zs);
     if (e == cudaSuccess && grad_alpha) e = cudaMemsetAsync(grad_alpha, 0, size_t(f.n) * 4, zs);
     if (e == cudaSuccess && grad_conic) e = cudaMemsetAsync(grad_conic, 0, size_t(f.n) * 12, zs);
     // the side stream joins the caller's stream again (also on an error path)
@@ -1117,12 +1124,17 @@ cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scal
     if (e != cudaSuccess) return e;
     // the selected Gaussians' rows in tile order, over the cleared outputs
     const uint32_t *tcount = slot<uint32_t>(f, S_TCOUNT);
-    bwd_rows<256><<<unsigned(sms_now() * 8), 256, 0, s>>>(
-        lists, lists + 2 * f.n, goff, tcount, slotmap, f.max_isect, partial, partial_s, C,
-        grad_feat, grad_alpha, grad_conic);
-    bwd_rows<1024><<<unsigned(sms_now() * 2), 1024, 0, s>>>(
-        lists + f.n, lists + 2 * f.n + 1, goff, tcount, slotmap, f.max_isect, partial, partial_s,
-        C, grad_feat, grad_alpha, grad_conic);
+    auto rows = [&](auto zero) {
+        using G = decltype(zero);
+        bwd_rows<256, G><<<unsigned(sms_now() * 8), 256, 0, s>>>(
+            lists, lists + 2 * f.n, goff, tcount, slotmap, f.max_isect, partial, partial_s, C,
+            static_cast<G *>(grad_feat), grad_alpha, grad_conic);
+        bwd_rows<1024, G><<<unsigned(sms_now() * 2), 1024, 0, s>>>(
+            lists + f.n, lists + 2 * f.n + 1, goff, tcount, slotmap, f.max_isect, partial, partial_s,
+            C, static_cast<G *>(grad_feat), grad_alpha, grad_conic);
+    };
+    if (bf16) rows(uint16_t(0));
+    else rows(0.f);
     count_launch(5);
     return cudaGetLastError();
 }
@@ -1137,9 +1149,9 @@ size_t backward_cos_workspace_bytes(const qr_frame &f, int C) {
 
 cudaError_t launch_backward(const qr_frame &f, const void *feat, const float *scale, qr_dtype dt,
                             int C, const int32_t *ids, const float *w, const uint8_t *cnt,
-                            const float *grad_out, float *grad_feat, float *grad_alpha,
+                            const float *grad_out, void *grad_feat, bool bf16, float *grad_alpha,
                             float *grad_conic, void *ws, cudaStream_t s) {
-    return backward_impl(f, feat, scale, dt, C, ids, w, cnt, grad_out, nullptr, grad_feat,
+    return backward_impl(f, feat, scale, dt, C, ids, w, cnt, grad_out, nullptr, grad_feat, bf16,
                          grad_alpha, grad_conic, ws, s);
 }
 
@@ -1153,12 +1165,12 @@ cudaError_t launch_backward_cos(const qr_frame &f, const void *feat, const float
         cudaError_t e = launch_cosine_loss(loss.F, loss.tgt, loss.mask, P, C, loss.term, loss.out2,
                                            loss.grad_map, s);
         if (e != cudaSuccess) return e;
-        return launch_backward(f, feat, scale, dt, C, ids, w, cnt, loss.grad_map, grad_feat,
+        return launch_backward(f, feat, scale, dt, C, ids, w, cnt, loss.grad_map, grad_feat, false,
                                grad_alpha, grad_conic, ws, s);
     }
     cudaError_t e = launch_cos_count(loss.mask, P, loss.out2, s);
     if (e != cudaSuccess) return e;
-    return backward_impl(f, feat, scale, dt, C, ids, w, cnt, loss.grad_map, &loss, grad_feat,
+    return backward_impl(f, feat, scale, dt, C, ids, w, cnt, loss.grad_map, &loss, grad_feat, false,
                          grad_alpha, grad_conic, ws, s);
 }
 

@@ -353,12 +353,13 @@ size_t qr_backward_workspace_bytes(const qr_frame *frame, int32_t C) {
     return backward_workspace_bytes(*frame, C);
 }
 
-qr_status qr_backward(const qr_frame *frame, const void *feat, const float *feat_scale,
-                      qr_dtype dtype, int32_t C, const int32_t *ids, const float *weights,
-                      const uint8_t *counts, const float *grad_out, float *grad_feat,
-                      float *grad_opacity, float *grad_conic, void *ws, size_t ws_bytes,
-                      qr_stream stream) {
-    if (!frame_ok(frame) || !ids || !weights || !counts || !grad_out || !grad_feat || !ws)
+qr_status qr_backward_typed(const qr_frame *frame, const void *feat, const float *feat_scale,
+                            qr_dtype dtype, int32_t C, const int32_t *ids, const float *weights,
+                            const uint8_t *counts, const float *grad_out, void *grad_feat,
+                            qr_dtype grad_dtype, float *grad_opacity, float *grad_conic, void *ws,
+                            size_t ws_bytes, qr_stream stream) {
+    if (!frame_ok(frame) || !ids || !weights || !counts || !grad_out || !grad_feat || !ws ||
+        (grad_dtype != QR_F32 && grad_dtype != QR_BF16))
         return QR_ERR_INVALID_ARG;
     qr_status st = check_feat(feat, feat_scale, dtype, C);
     if (st != QR_OK) return st;
@@ -368,8 +369,17 @@ qr_status qr_backward(const qr_frame *frame, const void *feat, const float *feat
     if (ws_bytes < backward_workspace_bytes(*frame, C)) return QR_ERR_INVALID_ARG;
     if (frame->n == 0) return QR_OK;
     return from_cuda(launch_backward(*frame, feat, feat_scale, dtype, C, ids, weights, counts,
-                                     grad_out, grad_feat, grad_opacity, grad_conic, ws,
-                                     reinterpret_cast<cudaStream_t>(stream)));
+                                     grad_out, grad_feat, grad_dtype == QR_BF16, grad_opacity,
+                                     grad_conic, ws, reinterpret_cast<cudaStream_t>(stream)));
+}
+
+qr_status qr_backward(const qr_frame *frame, const void *feat, const float *feat_scale,
+                      qr_dtype dtype, int32_t C, const int32_t *ids, const float *weights,
+                      const uint8_t *counts, const float *grad_out, float *grad_feat,
+                      float *grad_opacity, float *grad_conic, void *ws, size_t ws_bytes,
+                      qr_stream stream) {
+    return qr_backward_typed(frame, feat, feat_scale, dtype, C, ids, weights, counts, grad_out,
+                             grad_feat, QR_F32, grad_opacity, grad_conic, ws, ws_bytes, stream);
 }
 
 size_t qr_cosine_backward_workspace_bytes(const qr_frame *frame, int32_t C) {
@@ -478,7 +488,7 @@ qr_status qr_contrastive_backward(const qr_frame *frame, const void *feat, const
     if (e != cudaSuccess) return QR_ERR_CUDA;
     if (frame->n == 0) return QR_OK;
     return from_cuda(launch_backward(*frame, feat, feat_scale, dtype, C, ids, weights, counts,
-                                     grad_map, grad_feat, grad_opacity, grad_conic, ws, s));
+                                     grad_map, grad_feat, false, grad_opacity, grad_conic, ws, s));
 }
 
 qr_status qr_blend_relevance(const void *feat, const float *feat_scale, qr_dtype dtype, int32_t C,

@@ -94,7 +94,7 @@ cudaError_t launch_select_rule(const qr_frame &f, int rule, int32_t *ids, float 
 size_t backward_workspace_bytes(const qr_frame &f, int C);
 cudaError_t launch_backward(const qr_frame &f, const void *feat, const float *scale, qr_dtype dt,
                             int C, const int32_t *ids, const float *w, const uint8_t *cnt,
-                            const float *grad_out, float *grad_feat, float *grad_alpha,
+                            const float *grad_out, void *grad_feat, bool bf16, float *grad_alpha,
                             float *grad_conic, void *ws, cudaStream_t s);
 cudaError_t launch_cosine_loss(const float *F, const float *tgt, const uint8_t *counts, int64_t P,
                                int C, float *term, float *out2, float *grad, cudaStream_t s);

@@ -102,6 +102,8 @@ SIGNATURES = {
     "qr_backward_workspace_bytes": (ctypes.c_size_t, [ctypes.POINTER(qr_frame), _I32]),
     "qr_backward": (_S, [ctypes.POINTER(qr_frame), _P, _P, _S, _I32, _P, _P, _P, _P, _P, _P, _P,
                          _P, ctypes.c_size_t, _P]),
+    "qr_backward_typed": (_S, [ctypes.POINTER(qr_frame), _P, _P, _S, _I32, _P, _P, _P, _P, _P, _S,
+                               _P, _P, _P, ctypes.c_size_t, _P]),
     "qr_cosine_loss": (_S, [_P, _P, _P, _I64, _I32, _P, _P, _P, _P]),
     "qr_cosine_backward_workspace_bytes": (ctypes.c_size_t, [ctypes.POINTER(qr_frame), _I32]),
     "qr_cosine_backward": (_S, [ctypes.POINTER(qr_frame), _P, _P, _S, _I32, _P, _P, _P, _P, _P,
@@ -361,11 +363,15 @@ def qr_render_noalloc(mean, log_scale, quat, opacity, cam, params, feat, feat_sc
 
 
 def qr_backward(fr: Frame, feat, feat_scale, ids, weights, counts, grad_out, want_conic=True,
-                stream=None):
+                stream=None, grad_dtype=None):
     """Gradients of the Q-Render forward of `fr` w.r.t. features, opacity and conic.
 
-    Returns (grad_feat [n, C] float32, grad_opacity [n], grad_conic [n, 3] or None)."""
+    Returns (grad_feat [n, C] float32 or, with grad_dtype=torch.bfloat16, rounded to it,
+    grad_opacity [n], grad_conic [n, 3] or None)."""
     torch = _torch()
+    grad_dtype = grad_dtype or torch.float32
+    if grad_dtype not in (torch.float32, torch.bfloat16):
+        raise TypeError(f"unsupported gradient dtype {grad_dtype}")
     n = int(fr.frame.n)
     C = feat.shape[1]
     dev = grad_out.device
@@ -374,13 +380,14 @@ def qr_backward(fr: Frame, feat, feat_scale, ids, weights, counts, grad_out, wan
         raise QRError(QR_ERR_INVALID_ARG, "qr_backward_workspace_bytes")
     ws = torch.empty(nbytes + 256, dtype=torch.uint8, device=dev)
     wsp = ctypes.c_void_p((ws.data_ptr() + 255) // 256 * 256)
-    gf = torch.empty((n, C), dtype=torch.float32, device=dev)
+    gf = torch.empty((n, C), dtype=grad_dtype, device=dev)
     ga = torch.empty(n, dtype=torch.float32, device=dev)
     gc = torch.empty((n, 3), dtype=torch.float32, device=dev) if want_conic else None
-    _check(load().qr_backward(ctypes.byref(fr.frame), _ptr(feat), _ptr(feat_scale),
-                              _dtype_code(feat), C, _ptr(ids), _ptr(weights), _ptr(counts),
-                              _ptr(grad_out.contiguous()), _ptr(gf), _ptr(ga), _ptr(gc), wsp,
-                              nbytes, _stream(stream)), "qr_backward")
+    _check(load().qr_backward_typed(ctypes.byref(fr.frame), _ptr(feat), _ptr(feat_scale),
+                                    _dtype_code(feat), C, _ptr(ids), _ptr(weights), _ptr(counts),
+                                    _ptr(grad_out.contiguous()), _ptr(gf), _dtype_code(gf),
+                                    _ptr(ga), _ptr(gc), wsp, nbytes, _stream(stream)),
+           "qr_backward")
     return gf, ga, gc
 
 

@@ -161,6 +161,23 @@ def test_backward_pixel_groups(kind, C, K):
     _check_all(got, ref)
 
 
+@pytest.mark.parametrize("C,K", [(64, 16), (136, 8), (512, 8)])
+def test_backward_bf16_gradient_is_the_rounded_one(C, K):
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=C)
+    cam = scenes.room_camera(61, 45)
+    table = q.qr_quantize_bf16(torch.from_numpy(f).cuda())
+    res = q.render_frame(q.gaussians_to_device(g), None, cam, K=K)
+    gout = torch.randn(cam.width * cam.height, C, device="cuda", generator=torch.Generator("cuda").manual_seed(2))
+    args = (res["frame"], table, None, res["ids"], res["weights"], res["counts"], gout)
+    wide, wa, wc = q.qr_backward(*args)
+    half, ha, hc = q.qr_backward(*args, grad_dtype=torch.bfloat16)
+    assert half.dtype == torch.bfloat16 and wide.abs().max() > 0
+    assert torch.equal(half, wide.to(torch.bfloat16))
+    assert torch.equal(ha, wa) and torch.equal(hc, wc)
+
+
 def test_backward_non_finite_gradient_stays_with_its_pixels():
     """An infinite upstream gradient reaches the Gaussians its pixel lists and
     no others; the rest is what it is without that pixel."""
