@@ -238,8 +238,8 @@ eq2_terms(const float *__restrict__ F, const float *__restrict__ tn, int M, int 
 // mma_tf32.cuh (mma.sync m16n8k8, FP32-class accuracy).
 
 // eq2_mma: M <= 16 MT targets.  One CTA per SM holds the unit targets split
-// into TF32 hi / lo parts in shared memory ([16 MT][C + 16] each; the row pad
-// makes the fragment loads conflict-free); each warp takes 16 pixels at a
+// into TF32 hi / lo parts in shared memory ([16 MT][C] each, 8-word
+// groups swizzled by row so that no fragment read conflicts); each warp takes 16 pixels at a
 // time (two 8-pixel n-tiles; g = lane / 4, t = lane % 4):
 //   1. S^T = T^ F^T (M = targets, N = pixels, K = channels): per 16
 //      channels a lane loads one float4 of each of its two pixel rows, the
@@ -255,9 +255,10 @@ eq2_terms(const float *__restrict__ F, const float *__restrict__ tn, int M, int 
 //      each 16 x 16 result, (G / nf - (sum_j c_j s_j) F / nf^2) / n, is
 //      written (streaming stores) with the F values it needs re-read (they
 //      were read moments before and come from L2).
-// Bound by shared-memory reads of T^ (68 %), issue (51 %) and the tensor pipe.
-// Room VGA, 512 channels, 32 patches: 531 us with 8-channel steps, 4-byte
-// fragment reads and the F values loaded one step ahead; 478 us now.
+// Bound by shared-memory reads of T^ (58 %), issue (55 %) and the tensor pipe.
+// Room VGA, 512 channels, 32 patches: 531 us with 8-channel gradient steps,
+// 4-byte fragment reads and the F values loaded one step ahead; 478 us with
+// 16-channel steps and 8-byte reads; 452 us with the swizzled rows.
 constexpr int kMmaThreads = 512;
 
 template <int MT>
@@ -271,16 +272,20 @@ eq2_mma(const float *__restrict__ F, const float *__restrict__ tn, int M, int C,
     constexpr int NPX = 8 * NT;            // pixels per warp block
     constexpr int MR = 16 * MT;            // target rows held
     extern __shared__ __align__(16) float s_t[];
-    const int S = C + 16;
+    const int S = C;
     float *s_hi = s_t, *s_lo = s_t + MR * S;
+    // channel c of target row j stands at c ^ swz(j): the 16-byte reads of rows
+    // g, g + 1 (similarities) and the 8-byte reads of rows t .. t + 3 (gradient)
+    // then fall in different banks
+    auto swz = [](int j) { return 16 * (j & 1) + 8 * ((j >> 1) & 1); };
     __shared__ float s_a1[NW][NPX], s_a2[NW][NPX];
     for (int i = threadIdx.x; i < MR * C; i += kMmaThreads) {
         const int j = i / C, c = i - j * C;
         const float x = j < M ? tn[int64_t(j) * C + c] : 0.f;
         uint32_t h, l;
         split_tf32(x, h, l);
-        s_hi[j * S + c] = __uint_as_float(h);
-        s_lo[j * S + c] = __uint_as_float(l);
+        s_hi[j * S + (c ^ swz(j))] = __uint_as_float(h);
+        s_lo[j * S + (c ^ swz(j))] = __uint_as_float(l);
     }
     __syncthreads();
     const float inv_n = cos_inv_count(out2);
@@ -320,12 +325,13 @@ eq2_mma(const float *__restrict__ F, const float *__restrict__ tn, int M, int C,
             // A fragments of every m-tile (rows g and g + 8, channels cg + 4t ..):
             // k-step 0 takes .x (slot t) and .y (slot t + 4), k-step 1 .z and .w
             uint32_t ah[MT][2][4], al[MT][2][4];
+            const int at = (cg + 4 * t) ^ swz(g);
 #pragma unroll
             for (int mt = 0; mt < MT; ++mt) {
-                const float4 h0 = *reinterpret_cast<const float4 *>(s_hi + (16 * mt + g) * S + cg + 4 * t);
-                const float4 h1 = *reinterpret_cast<const float4 *>(s_hi + (16 * mt + g + 8) * S + cg + 4 * t);
-                const float4 l0 = *reinterpret_cast<const float4 *>(s_lo + (16 * mt + g) * S + cg + 4 * t);
-                const float4 l1 = *reinterpret_cast<const float4 *>(s_lo + (16 * mt + g + 8) * S + cg + 4 * t);
+                const float4 h0 = *reinterpret_cast<const float4 *>(s_hi + (16 * mt + g) * S + at);
+                const float4 h1 = *reinterpret_cast<const float4 *>(s_hi + (16 * mt + g + 8) * S + at);
+                const float4 l0 = *reinterpret_cast<const float4 *>(s_lo + (16 * mt + g) * S + at);
+                const float4 l1 = *reinterpret_cast<const float4 *>(s_lo + (16 * mt + g + 8) * S + at);
                 ah[mt][0][0] = __float_as_uint(h0.x); ah[mt][0][1] = __float_as_uint(h1.x);
                 ah[mt][0][2] = __float_as_uint(h0.y); ah[mt][0][3] = __float_as_uint(h1.y);
                 ah[mt][1][0] = __float_as_uint(h0.z); ah[mt][1][1] = __float_as_uint(h1.z);
@@ -457,7 +463,7 @@ eq2_mma(const float *__restrict__ F, const float *__restrict__ tn, int M, int C,
                 float d[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
                 for (int kk = 0; kk < 2 * MT; ++kk) {
-                    const int r0 = (8 * kk + t) * S + c0 + 2 * g, r1 = r0 + 4 * S;
+                    const int r0 = (8 * kk + t) * S + ((c0 + 2 * g) ^ swz(t)), r1 = r0 + 4 * S;
                     const float2 h0 = *reinterpret_cast<const float2 *>(s_hi + r0);
                     const float2 h1 = *reinterpret_cast<const float2 *>(s_hi + r1);
                     const float2 l0 = *reinterpret_cast<const float2 *>(s_lo + r0);
@@ -524,8 +530,8 @@ cudaError_t launch_contrastive_loss(const float *F, const float *tgt, int M, int
         return cudaGetLastError();
     };
     if (M <= 32) {
-        // tensor cores: the unit targets split into TF32 hi / lo rows of C + 16
-        const size_t dyn2 = size_t(2) * (M <= 16 ? 16 : 32) * size_t(C + 16) * 4;
+        // tensor cores: the unit targets split into TF32 hi / lo rows
+        const size_t dyn2 = size_t(2) * (M <= 16 ? 16 : 32) * size_t(C) * 4;
         e = M <= 16 ? go(eq2_mma<1>, dyn2, kMmaThreads) : go(eq2_mma<2>, dyn2, kMmaThreads);
     } else {
         const size_t dyn = size_t(M) * C * 4;
