@@ -125,13 +125,25 @@ __device__ __forceinline__ void slot_owner(const ExpandSmem &sm, uint32_t len, u
 // array itself.  Rows are summed by one warp each (shuffle scans), columns by
 // one thread each.  Partial sums may be negative; the uint32 arithmetic is
 // exact modulo 2^32 and the integrated counts are not.
-__global__ void __launch_bounds__(1024)
+__global__ void __launch_bounds__(1024, 1)
 bin_scan(uint32_t *kept, uint32_t *tsum, int nblk, uint32_t *counters, uint32_t capacity,
          const int *__restrict__ diff, uint32_t *tcnt, int tiles_x, int tiles_y, uint2 *ranges,
          int in_smem) {
     pdl_wait();   // the predecessor's outputs are complete and visible
     extern __shared__ uint32_t s_cnt[];
     __shared__ uint32_t s_w[64];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+    const int stride = tiles_x + 1;
+    const int tiles = tiles_x * tiles_y;
+    // the warp's first row of the difference arrays (64 columns of it) is loaded
+    // ahead of the scans that do not need it
+    int ahead[2][kDiffCopies];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int r = 0; r < kDiffCopies; ++r)
+            ahead[h][r] = warp < tiles_y && lane + 32 * h < tiles_x
+                              ? diff[size_t(r) * stride * (tiles_y + 1) + warp * stride + lane + 32 * h] : 0;
     // both per-block scans in one pass, each thread owning `per` consecutive blocks
     const int per = (nblk + int(blockDim.x) - 1) / int(blockDim.x);
     const int b0 = int(threadIdx.x) * per;
@@ -162,8 +174,6 @@ bin_scan(uint32_t *kept, uint32_t *tsum, int nblk, uint32_t *counters, uint32_t 
         if (over) counters[CNT_STATUS] = QR_ERR_CAPACITY;
         counters[CNT_SORT_N] = over ? 0u : isect;
     }
-    const int stride = tiles_x + 1;
-    const int tiles = tiles_x * tiles_y;
     if (over) {   // capacity exceeded: every tile list is empty
         for (int t = threadIdx.x; t < tiles; t += blockDim.x) {
             ranges[t] = make_uint2(0u, 0u);
@@ -172,16 +182,19 @@ bin_scan(uint32_t *kept, uint32_t *tsum, int nblk, uint32_t *counters, uint32_t 
         return;
     }
     uint32_t *A = in_smem ? s_cnt : tcnt;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
     for (int y = warp; y < tiles_y; y += nwarps) {
         uint32_t carry = 0;
         for (int x0 = 0; x0 < tiles_x; x0 += 32) {
             const int x = x0 + lane;
             uint32_t v = 0u;
-            if (x < tiles_x)
+            if (y == warp && x0 < 64) {
+#pragma unroll
+                for (int r = 0; r < kDiffCopies; ++r) v += uint32_t(x0 == 0 ? ahead[0][r] : ahead[1][r]);
+            } else if (x < tiles_x) {
 #pragma unroll
                 for (int r = 0; r < kDiffCopies; ++r)
                     v += uint32_t(diff[size_t(r) * stride * (tiles_y + 1) + y * stride + x]);
+            }
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
                 const uint32_t t = __shfl_up_sync(0xffffffffu, v, o);
@@ -194,20 +207,29 @@ bin_scan(uint32_t *kept, uint32_t *tsum, int nblk, uint32_t *counters, uint32_t 
     __syncthreads();
     for (int x = threadIdx.x; x < tiles_x; x += blockDim.x) {
         uint32_t run = 0;
-        for (int y = 0; y < tiles_y; ++y) {
-            run += A[y * tiles_x + x];
-            A[y * tiles_x + x] = run;
+        for (int y0 = 0; y0 < tiles_y; y0 += 8) {   // eight reads at a time
+            uint32_t v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = y0 + i < tiles_y ? A[(y0 + i) * tiles_x + x] : 0u;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                run += v[i];
+                if (y0 + i < tiles_y) A[(y0 + i) * tiles_x + x] = run;
+            }
         }
     }
     __syncthreads();
-    uint32_t carry = 0;
-    for (int base = 0; base < tiles; base += blockDim.x) {
-        const int t = base + threadIdx.x;
-        const uint32_t c = t < tiles ? A[t] : 0u;
-        uint32_t chunk;
-        const uint32_t inc = block_inclusive_scan(c, s_w, chunk);
-        if (t < tiles) ranges[t] = make_uint2(carry + inc - c, carry + inc);
-        carry += chunk;
+    // exclusive offsets, each thread owning `mine` consecutive tiles
+    const int mine = (tiles + int(blockDim.x) - 1) / int(blockDim.x);
+    const int t0 = min(tiles, int(threadIdx.x) * mine), t1 = min(tiles, t0 + mine);
+    uint32_t sum = 0;
+    for (int t = t0; t < t1; ++t) sum += A[t];
+    uint32_t all;
+    uint32_t at = block_inclusive_scan(sum, s_w, all) - sum;
+    for (int t = t0; t < t1; ++t) {
+        const uint32_t c = A[t];
+        ranges[t] = make_uint2(at, at + c);
+        at += c;
     }
     __syncthreads();
     for (int t = threadIdx.x; t < tiles; t += blockDim.x) tcnt[t] = 0u;
