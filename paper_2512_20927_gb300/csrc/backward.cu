@@ -108,6 +108,21 @@ __device__ __forceinline__ float reduce4(float (&v)[4], int lane) {
 }
 __device__ __forceinline__ int red4_lane(int u) { return ((u >> 1) << 4) | ((u & 1) << 3); }
 
+// acc += (x0, x1) * g for both halves
+__device__ __forceinline__ void fma2x(float2 &acc, float x0, float x1, float2 g) {
+    asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %3};\n"
+        " mov.b64 xx, {%4, %5};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
+        : "+f"(acc.x), "+f"(acc.y) : "f"(x0), "f"(x1), "f"(g.x), "f"(g.y));
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float b) {
+    float2 d;
+    asm("{\n .reg .b64 x, y;\n mov.b64 x, {%2, %3};\n mov.b64 y, {%4, %4};\n"
+        " mul.rn.f32x2 x, x, y;\n mov.b64 {%0, %1}, x;\n}\n"
+        : "=f"(d.x), "=f"(d.y) : "f"(a.x), "f"(a.y), "f"(b));
+    return d;
+}
+
 template <int DT, int VPL, bool LOSS>
 __global__ void __launch_bounds__(T)
 bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
@@ -136,7 +151,7 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
             // outside the mask), as the loss's own pass computes them
             const bool on = loss.mask[p] > 0;
             float tr[VPL > 0 ? VPL : 1][CPV];
-            float dot = 0.f, ff = 0.f, tt = 0.f;
+            float2 dot2 = make_float2(0.f, 0.f), ff2 = dot2, tt2 = dot2;
 #pragma unroll
             for (int t = 0; t < VPL; ++t) {
                 const float4 *fv = reinterpret_cast<const float4 *>(loss.F + p * int64_t(C) + (lane + 32 * t) * CPV);
@@ -151,13 +166,15 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 #pragma unroll
             for (int t = 0; t < VPL; ++t)
 #pragma unroll
-                for (int q = 0; q < CPV; ++q) {
-                    dot = fmaf(gr[t][q], tr[t][q], dot);
-                    ff = fmaf(gr[t][q], gr[t][q], ff);
-                    tt = fmaf(tr[t][q], tr[t][q], tt);
+                for (int q = 0; q < CPV; q += 2) {
+                    const float2 a = make_float2(gr[t][q], gr[t][q + 1]), b = make_float2(tr[t][q], tr[t][q + 1]);
+                    fma2x(dot2, a.x, a.y, b);
+                    fma2x(ff2, a.x, a.y, a);
+                    fma2x(tt2, b.x, b.y, b);
                 }
+            float dot, ff, tt;
             {
-                float v4[4] = {dot, ff, tt, 0.f};
+                float v4[4] = {dot2.x + dot2.y, ff2.x + ff2.y, tt2.x + tt2.y, 0.f};
                 const float x = reduce4(v4, lane);
                 dot = __shfl_sync(FULL, x, red4_lane(0));
                 ff = __shfl_sync(FULL, x, red4_lane(1));
@@ -168,8 +185,14 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 #pragma unroll
             for (int t = 0; t < VPL; ++t) {
 #pragma unroll
-                for (int q = 0; q < CPV; ++q)
-                    gr[t][q] = on ? -(tr[t][q] * cc.k1 - gr[t][q] * cc.k2) * inv_n : 0.f;
+                for (int q = 0; q < CPV; q += 2) {
+                    // (F k2 - t k1) / n
+                    float2 x = mul2(make_float2(gr[t][q], gr[t][q + 1]), cc.k2);
+                    fma2x(x, -cc.k1, -cc.k1, make_float2(tr[t][q], tr[t][q + 1]));
+                    x = mul2(x, inv_n);
+                    gr[t][q] = on ? x.x : 0.f;
+                    gr[t][q + 1] = on ? x.y : 0.f;
+                }
                 float4 *gv = reinterpret_cast<float4 *>(g + (lane + 32 * t) * CPV);
 #pragma unroll
                 for (int q = 0; q < CPV / 4; ++q)
@@ -210,14 +233,16 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
                 float part[4];
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
-                    part[u] = 0.f;
+                    float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
                     for (int t = 0; t < VPL; ++t) {
                         float fv[CPV];
                         widen<DT>(rv[u][t], fv);
 #pragma unroll
-                        for (int q = 0; q < CPV; ++q) part[u] = fmaf(fv[q], gr[t][q], part[u]);
+                        for (int q = 0; q < CPV; q += 2)
+                            fma2x(sum, fv[q], fv[q + 1], make_float2(gr[t][q], gr[t][q + 1]));
                     }
+                    part[u] = sum.x + sum.y;
                 }
                 // lane j0 + u takes row u's dot from a lane that holds it
                 const float x = reduce4(part, lane);
@@ -287,13 +312,6 @@ bwd_pixel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
             E[p * K + lane] = e;
         }
     }
-}
-
-// acc += (x0, x1) * g for both halves
-__device__ __forceinline__ void fma2x(float2 &acc, float x0, float x1, float2 g) {
-    asm("{\n .reg .b64 a, ww, xx;\n mov.b64 a, {%0, %1};\n mov.b64 ww, {%2, %3};\n"
-        " mov.b64 xx, {%4, %5};\n fma.rn.f32x2 a, ww, xx, a;\n mov.b64 {%0, %1}, a;\n}\n"
-        : "+f"(acc.x), "+f"(acc.y) : "f"(x0), "f"(x1), "f"(g.x), "f"(g.y));
 }
 
 // The same without the loss, for K <= 8 and rows of up to 512 channels, a warp per 2 x 2 pixels:
