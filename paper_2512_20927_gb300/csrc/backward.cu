@@ -1047,14 +1047,13 @@ cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scal
         case QR_BF16: launch_bwd_pixel<QR_BF16>(f, feat, scale, C, ids, w, cnt, g, E, loss, s); break;
         case QR_FP8E4M3: launch_bwd_pixel<QR_FP8E4M3>(f, feat, scale, C, ids, w, cnt, g, E, loss, s); break;
     }
-    if (loss) {
-        e = cudaGetLastError();
-        if (e == cudaSuccess) e = launch_cos_final(loss->term, num_pixels(f), loss->out2, s);
-        if (e != cudaSuccess) return e;
-    }
-    // rows of Gaussians that no tile selects are zero: clear the outputs on the
-    // side stream, overlapping the tile kernel (which is not bandwidth-bound),
-    // and join before the rows are written; without a side stream, in order
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    // Beside the tile kernel, on the side stream: the final sum of the loss,
+    // which nothing here reads, and the clearing of the outputs (rows of
+    // Gaussians that no tile selects are zero; the tile kernel is not
+    // bandwidth-bound).  It joins before the rows are written, then takes half
+    // of them.  Without a side stream all of it runs in order.
     cudaStream_t side = side_stream();
     cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     if (side && (cudaEventCreateWithFlags(&ev_fork, cudaEventDisableTiming) != cudaSuccess ||
@@ -1063,30 +1062,32 @@ cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scal
         ev_fork = nullptr;
         side = nullptr;
     }
-    cudaStream_t zs = s;
-    if (side) {
-        e = cudaEventRecord(ev_fork, s);
-        if (e == cudaSuccess) e = cudaStreamWaitEvent(side, ev_fork, 0);
-        if (e != cudaSuccess) {
-            cudaEventDestroy(ev_fork);
-            cudaEventDestroy(ev_join);
-            return e;
-        }
-        zs = side;
-    }
-    e = cudaMemsetAsync(grad_feat, 0, size_t(f.n) * size_t(C) * (bf16 ? 2 : 4), zs);
-    if (e == cudaSuccess && grad_alpha) e = cudaMemsetAsync(grad_alpha, 0, size_t(f.n) * 4, zs);
-    if (e == cudaSuccess && grad_conic) e = cudaMemsetAsync(grad_conic, 0, size_t(f.n) * 12, zs);
+    const cudaStream_t zs = side ? side : s;
+    auto fork = [&]() -> cudaError_t {
+        if (!side) return cudaSuccess;
+        const cudaError_t ef = cudaEventRecord(ev_fork, s);
+        return ef != cudaSuccess ? ef : cudaStreamWaitEvent(side, ev_fork, 0);
+    };
     // the side stream joins the caller's stream again (also on an error path)
     auto join = [&](cudaError_t err) {
         if (!side) return err;
         cudaError_t ej = cudaEventRecord(ev_join, side);
         if (ej == cudaSuccess) ej = cudaStreamWaitEvent(s, ev_join, 0);
-        cudaEventDestroy(ev_fork);
-        cudaEventDestroy(ev_join);
-        side = nullptr;
         return err != cudaSuccess ? err : ej;
     };
+    struct Events {   // released on every way out (work that waits on them keeps what it needs)
+        cudaEvent_t &a, &b;
+        ~Events() {
+            if (a) cudaEventDestroy(a);
+            if (b) cudaEventDestroy(b);
+        }
+    } events{ev_fork, ev_join};
+    e = fork();
+    if (e != cudaSuccess) return e;
+    if (loss) e = launch_cos_final(loss->term, num_pixels(f), loss->out2, zs);
+    if (e == cudaSuccess) e = cudaMemsetAsync(grad_feat, 0, size_t(f.n) * size_t(C) * (bf16 ? 2 : 4), zs);
+    if (e == cudaSuccess && grad_alpha) e = cudaMemsetAsync(grad_alpha, 0, size_t(f.n) * 4, zs);
+    if (e == cudaSuccess && grad_conic) e = cudaMemsetAsync(grad_conic, 0, size_t(f.n) * 12, zs);
     if (e != cudaSuccess) return join(e);
     // per-tile partials; for K <= 8 the tile's rows of g are staged by TMA
     // (3-D boxes {64 channels, tile_w pixels, tile_h rows} of the [H][W][C]
@@ -1139,22 +1140,24 @@ cudaError_t backward_impl(const qr_frame &f, const void *feat, const float *scal
                    : tp(bwd_tile_partials<0, unsigned long long>);
     }
     e = join(e);
+    if (e == cudaSuccess) e = fork();
     if (e != cudaSuccess) return e;
-    // the selected Gaussians' rows in tile order, over the cleared outputs
+    // the selected Gaussians' rows in tile order, over the cleared outputs:
+    // those of many tiles on the side stream, beside the others
     const uint32_t *tcount = slot<uint32_t>(f, S_TCOUNT);
     auto rows = [&](auto zero) {
         using G = decltype(zero);
         bwd_rows<256, G><<<unsigned(sms_now() * 8), 256, 0, s>>>(
             lists, lists + 2 * f.n, goff, tcount, slotmap, f.max_isect, partial, partial_s, C,
             static_cast<G *>(grad_feat), grad_alpha, grad_conic);
-        bwd_rows<1024, G><<<unsigned(sms_now() * 2), 1024, 0, s>>>(
+        bwd_rows<1024, G><<<unsigned(sms_now() * 2), 1024, 0, zs>>>(
             lists + f.n, lists + 2 * f.n + 1, goff, tcount, slotmap, f.max_isect, partial, partial_s,
             C, static_cast<G *>(grad_feat), grad_alpha, grad_conic);
     };
     if (bf16) rows(uint16_t(0));
     else rows(0.f);
     count_launch(5);
-    return cudaGetLastError();
+    return join(cudaGetLastError());
 }
 
 }  // namespace
