@@ -204,30 +204,12 @@ blend_kernel(const uint4 *__restrict__ feat, const float *__restrict__ scale, in
     }
 }
 
-// Wide rows (one warp per row): a warp owns a group of G neighbouring pixels
-// (2x2 for G = 4, 2x1 for G = 2) whose selections are subsequences of the same
-// tile list and mostly share rows.  Lane g*K + j holds entry j of pixel g;
-// __match_any_sync groups equal ids and each distinct row is loaded once and
+// Wide rows (one warp per row): a warp owns a group of G = 4 (2x2) neighbouring
+// pixels whose selections are subsequences of the same tile list and mostly
+// share rows.  __match_any_sync groups equal ids and each distinct row is loaded once and
 // accumulated into every pixel of the group with that pixel's weight (zero
 // weights are skipped).  L1 row traffic drops from sum(counts) to the number
 // of distinct rows of the group.
-template <int G>
-__device__ __forceinline__ int64_t group_pixel(int64_t chunk0, int gi, int m, int W, int H,
-                                               int64_t items) {
-    int r;
-    if (G == 4) {
-        const int qx = gi & 7, qy = gi >> 3;
-        r = (2 * qy + (m >> 1)) * 16 + 2 * qx + (m & 1);
-    } else if (G == 2) {
-        r = (gi >> 3) * 16 + 2 * (gi & 7) + m;
-    } else {
-        r = gi;
-    }
-    const int64_t item = chunk0 + r;
-    if (item >= items) return -1;
-    return tile_order_pixel(item, W, H);
-}
-
 // The G weights of each distinct row are gathered once into a shared-memory
 // table (slot = rank of the row's leader lane, one float per pixel; a pixel
 // that lists an id twice gets the sum), so the row loop reads them with one
@@ -242,7 +224,14 @@ __device__ __forceinline__ int64_t group_pixel(int64_t chunk0, int gi, int m, in
 // the row's weights, so no load waits on another's result.  An FP8 row's
 // weight for a pixel is (the pixel's weight for it) * scale, rounded once: a
 // selection lists a Gaussian at most once per pixel.
-template <int DT, int QPL, int G, int NCH>
+// EPL of the group's 4 K entries per lane: 1 for K <= 8, 2 for K <= 16, 4 above;
+// lane l holds entries l, l + 32, ... (pixel e / K, entry e % K), and each
+// further set looks its ids up among the rows of the sets before it.
+// Measured (groups of 4 pixels for K <= 8, 2 for K <= 16, 1 above -> 4 for every
+// K, the tile's origin worked out once; us, 512 FP32 channels): room VGA K = 8
+// 120 -> 115, K = 16 191 -> 163, K = 32 380 -> 244; object VGA K = 16 246 -> 234, K =
+// 32 412 -> 351; 256 BF16 channels, room VGA, K = 16 108 -> 109, K = 32 222 -> 187.
+template <int DT, int QPL, int NCH, int EPL>
 __global__ void __launch_bounds__(kThreads)
 blend_group_kernel(const unsigned char *__restrict__ feat, const float *__restrict__ scale,
                    int64_t n_gauss, const int32_t *__restrict__ ids,
@@ -255,17 +244,24 @@ blend_group_kernel(const unsigned char *__restrict__ feat, const float *__restri
     constexpr int U = (QPL * QB >= 64) ? 2 : (QPL * QB >= 32 ? 128 / (QPL * QB) : 4);
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int NW = kThreads / 32;
+    constexpr int G = 4;                     // pixels of a group
     constexpr int NITEMS = (256 / G) * NCH;
-    __shared__ __align__(16) float s_w[NW][32][G];
-    __shared__ int s_id[NW][32];
+    __shared__ __align__(16) float s_w[NW][32 * EPL][G];
+    __shared__ int s_id[NW][32 * EPL];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t items = (W > 0) ? int64_t((W + 15) >> 4) * ((H + 15) >> 4) * 256 : P;
     const int64_t chunk0 = int64_t(blockIdx.x) * 256;
-    const int m = lane / K, j = lane - m * K;
-    auto fetch = [&](int gi, int64_t &p, int &idr, float &wr, int &c) {
-        p = -1;
-        if (m < G) p = (W > 0) ? group_pixel<G>(chunk0, gi, m, W, H, items)
-                               : (chunk0 + gi * G + m < items ? chunk0 + gi * G + m : -1);
+    const int tiles_x = (W + 15) >> 4;
+    const int tx0 = W > 0 ? int(blockIdx.x) % tiles_x * 16 : 0, ty0 = W > 0 ? int(blockIdx.x) / tiles_x * 16 : 0;
+    // pixel m of group gi of this CTA's 16x16 tile (or 256 consecutive pixels)
+    auto pixel = [&](int gi, int m) -> int64_t {
+        if (W <= 0) return chunk0 + gi * G + m < P ? chunk0 + gi * G + m : -1;
+        const int x = tx0 + 2 * (gi & 7) + (m & 1), y = ty0 + 2 * (gi >> 3) + (m >> 1);
+        return x < W && y < H ? int64_t(y) * W + x : -1;
+    };
+    // entry e of the group: raw values by three independent loads
+    auto fetch = [&](int gi, int e, int &idr, float &wr, int &c) {
+        const int m = e / K, j = e - m * K;
+        const int64_t p = m < G ? pixel(gi, m) : -1;
         idr = -1;
         wr = 0.f;
         c = 0;
@@ -275,30 +271,48 @@ blend_group_kernel(const unsigned char *__restrict__ feat, const float *__restri
             wr = wts[p * K + j];
         }
     };
-    int64_t p;
-    int idr, c;
-    float wr;
-    fetch(warp / NCH, p, idr, wr, c);
+    int idr[EPL], c[EPL];
+    float wr[EPL];
+    if constexpr (EPL == 1) fetch(warp / NCH, lane, idr[0], wr[0], c[0]);
     for (int it = warp; it < NITEMS; it += NW) {
-        const int ch = it % NCH;
-        const bool ok = p >= 0 && j < c && uint64_t(int64_t(idr)) < uint64_t(n_gauss);
-        const int id = ok ? idr : -1;
-        const float w = ok ? wr : 0.f;
-        const int64_t pc = p;
-        if (it + NW < NITEMS) fetch((it + NW) / NCH, p, idr, wr, c);
-        const unsigned peers = __match_any_sync(FULL, id);
-        const int leader = __ffs(peers) - 1;
-        const unsigned leaders = __ballot_sync(FULL, id >= 0 && lane == leader);
-        const int nrows = __popc(leaders);
+        const int ch = it % NCH, gi = it / NCH;
+        if constexpr (EPL > 1) {
 #pragma unroll
-        for (int g = 0; g < G; ++g) s_w[warp][lane][g] = 0.f;
-        __syncwarp();
-        if (id >= 0) {
-            const int slot = __popc(leaders & ((1u << leader) - 1u));
-            atomicAdd(&s_w[warp][slot][m], w);   // m < G for every listed entry
-            if (lane == leader) s_id[warp][slot] = id;
+            for (int h = 0; h < EPL; ++h) fetch(gi, lane + 32 * h, idr[h], wr[h], c[h]);
         }
+        int id[EPL];
+        float w[EPL];
+#pragma unroll
+        for (int h = 0; h < EPL; ++h) {
+            const bool ok = (lane + 32 * h) % K < c[h] && uint64_t(int64_t(idr[h])) < uint64_t(n_gauss);
+            id[h] = ok ? idr[h] : -1;
+            w[h] = ok ? wr[h] : 0.f;
+        }
+        if constexpr (EPL == 1)   // the next item's entries, before this one's rows
+            if (it + NW < NITEMS) fetch((it + NW) / NCH, lane, idr[0], wr[0], c[0]);
+#pragma unroll
+        for (int h = 0; h < EPL; ++h)
+#pragma unroll
+            for (int g = 0; g < G; ++g) s_w[warp][lane + 32 * h][g] = 0.f;
         __syncwarp();
+        int nrows = 0;
+#pragma unroll
+        for (int h = 0; h < EPL; ++h) {
+            int slot = -1;
+            if (h > 0)
+                for (int k = 0; k < nrows; ++k)
+                    if (s_id[warp][k] == id[h]) slot = k;
+            const unsigned peers = __match_any_sync(FULL, id[h]);
+            const int leader = __ffs(peers) - 1;
+            const unsigned fresh = __ballot_sync(FULL, id[h] >= 0 && slot < 0 && lane == leader);
+            if (slot < 0) slot = nrows + __popc(fresh & ((1u << leader) - 1u));
+            if (id[h] >= 0) {
+                atomicAdd(&s_w[warp][slot][(lane + 32 * h) / K], w[h]);   // pixel < G for every listed entry
+                if ((fresh >> lane) & 1u) s_id[warp][slot] = id[h];
+            }
+            nrows += __popc(fresh);
+            __syncwarp();
+        }
         float acc[G][QPL][4];
 #pragma unroll
         for (int g = 0; g < G; ++g)
@@ -340,7 +354,7 @@ blend_group_kernel(const unsigned char *__restrict__ feat, const float *__restri
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int64_t pg = __shfl_sync(FULL, pc, g * K < 32 ? g * K : 0);
+            const int64_t pg = pixel(gi, g);
             if (pg >= 0) {
                 float4 *o = out + pg * int64_t(ROWQ) + ch * CQ + lane;
 #pragma unroll
@@ -362,13 +376,13 @@ constexpr int default_chunks() {
 
 int g_blend_chunks = 0;   // qr_set_blend_chunks: 0 = default_chunks
 
-template <int DT, int QT, int G, int NCH>
+template <int DT, int QT, int NCH, int EPL>
 cudaError_t go_group(const void *feat, const float *scale, int64_t n_gauss, const int32_t *ids,
                      const float *w, const uint8_t *cnt, int64_t P, int K, int W, int H,
                      float *out, cudaStream_t s) {
     const int64_t items = (W > 0) ? int64_t((W + 15) >> 4) * ((H + 15) >> 4) * 256 : P;
     const unsigned blocks = unsigned((items + 255) / 256);
-    return pdl_launch(blend_group_kernel<DT, QT / NCH, G, NCH>, dim3(blocks), dim3(kThreads), 0, s,
+    return pdl_launch(blend_group_kernel<DT, QT / NCH, NCH, EPL>, dim3(blocks), dim3(kThreads), 0, s,
                       static_cast<const unsigned char *>(feat), scale, n_gauss, ids, w, cnt, P, K,
                       W, H, reinterpret_cast<float4 *>(out));
 }
@@ -387,18 +401,18 @@ cudaError_t run_group(const void *feat, const float *scale, int64_t n_gauss, con
         const int want = g_blend_chunks > 0 ? g_blend_chunks : DEF;
         if constexpr (QT == 4) {
             if (want == 2)
-                e = go_group<DT, QT, 4, 2>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
+                e = go_group<DT, QT, 2, 1>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
             else if (want == 4)
-                e = go_group<DT, QT, 4, 4>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
-            else
                 e = go_group<DT, QT, 4, 1>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
+            else
+                e = go_group<DT, QT, 1, 1>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
         } else {
-            e = go_group<DT, QT, 4, DEF>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
+            e = go_group<DT, QT, DEF, 1>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
         }
     } else if (K <= 16) {
-        e = go_group<DT, QT, 2, DEF>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
+        e = go_group<DT, QT, DEF, 2>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
     } else {
-        e = go_group<DT, QT, 1, DEF>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
+        e = go_group<DT, QT, DEF, 4>(feat, scale, n_gauss, ids, w, cnt, P, K, W, H, out, s);
     }
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();

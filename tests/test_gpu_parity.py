@@ -505,6 +505,32 @@ def test_blend_channel_chunks_bit_identical(dtype, C):
         q.qr_set_blend_chunks(3)
 
 
+@pytest.mark.parametrize("K,C,dtype,width", [(8, 512, "f32", 67), (9, 512, "bf16", 67), (16, 128, "f32", 0),
+                                             (16, 512, "fp8", 67), (17, 256, "f32", 67), (32, 512, "f32", 0)])
+def test_blend_of_many_entries_per_group(K, C, dtype, width):
+    """Pixel groups whose entries fill one, two and four sets of a warp's lanes,
+    partly listed, on an image with cut groups and as consecutive pixels."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    rng = np.random.default_rng(K + C)
+    n, P = 60, 67 * 35
+    f = rng.normal(size=(n, C)).astype(np.float32)
+    ids, w, cnt = scenes.random_selection(seed=K, pixels=P, k=K, n=n)
+    fdev = torch.from_numpy(f).cuda()
+    table, scale, fdec = fdev, None, f.astype(np.float64)
+    if dtype == "bf16":
+        table, fdec = q.qr_quantize_bf16(fdev), oracle.bf16_decode(oracle.bf16_encode(f))
+    elif dtype == "fp8":
+        (table, scale), fdec = q.qr_quantize_fp8(fdev), oracle.fp8_dequantize_rows(*oracle.fp8_quantize_rows(f))
+    out = torch.full((P, C), float("nan"), device="cuda")
+    q.qr_blend(table, scale, *(torch.from_numpy(a).cuda() for a in (ids, w, cnt)), out, width=width)
+    torch.cuda.synchronize()
+    want = compare.blend(ids, w, cnt, fdec)
+    mag = compare.blend(ids, np.abs(w), cnt, np.abs(fdec))
+    # K products and sums in FP32 (and the FP8 scale folded into the weight)
+    assert (np.abs(out.cpu().numpy() - want) <= (K + 2) * 2.0 ** -23 * mag + 1e-30).all()
+
+
 @pytest.mark.parametrize("w,h,K,tile", [(1, 1, 8, (16, 16)), (7, 9, 3, (16, 16)),
                                         (9, 17, 4, (32, 8)), (33, 8, 12, (8, 32)),
                                         (16, 31, 32, (32, 8)), (50, 23, 8, (8, 32))])
