@@ -31,7 +31,8 @@
 //     than the smallest kept weight, no later entry can enter (T only falls
 //     and alpha' <= alpha_max), so the pixel stops early without changing the
 //     result.  Shared-memory slots with a replaced minimum, two pixels per
-//     lane, took 238 us where this takes 187 (below).
+//     lane, took 238 us where this takes 187 (below).  With many entries the
+//     insertions cost more than a search of slots: topk_tile_kernel.
 //   * Stratified-K sums T and T^2 in compensated double-FP32 arithmetic, both
 //     pixels of a lane in one packed FP32x2 instruction stream (adding an
 //     exact 0 where an entry is no member) and four entries at a time, forms
@@ -48,6 +49,11 @@ namespace qr {
 namespace {
 
 enum { kTopK = 1, kStratified = 2 };
+
+// 8 x 8 blocks up to which, and list capacity per tile from which, latency
+// rather than issue bounds top-K's walk
+constexpr int kFewBlocks = 152 * 8;
+constexpr int64_t kLongTopLists = 768;
 
 // ------------------------------------------------------------------ top-K
 constexpr int kTopPix = 32;        // pixels per warp: 8 x 4, one per lane
@@ -141,7 +147,7 @@ __device__ __forceinline__ BlockAt block_at(int block, int tile_w, int tiles_x) 
 // entry that some pixel of the warp may keep costs the warp one top_insert,
 // the others a vote.
 template <int KT>
-__global__ void __launch_bounds__(32, KT > 16 ? 16 : 24)
+__global__ void __launch_bounds__(32, 24)
 topk_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
             const float *__restrict__ rec_a, const float *__restrict__ rec_h,
             const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
@@ -209,6 +215,171 @@ topk_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
     store_slots<1>(W, H, at.x0, at.y0, K, vec != 0, reinterpret_cast<const int32_t *>(s_key), ids);
     store_slots<1>(W, H, at.x0, at.y0, K, vec != 0, (const float *)s_w, wout);
     if (inside) cnt[int64_t(py) * W + px] = uint8_t(m);
+}
+
+// ------------------------------------------------------------------ top-K, many entries
+// One CTA per screen tile, one pixel per thread: the list is staged 256 records
+// at a time and culled per warp, and a pixel's candidates sit in shared-memory
+// slots whose smallest a replacement searches again.  With more entries an
+// insertion into sorted registers costs more than that search, unless latency
+// bounds the walk.
+constexpr int kPix = 256;
+constexpr int kThreads = 256;
+constexpr int kTileBatch = 256;
+
+struct Stage {
+    float4 *m, *c;
+    float *a, *h;
+};
+
+// Walks the tile's list for this thread's pixel: stages records, culls them
+// per warp against the warp's pixel box and calls visit(pos, alpha') for
+// every member entry (alpha' >= alpha_min) in list order until the pixel is
+// done.  visit returns true when the pixel has finished its walk.  All
+// threads of the CTA must call it.
+template <typename Visit>
+__device__ __forceinline__ void walk_list(const float4 *__restrict__ rec_m,
+                                          const float4 *__restrict__ rec_w,
+                                          const float *__restrict__ rec_a,
+                                          const float *__restrict__ rec_h,
+                                          const uint32_t *__restrict__ isect_gid, uint2 range,
+                                          const Stage &st, float ux, float uy, float bx0,
+                                          float bx1, float by0, float by1, float alpha_min,
+                                          float alpha_max, bool &done, Visit visit) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    for (uint32_t b = range.x; b < range.y; b += kTileBatch) {
+        if (__syncthreads_count(done) == kThreads) break;
+        if (b + threadIdx.x < range.y) {
+            const uint32_t g = isect_gid[b + threadIdx.x];
+            st.m[threadIdx.x] = rec_m[g];
+            st.c[threadIdx.x] = rec_w[g];
+            st.a[threadIdx.x] = rec_a[g];
+            st.h[threadIdx.x] = rec_h[g];
+        }
+        __syncthreads();
+        const int nb = int(min(uint32_t(kTileBatch), range.y - b));
+        for (int c0 = 0; c0 < nb; c0 += 32) {
+            if (__all_sync(FULL, done)) break;
+            const int jl = c0 + lane;
+            bool pass = false;
+            if (jl < nb)
+                pass = !(box_min_half_q(st.m[jl], st.c[jl], bx0, bx1, by0, by1) * 0.999f >
+                         st.h[jl] + 1e-3f);
+            unsigned todo = __ballot_sync(FULL, pass);
+            while (todo && !done) {
+                const int j = c0 + __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const PixelTerm pt = eval_half_q(ux, uy, st.m[j], st.c[j]);
+                if (pt.half_q > st.h[j]) continue;
+                const float a = eval_alpha(st.a[j], pt.half_q, alpha_max);
+                if (a < alpha_min) continue;
+                done = visit(b + uint32_t(j), a);
+            }
+        }
+        __syncthreads();   // the stage is rewritten by the next batch
+    }
+}
+
+__global__ void __launch_bounds__(kThreads)
+topk_tile_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+            const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+            const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
+            int H, int tile_w, int tiles_x, int K, float alpha_min, float alpha_max,
+            float T_min, int32_t *__restrict__ ids, float *__restrict__ wout,
+            uint8_t *__restrict__ cnt) {
+    pdl_wait();
+    __shared__ float4 s_m[kTileBatch];
+    __shared__ float4 s_c[kTileBatch];
+    __shared__ float s_a[kTileBatch];
+    __shared__ float s_h[kTileBatch];
+    extern __shared__ unsigned char s_dyn[];
+    const int KS = K | 1;   // odd stride: a thread's slots fall in their own banks
+    uint32_t *s_key = reinterpret_cast<uint32_t *>(s_dyn);                 // [256][KS]
+    float *s_w = reinterpret_cast<float *>(s_dyn) + KS * kPix;             // [256][KS]
+    const Stage st{s_m, s_c, s_a, s_h};
+
+    const int tile = blockIdx.x;
+    const int tx = tile % tiles_x, ty = tile / tiles_x;
+    const int tile_h = kPix / tile_w;
+    const int lx = threadIdx.x % tile_w, ly = threadIdx.x / tile_w;
+    const int px = tx * tile_w + lx, py = ty * tile_h + ly;
+    const bool inside = px < W && py < H;
+    const float ux = float(px) + 0.5f, uy = float(py) + 0.5f;
+    const uint2 range = ranges[tile];
+    uint32_t *my_key = s_key + threadIdx.x * KS;
+    float *my_w = s_w + threadIdx.x * KS;
+
+    constexpr unsigned FULL = 0xffffffffu;
+    float bx0 = ux, bx1 = ux, by0 = uy, by1 = uy;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        bx0 = fminf(bx0, __shfl_xor_sync(FULL, bx0, o));
+        bx1 = fmaxf(bx1, __shfl_xor_sync(FULL, bx1, o));
+        by0 = fminf(by0, __shfl_xor_sync(FULL, by0, o));
+        by1 = fmaxf(by1, __shfl_xor_sync(FULL, by1, o));
+    }
+
+    int m = 0;          // kept entries
+    float D = 0.0f;     // normaliser
+    {
+        // ---- one dense walk keeping the K largest weights
+        float T = 1.0f, wmin = 0.0f;
+        int smin = 0;
+        bool done = !inside;
+        walk_list(rec_m, rec_w, rec_a, rec_h, isect_gid, range, st, ux, uy, bx0, bx1, by0, by1,
+                  alpha_min, alpha_max, done, [&](uint32_t pos, float a) -> bool {
+                      const float Tt = __fmul_rn(T, __fsub_rn(1.0f, a));
+                      if (T_min > 0.0f && Tt < T_min) return true;
+                      const float w = __fmul_rn(T, a);
+                      T = Tt;
+                      if (m < K) {
+                          my_key[m] = pos;
+                          my_w[m] = w;
+                          ++m;
+                          if (m < K) return false;
+                      } else if (w > wmin) {
+                          my_key[smin] = pos;
+                          my_w[smin] = w;
+                      } else {
+                          return __fmul_rn(T, alpha_max) <= wmin;
+                      }
+                      // the smallest kept weight, the latest entry among equal ones
+                      smin = 0;
+                      for (int j = 1; j < K; ++j)
+                          if (my_w[j] < my_w[smin] ||
+                              (my_w[j] == my_w[smin] && my_key[j] > my_key[smin]))
+                              smin = j;
+                      wmin = my_w[smin];
+                      return __fmul_rn(T, alpha_max) <= wmin;
+                  });
+        // depth order (list position), then the kept sum in that order
+        for (int i = 1; i < m; ++i) {
+            const uint32_t kk = my_key[i];
+            const float ww = my_w[i];
+            int j = i;
+            while (j > 0 && my_key[j - 1] > kk) {
+                my_key[j] = my_key[j - 1];
+                my_w[j] = my_w[j - 1];
+                --j;
+            }
+            my_key[j] = kk;
+            my_w[j] = ww;
+        }
+        for (int j = 0; j < m; ++j) D = __fadd_rn(D, my_w[j]);
+        for (int j = 0; j < m; ++j) my_key[j] = isect_gid[my_key[j]];
+    }
+
+    // ---- outputs (a pixel outside the image writes nothing)
+    if (inside) {
+        const int64_t p = int64_t(py) * W + px;
+        for (int j = 0; j < K; ++j) {
+            const bool has = j < m;
+            ids[p * K + j] = has ? int32_t(my_key[j]) : -1;
+            wout[p * K + j] = has ? __fdiv_rn(my_w[j], D) : 0.0f;
+        }
+        cnt[p] = uint8_t(m);
+    }
 }
 
 // ------------------------------------------------------------------ Stratified-K
@@ -425,12 +596,33 @@ cudaError_t launch_select_rule(const qr_frame &f, int rule, int32_t *ids, float 
                           f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
                           f.params.alpha_max, f.params.T_min, ids, w, cnt, last...);
     };
+    // Top-K with registers / in the tile kernel (us): K = 8 room VGA 64 / 83, object
+    // 517 x 389 101 / 216; K = 16 room VGA 169 / 141, object of 30k at VGA 176 / 139,
+    // but where latency bounds the walk (few blocks, or long lists, for which
+    // the capacity per tile stands) room 160 x 120 36 / 62, room 320 x 240 79 / 99,
+    // object 517 x 389 191 / 325; K = 32 room 800 x 600 903 / 441, object VGA 806 /
+    // 714.
+    const bool latency = tiles * 4 <= kFewBlocks || f.max_isect >= kLongTopLists * tiles;
     cudaError_t e;
-    if (rule == kStratified) e = go(stratified_kernel, 4, size_t(kSelBlock) * 4 * 3 * K, tau, vec);
-    else if (K <= 4) e = go(topk_kernel<4>, 8, 0, vec);
-    else if (K <= 8) e = go(topk_kernel<8>, 8, 0, vec);
-    else if (K <= 16) e = go(topk_kernel<16>, 8, 0, vec);
-    else e = go(topk_kernel<32>, 8, 0, vec);
+    if (rule == kStratified) {
+        e = go(stratified_kernel, 4, size_t(kSelBlock) * 4 * 3 * K, tau, vec);
+    } else if (K <= 4) {
+        e = go(topk_kernel<4>, 8, 0, vec);
+    } else if (K <= 8) {
+        e = go(topk_kernel<8>, 8, 0, vec);
+    } else if (K <= 16 && latency) {
+        e = go(topk_kernel<16>, 8, 0, vec);
+    } else {
+        const size_t dyn = size_t(K | 1) * kPix * 4 * 2;
+        e = cudaFuncSetAttribute(topk_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
+        if (e != cudaSuccess) return e;
+        e = pdl_launch(topk_tile_kernel, dim3(unsigned(tiles)), dim3(kThreads), dyn, s,
+                       (const float4 *)slot<float4>(f, S_REC_M), (const float4 *)slot<float4>(f, S_REC_C),
+                       (const float *)slot<float>(f, S_REC_A), (const float *)slot<float>(f, S_REC_H),
+                       (const uint32_t *)slot<uint32_t>(f, S_IGID), (const uint2 *)slot<uint2>(f, S_RANGES),
+                       f.camera.width, f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
+                       f.params.alpha_max, f.params.T_min, ids, w, cnt);
+    }
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -172,3 +172,21 @@ def test_riemann_selection_is_algorithm_1(K):
         ok = (np.abs(c - cj) <= 1e-5 * D).all(1) & ((cj >= 1) | (wk == 0)).all(1) & (ck <= D)
         found |= ok
     assert found.all()
+
+
+@pytest.mark.parametrize("K", [9, 16])
+def test_topk_kernels_agree(K):
+    """Top-K in registers and in the tile kernel (by the capacity of the lists
+    per tile) keep the same Gaussians with the same weights on a ragged image."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=16)
+    cam = scenes.room_camera(517, 389)
+    gdev = q.gaussians_to_device(g)
+    tiles = 33 * 25
+    a, b = (q.render_frame(gdev, None, cam, K=K, max_isect=per_tile * tiles, rule=q.QR_RULE_TOPK)
+            for per_tile in (500, 768))
+    torch.cuda.synchronize()
+    assert a["frame"].frame.max_isect == 500 * tiles and int(a["counts"].max()) == K
+    for k in ("ids", "weights", "counts"):
+        assert torch.equal(a[k], b[k]), k
