@@ -41,7 +41,7 @@
 //     for pass 2, which re-walks the list as the selection does.
 // Bound by instruction issue (room) and by the longest lists' chains (object).
 // Measured (CTAs of eight warps walking a tile in step, one pixel per lane ->
-// now): Stratified-K, room VGA, K = 8: 183 -> 112 us; top-K, object 517 x 389,
+// now): Stratified-K, room VGA, K = 8: 183 -> 109 us; top-K, object 517 x 389,
 // 200k Gaussians, K = 16: 315 -> 187 us.
 #include "select_tile.cuh"
 
@@ -417,28 +417,23 @@ __device__ __forceinline__ df2 two_prod2(float2 a, float2 b) {
     return {p, sel_fma2(a, b, make_float2(-p.x, -p.y))};
 }
 
-// The K boundaries of one pixel from its transmittance statistics.
-__device__ __forceinline__ void boundaries(df s1, df s2, int nb, int K, float *tau) {
-    if (nb >= 2) {
-        const df n = df_from(float(nb));
-        const df mu2 = df_div(s1, n);
-        const df var = df_sub(df_div(s2, n), df_mul(mu2, mu2));
-        const float mu = mu2.hi;
-        const float sigma = df_sqrt(var).hi;
-        const float zlo = __fdiv_rn(-mu, sigma);
-        const float zhi = __fdiv_rn(__fsub_rn(1.0f, mu), sigma);
-        const float ulo = normcdff(zlo), uhi = normcdff(zhi);
-        const float d = __fsub_rn(uhi, ulo);
-#pragma unroll 1
-        for (int k = 1; k <= K; ++k) {
-            const float c = __fdiv_rn(float(K + 1 - k), float(K + 1));
-            const float z = normcdfinvf(__fmaf_rn(d, c, ulo));
-            tau[(k - 1) * kSelBlock] = __fmaf_rn(sigma, z, mu);
-        }
-    } else {
-        for (int k = 1; k <= K; ++k)
-            tau[(k - 1) * kSelBlock] = __fdiv_rn(float(K + 1 - k), float(K + 1));
-    }
+// What the boundaries of a pixel are formed from (nb >= 2 blended entries).
+struct Spread {
+    float mu, sigma, ulo, d;
+};
+__device__ __forceinline__ Spread spread_of(df s1, df s2, int nb) {
+    const df n = df_from(float(nb));
+    const df mu2 = df_div(s1, n);
+    const df var = df_sub(df_div(s2, n), df_mul(mu2, mu2));
+    const float mu = mu2.hi;
+    const float sigma = df_sqrt(var).hi;
+    const float zlo = __fdiv_rn(-mu, sigma);
+    const float zhi = __fdiv_rn(__fsub_rn(1.0f, mu), sigma);
+    const float ulo = normcdff(zlo), uhi = normcdff(zhi);
+    return {mu, sigma, ulo, __fsub_rn(uhi, ulo)};
+}
+__device__ __forceinline__ float boundary_of(const Spread &p, float c, int nb) {
+    return nb >= 2 ? __fmaf_rn(p.sigma, normcdfinvf(__fmaf_rn(p.d, c, p.ulo)), p.mu) : c;
 }
 
 // Pass 2 of one pixel: Algorithm 1's state (Walk) with its own boundaries.
@@ -513,10 +508,21 @@ stratified_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ r
     };
     walk_block<false, 2>(rec_m, rec_w, rec_a, rec_h, isect_gid, range, W, H, at.x0, at.y0, alpha_min, alpha_max,
                       st, stats);
+    {
+        Spread p[2];
 #pragma unroll 1
-    for (int i = 0; i < 2; ++i)   // the code once: it is long
-        boundaries(i ? df{s1.hi.y, s1.lo.y} : df{s1.hi.x, s1.lo.x},
-                   i ? df{s2.hi.y, s2.lo.y} : df{s2.hi.x, s2.lo.x}, i ? n1 : n0, K, s_tau + 32 * i + lane);
+        for (int i = 0; i < 2; ++i) {   // the code once: it is long
+            const Spread q = spread_of(i ? df{s1.hi.y, s1.lo.y} : df{s1.hi.x, s1.lo.x},
+                                       i ? df{s2.hi.y, s2.lo.y} : df{s2.hi.x, s2.lo.x}, max(i ? n1 : n0, 1));
+            if (i) p[1] = q; else p[0] = q;
+        }
+#pragma unroll 1
+        for (int k = 1; k <= K; ++k) {   // both pixels' chains side by side
+            const float c = __fdiv_rn(float(K + 1 - k), float(K + 1));
+            s_tau[(k - 1) * kSelBlock + lane] = boundary_of(p[0], c, n0);
+            s_tau[(k - 1) * kSelBlock + 32 + lane] = boundary_of(p[1], c, n1);
+        }
+    }
     __syncwarp();
     // ---- pass 2: Algorithm 1 with the boundaries tau_k
     const float *tau0 = s_tau + lane, *tau1 = s_tau + 32 + lane;
