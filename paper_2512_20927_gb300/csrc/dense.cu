@@ -374,7 +374,8 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
         unsigned long long n_exec = 0;
         for (uint32_t it = 0;; ++it) {
             const uint32_t r = it % kRows, ph = (it / kRows) & 1u;
-            if (!dense_wait(&sh.r_full[r], ph, abort)) break;
+            // one verdict per warp: its lanes meet again below
+            if (!__all_sync(FULL, dense_wait(&sh.r_full[r], ph, abort))) break;
             const DenseRow &R = sh.row[r];
             const int block = R.block, last = R.last, at = R.slot;
             if (block == kItemEnd) break;

@@ -1,0 +1,42 @@
+"""The dense block kernel's way out of a wait that ran out, read in its source:
+whatever the lanes of a warp see, they leave together, and nothing that writes
+shared memory asynchronously outlives the CTA.  (The kernel's waits run out on
+the GPU in test_gpu_errors.py.)"""
+import re
+from pathlib import Path
+
+SOURCE = Path(__file__).parents[1] / "paper_2512_20927_gb300" / "csrc" / "dense.cu"
+
+
+def _roles():
+    """The kernel's text by role, without comments."""
+    text = SOURCE.read_text()
+    text = text[text.index("dense_block_kernel(const float4"):text.index("cudaError_t run_block")]
+    cut = [text.index("- " + r) for r in ("consumers", "producers", "loader")] + [len(text)]
+    parts = [re.sub(r"//[^\n]*", "", text[a:b]) for a, b in zip(cut, cut[1:])]
+    return dict(zip(("consumers", "producers", "loader"), parts))
+
+
+def _calls(text, name):
+    """(start, whole call) of every call of name, its brackets matched."""
+    for m in re.finditer(rf"\b{name}\(", text):
+        depth, i = 1, m.end()
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[i], 0)
+            i += 1
+        yield m.start(), text[m.start():i]
+
+
+def test_every_wait_is_voted_by_its_warp():
+    """A wait of all lanes is the argument of a vote, or of the `ok` that the
+    next statement votes on; the waits of lane 0 alone are voted on after its
+    branch."""
+    for role, text in _roles().items():
+        voted = [c for _, c in _calls(text, "__all_sync")]
+        waits = list(_calls(text, "dense_wait"))
+        assert waits, role
+        for at, call in waits:
+            if any(call in v for v in voted):
+                continue
+            assert re.search(r"ok = (ok && )?$", text[:at]), (role, call)
+            assert "ok = __all_sync(FULL, ok);" in text[at:], (role, call)
