@@ -473,6 +473,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                     try_cancel(&sh.response, &sh.clc);
                     ok = dense_wait(&sh.clc, i & 1u, abort);
                     if (ok) next = cancelled_cta(&sh.response);
+                    else tma_mbar_wait(&sh.clc, i & 1u, kDenseSpin);   // it lands before the CTA exits
                 }
                 ok = ok && dense_wait(&sh.mail_empty[p1], (((i + 1) / kProd) & 1u) ^ 1u, abort);
                 if (ok) {
@@ -571,10 +572,10 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                 }
             }
         }
-        // after a timeout: the copies issued last land before the CTA exits
-        if (!ok)
-            for (uint32_t i = rc > kRows ? rc - kRows : 0; i < rc; ++i)
-                tma_mbar_wait(&sh.r_full[i % kRows], (i / kRows) & 1u, kDenseSpin);
+        // the copies issued last land before the CTA exits, whichever role gave
+        // up and whenever it did
+        for (uint32_t i = rc > kRows ? rc - kRows : 0; i < rc; ++i)
+            tma_mbar_wait(&sh.r_full[i % kRows], (i / kRows) & 1u, kDenseSpin);
     }
     __syncthreads();
     if (threadIdx.x == 0 && *abort) atomicExch(&counters[CNT_STATUS], uint32_t(QR_ERR_DEVICE_TIMEOUT));

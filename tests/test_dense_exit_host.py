@@ -40,3 +40,19 @@ def test_every_wait_is_voted_by_its_warp():
                 continue
             assert re.search(r"ok = (ok && )?$", text[:at]), (role, call)
             assert "ok = __all_sync(FULL, ok);" in text[at:], (role, call)
+
+
+def test_nothing_in_flight_outlives_the_cta():
+    """A work request is waited for, with the full limit, by the lane that
+    issued it when its wait gave up; the loader waits for its last row copies
+    on every way out, as another role may give up after it has finished."""
+    roles = _roles()
+    ask = roles["producers"].index("try_cancel(")
+    after = roles["producers"][ask:roles["producers"].index("mail_empty", ask)]
+    assert re.search(r"else\s+tma_mbar_wait\(&sh\.clc, i & 1u, kDenseSpin\);", after)
+    loader = roles["loader"]
+    drain = re.search(r"(\S+)\s+for \(uint32_t i = rc > kRows [^\n]*\n\s*"
+                      r"tma_mbar_wait\(&sh\.r_full\[i % kRows\], \(i / kRows\) & 1u, kDenseSpin\);",
+                      loader)
+    assert drain and drain[1] == "}", "the loader's drain depends on a condition"
+    assert drain.start() > loader.rindex("bulk_row(")
