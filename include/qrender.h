@@ -236,14 +236,19 @@ qr_status qr_blend(const void *feat, const float *feat_scale, qr_dtype dtype, in
 /* Eq. 1 (V-Render, the dense method the paper compares against):
  * out[p] = sum_i T_i alpha'_i f_i over the pixel's whole list with the same
  * alpha' rules, stopping before a Gaussian whose test transmittance would fall
- * below T_min.  out [P][C] float32; T_final [P] float32 (nullable). */
+ * below T_min.  out [P][C] float32; T_final [P] float32 (nullable).
+ * Rows of 64, 128, 256 and 512 channels take a kernel whose warps hand work to
+ * each other behind bounded waits (qr_set_wait_limit); if one runs out (a lost
+ * hand-over: not in normal use) the frame's status becomes
+ * QR_ERR_DEVICE_TIMEOUT, which qr_frame_status reports until the next
+ * qr_project, and out and T_final are incomplete. */
 qr_status qr_dense(const qr_frame *frame, const void *feat, const float *feat_scale,
                    qr_dtype dtype, int32_t C, float *out, float *T_final, qr_stream stream);
 
 /* qr_dense that also counts its work, for measurement: counts [2] device
  * uint64 (zeroed by the call) receive the blended (pixel, Gaussian) pairs --
  * each C multiply-adds of useful work -- and the multiply-adds the kernel
- * executed (rows of 128, 256 or 512 channels; both stay 0 for other widths). */
+ * executed (rows of 64, 128, 256 or 512 channels; both stay 0 for other widths). */
 qr_status qr_dense_work(const qr_frame *frame, const void *feat, const float *feat_scale,
                         qr_dtype dtype, int32_t C, float *out, float *T_final, uint64_t *counts,
                         qr_stream stream);
@@ -514,12 +519,12 @@ qr_status qr_render_noalloc(const float *mean, const float *log_scale, const flo
 uint64_t qr_launch_count(void);
 
 /* Test hook for the device-side error path.  The relevance kernels
- * (qr_relevance's TMA kernel, qr_blend_relevance) bound each of their waits
- * on a producer, the tensor cores or the epilogue to a number of polls
- * (2^26 by default, seconds); when one runs out the CTA stops every role,
- * waits (with the default bound) for its own copies and MMAs in flight,
+ * (qr_relevance's TMA kernel, qr_blend_relevance) and qr_dense's block kernel
+ * bound each of their waits on another role or the tensor cores to a number
+ * of polls (2^26 by default, seconds); when one runs out the CTA stops every
+ * role, waits (with the default bound) for its own copies and MMAs in flight,
  * frees its tensor memory and writes QR_ERR_DEVICE_TIMEOUT to the call's
- * status word.  qr_set_wait_limit(polls) sets that bound for the launches
+ * status word (qr_dense: the frame's).  qr_set_wait_limit(polls) sets that bound for the launches
  * that follow (0 restores the default), so a test can make a wait run out
  * without anything hanging.  Not for production use; not thread-safe. */
 void qr_set_wait_limit(uint32_t polls);

@@ -165,6 +165,7 @@ cudaError_t launch_contrastive_loss(const float *F, const float *tgt, int M, int
                                     void *ws, cudaStream_t s);
 bool relevance_supported(int Q, int C);
 void set_wait_limit(unsigned polls);
+unsigned wait_limit();
 bool set_blend_chunks(int chunks);
 // blend of qr_blend fused with the relevance product (the map is never written)
 bool blend_relevance_supported(qr_dtype dt, int Q, int C, int K);

@@ -204,8 +204,9 @@ __device__ __forceinline__ bool lane_wait(uint64_t *bar, uint32_t parity, volati
     return false;
 }
 
-// Polls allowed to the first-level waits of the relevance kernels (those
-// that set the abort flag); the drains after an abort keep kSpinLimit.
+// Polls allowed to the first-level waits of the relevance kernels and the dense
+// block kernel (those that set the abort flag); the drains after an abort keep
+// kSpinLimit.
 // Changed only through qr_set_wait_limit (a test hook).
 unsigned g_wait_limit = kSpinLimit;
 
@@ -893,6 +894,7 @@ cudaError_t run(const float *map, const uint16_t *q, int64_t P, int C, float *ou
 }  // namespace
 
 void set_wait_limit(unsigned polls) { g_wait_limit = polls ? polls : kSpinLimit; }
+unsigned wait_limit() { return g_wait_limit < 1u << 31 ? g_wait_limit : 1u << 31; }
 
 bool blend_relevance_supported(qr_dtype dt, int Q, int C, int K) {
     if (C < FB_CHUNK || C % FB_CHUNK || K < 1 || K > 8) return false;

@@ -548,7 +548,8 @@ def qr_launch_count() -> int:
 
 
 def qr_set_wait_limit(polls: int):
-    """Test hook: bound the relevance kernels' waits to `polls` polls (0 = default)."""
+    """Test hook: bound the waits of the relevance kernels and of qr_dense's block kernel
+    to `polls` polls (0 = default)."""
     load().qr_set_wait_limit(int(polls))
 
 
@@ -610,6 +611,8 @@ def render_frame(gdev, feat, cam, K=8, max_isect=None, params=None, stream=None,
             dout = torch.empty((P, C), dtype=torch.float32, device=mean.device)
             tf = torch.empty(P, dtype=torch.float32, device=mean.device)
             qr_dense(fr, f, fs, dout, tf, stream=stream)
+            # a wait that ran out on the device leaves the map incomplete
+            _check(qr_frame_status(fr, stream)[0], "qr_dense")
             res["dense"] = dout
             res["T_final"] = tf
     return res

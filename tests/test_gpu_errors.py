@@ -61,6 +61,41 @@ def test_wait_that_runs_out_reports_timeout_and_recovers(fused):
     assert torch.equal(again, good)
 
 
+@pytest.mark.parametrize("channels,dtype", [(64, "f32"), (128, "fp8"), (256, "bf16"), (512, "f32")])
+def test_dense_wait_that_runs_out_reports_timeout_and_recovers(channels, dtype):
+    """qr_dense's block kernel: the same hook; the frame's status reports it
+    until the frame is projected again, and render_frame does not hand out a
+    map that may be incomplete."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = scenes.room_scene(seed=4, n=100_000, channels=channels)
+    cam = scenes.room_camera(320, 240)
+    gdev = q.gaussians_to_device(g)
+    table, scale = torch.from_numpy(f).cuda(), None
+    if dtype == "bf16":
+        table = q.qr_quantize_bf16(table)
+    elif dtype == "fp8":
+        table, scale = q.qr_quantize_fp8(table)
+    feat = table if scale is None else (table, scale)
+    res = q.render_frame(gdev, feat, cam, K=8, dense=True)
+    fr, good, good_T = res["frame"], res["dense"], res["T_final"]
+    out, T = torch.empty_like(good), torch.empty_like(good_T)
+    try:
+        q.qr_set_wait_limit(1)
+        q.qr_dense(fr, table, scale, out, T)
+        assert q.qr_frame_status(fr)[0] == q.QR_ERR_DEVICE_TIMEOUT
+        with pytest.raises(q.QRError) as e:
+            q.render_frame(gdev, feat, cam, K=8, dense=True)
+        assert e.value.code == q.QR_ERR_DEVICE_TIMEOUT
+    finally:
+        q.qr_set_wait_limit(0)
+    q.qr_project(fr, *gdev)
+    q.qr_sort(fr)
+    q.qr_dense(fr, table, scale, out, T)
+    assert q.qr_frame_status(fr)[0] == q.QR_OK
+    assert torch.equal(out, good) and torch.equal(T, good_T)
+
+
 def test_non_finite_gaussians_are_culled():
     g, f = scenes.tiny_scene(seed=6)
     rng = np.random.default_rng(6)
