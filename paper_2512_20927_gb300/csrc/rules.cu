@@ -30,9 +30,9 @@
 //     smallest (latest among equal) out.  Once fl(T alpha_max) is no larger
 //     than the smallest kept weight, no later entry can enter (T only falls
 //     and alpha' <= alpha_max), so the pixel stops early without changing the
-//     result.  Shared-memory slots with a replaced minimum, two pixels per
-//     lane, took 238 us where this takes 187 (below).  With many entries the
-//     insertions cost more than a search of slots: topk_tile_kernel.
+//     result.  With more than 8 entries the insertions cost more than
+//     replacing the smallest of K slots in shared memory (topk_slots_kernel),
+//     unless the latency of a walk bounds the frame.
 //   * Stratified-K sums T and T^2 in compensated double-FP32 arithmetic, both
 //     pixels of a lane in one packed FP32x2 instruction stream (adding an
 //     exact 0 where an entry is no member) and four entries at a time, forms
@@ -41,8 +41,8 @@
 //     for pass 2, which re-walks the list as the selection does.
 // Bound by instruction issue (room) and by the longest lists' chains (object).
 // Measured (CTAs of eight warps walking a tile in step, one pixel per lane ->
-// now): Stratified-K, room VGA, K = 8: 183 -> 109 us; top-K, object 517 x 389,
-// 200k Gaussians, K = 16: 315 -> 187 us.
+// now): Stratified-K, room VGA, K = 8: 183 -> 109 us; top-K, K = 8, room VGA
+// 90 -> 73 us; top-K in slots: with its kernel.
 #include "select_tile.cuh"
 
 namespace qr {
@@ -50,10 +50,10 @@ namespace {
 
 enum { kTopK = 1, kStratified = 2 };
 
-// 8 x 8 blocks up to which, and list capacity per tile from which, latency
-// rather than issue bounds top-K's walk
+// 8 x 8 blocks up to which, and capacity per tile from which, the chain of a
+// walk rather than issue bounds top-K (launch_select_rule)
 constexpr int kFewBlocks = 152 * 8;
-constexpr int64_t kLongTopLists = 768;
+constexpr int64_t kLongTopLists = 320;
 
 // ------------------------------------------------------------------ top-K
 constexpr int kTopPix = 32;        // pixels per warp: 8 x 4, one per lane
@@ -218,168 +218,119 @@ topk_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 }
 
 // ------------------------------------------------------------------ top-K, many entries
-// One CTA per screen tile, one pixel per thread: the list is staged 256 records
-// at a time and culled per warp, and a pixel's candidates sit in shared-memory
-// slots whose smallest a replacement searches again.  With more entries an
-// insertion into sorted registers costs more than that search, unless latency
-// bounds the walk.
-constexpr int kPix = 256;
-constexpr int kThreads = 256;
-constexpr int kTileBatch = 256;
-
-struct Stage {
-    float4 *m, *c;
-    float *a, *h;
+// A pixel's K slots (shared memory, entry-major: a lane's accesses fall in its
+// own bank) stand in groups of four with the smallest of each group kept
+// beside them, so replacing the smallest searches four slots and the groups,
+// and only lanes whose entry enters take part.
+// Bound by instruction issue (room) and by the longest lists' chains (object).
+// K = 9 / 16 / 32, us (one CTA of eight warps per tile, the list staged for all
+// of them and K slots searched on each replacement -> sorted registers, K <= 16
+// -> this): room VGA 300k Gaussians 102 / 155 / 366 -> 135 / 181 -> 87 / 111 /
+// 210; room VGA 1M 100 / 149 / 316 -> 142 / 188 -> 92 / 112 / 187; room 1M at 1296
+// x 968 278 / 445 / 1037 -> 461 / 618 -> 275 / 339 / 584; object VGA 500k 358 / 474 /
+// 1141 -> 250 / 303 -> 220 / 269 / 430; object 517 x 389 200k 235 / 332 / 717 -> 158 /
+// 200 -> 143 / 178 / 274.  Two pixels per lane instead: that last K = 16 238.
+struct Slots {
+    uint32_t *key;   // [K][32]: list position
+    float *w;        // [K][32]: weight
+    float *gw;       // [G][32]: smallest weight of a group ...
+    uint32_t *gk;    // [G][32]: ... and its slot
 };
-
-// Walks the tile's list for this thread's pixel: stages records, culls them
-// per warp against the warp's pixel box and calls visit(pos, alpha') for
-// every member entry (alpha' >= alpha_min) in list order until the pixel is
-// done.  visit returns true when the pixel has finished its walk.  All
-// threads of the CTA must call it.
-template <typename Visit>
-__device__ __forceinline__ void walk_list(const float4 *__restrict__ rec_m,
-                                          const float4 *__restrict__ rec_w,
-                                          const float *__restrict__ rec_a,
-                                          const float *__restrict__ rec_h,
-                                          const uint32_t *__restrict__ isect_gid, uint2 range,
-                                          const Stage &st, float ux, float uy, float bx0,
-                                          float bx1, float by0, float by1, float alpha_min,
-                                          float alpha_max, bool &done, Visit visit) {
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    for (uint32_t b = range.x; b < range.y; b += kTileBatch) {
-        if (__syncthreads_count(done) == kThreads) break;
-        if (b + threadIdx.x < range.y) {
-            const uint32_t g = isect_gid[b + threadIdx.x];
-            st.m[threadIdx.x] = rec_m[g];
-            st.c[threadIdx.x] = rec_w[g];
-            st.a[threadIdx.x] = rec_a[g];
-            st.h[threadIdx.x] = rec_h[g];
+// Slot a goes before slot b: the smaller weight, the later entry of equal ones.
+__device__ __forceinline__ bool slot_less(float wa, uint32_t a, float wb, uint32_t b, const uint32_t *key) {
+    return wa < wb || (wa == wb && key[a * kTopPix] > key[b * kTopPix]);
+}
+__device__ __forceinline__ void rescan_group(const Slots &s, int g, int K) {
+    const int j0 = 4 * g;
+    float v[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = j0 + i < K ? s.w[(j0 + i) * kTopPix] : INFINITY;
+    uint32_t at = uint32_t(j0);
+    float b = v[0];
+#pragma unroll
+    for (int i = 1; i < 4; ++i)
+        if (v[i] <= b && j0 + i < K && slot_less(v[i], uint32_t(j0 + i), b, at, s.key)) {
+            at = uint32_t(j0 + i);
+            b = v[i];
         }
-        __syncthreads();
-        const int nb = int(min(uint32_t(kTileBatch), range.y - b));
-        for (int c0 = 0; c0 < nb; c0 += 32) {
-            if (__all_sync(FULL, done)) break;
-            const int jl = c0 + lane;
-            bool pass = false;
-            if (jl < nb)
-                pass = !(box_min_half_q(st.m[jl], st.c[jl], bx0, bx1, by0, by1) * 0.999f >
-                         st.h[jl] + 1e-3f);
-            unsigned todo = __ballot_sync(FULL, pass);
-            while (todo && !done) {
-                const int j = c0 + __ffs(todo) - 1;
-                todo &= todo - 1u;
-                const PixelTerm pt = eval_half_q(ux, uy, st.m[j], st.c[j]);
-                if (pt.half_q > st.h[j]) continue;
-                const float a = eval_alpha(st.a[j], pt.half_q, alpha_max);
-                if (a < alpha_min) continue;
-                done = visit(b + uint32_t(j), a);
-            }
-        }
-        __syncthreads();   // the stage is rewritten by the next batch
+    s.gw[g * kTopPix] = b;
+    s.gk[g * kTopPix] = at;
+}
+// Keeps the member at list position pos with weight x > wmin: a free slot
+// while there is one (wmin < 0), else the smallest's.
+__device__ __forceinline__ void slot_insert(const Slots &s, int K, uint32_t pos, float x, int &m,
+                                            uint32_t &smin, float &wmin) {
+    const int G = (K + 3) >> 2;
+    const uint32_t at = m < K ? uint32_t(m) : smin;
+    s.key[at * kTopPix] = pos;
+    s.w[at * kTopPix] = x;
+    if (m < K) {
+        if (++m < K) return;
+        for (int g = 0; g < G; ++g) rescan_group(s, g, K);
+    } else {
+        rescan_group(s, int(at >> 2), K);
     }
+    float b = s.gw[0];
+    uint32_t bs = s.gk[0];
+    for (int g = 1; g < G; ++g) {
+        const float v = s.gw[g * kTopPix];
+        const uint32_t vs = s.gk[g * kTopPix];
+        if (v <= b && slot_less(v, vs, b, bs, s.key)) {
+            b = v;
+            bs = vs;
+        }
+    }
+    wmin = b;
+    smin = bs;
 }
 
-__global__ void __launch_bounds__(kThreads)
-topk_tile_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
-            const float *__restrict__ rec_a, const float *__restrict__ rec_h,
-            const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
-            int H, int tile_w, int tiles_x, int K, float alpha_min, float alpha_max,
-            float T_min, int32_t *__restrict__ ids, float *__restrict__ wout,
-            uint8_t *__restrict__ cnt) {
-    pdl_wait();
-    __shared__ float4 s_m[kTileBatch];
-    __shared__ float4 s_c[kTileBatch];
-    __shared__ float s_a[kTileBatch];
-    __shared__ float s_h[kTileBatch];
-    extern __shared__ unsigned char s_dyn[];
-    const int KS = K | 1;   // odd stride: a thread's slots fall in their own banks
-    uint32_t *s_key = reinterpret_cast<uint32_t *>(s_dyn);                 // [256][KS]
-    float *s_w = reinterpret_cast<float *>(s_dyn) + KS * kPix;             // [256][KS]
-    const Stage st{s_m, s_c, s_a, s_h};
-
-    const int tile = blockIdx.x;
-    const int tx = tile % tiles_x, ty = tile / tiles_x;
-    const int tile_h = kPix / tile_w;
-    const int lx = threadIdx.x % tile_w, ly = threadIdx.x / tile_w;
-    const int px = tx * tile_w + lx, py = ty * tile_h + ly;
-    const bool inside = px < W && py < H;
-    const float ux = float(px) + 0.5f, uy = float(py) + 0.5f;
-    const uint2 range = ranges[tile];
-    uint32_t *my_key = s_key + threadIdx.x * KS;
-    float *my_w = s_w + threadIdx.x * KS;
-
+__global__ void __launch_bounds__(32, 24)
+topk_slots_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
+                  const float *__restrict__ rec_a, const float *__restrict__ rec_h,
+                  const uint32_t *__restrict__ isect_gid, const uint2 *__restrict__ ranges, int W,
+                  int H, int tile_w, int tiles_x, int K, float alpha_min, float alpha_max,
+                  float T_min, int32_t *__restrict__ ids, float *__restrict__ wout,
+                  uint8_t *__restrict__ cnt, int vec) {
     constexpr unsigned FULL = 0xffffffffu;
-    float bx0 = ux, bx1 = ux, by0 = uy, by1 = uy;
+    __shared__ SelStage st;
+    extern __shared__ unsigned char s_dyn[];
+    const int lane = threadIdx.x & 31, G = (K + 3) >> 2;
+    uint32_t *s_key = reinterpret_cast<uint32_t *>(s_dyn);
+    float *s_w = reinterpret_cast<float *>(s_key + K * kTopPix);
+    float *s_gw = s_w + K * kTopPix;
+    const Slots s{s_key + lane, s_w + lane, s_gw + lane, reinterpret_cast<uint32_t *>(s_gw + G * kTopPix) + lane};
+    pdl_wait();   // the predecessor's outputs are complete and visible
+    const BlockAt at = block_at<1>(int(blockIdx.x), tile_w, tiles_x);
+    const int px = at.x0 + (lane & 7), py = at.y0 + (lane >> 3);
+    const bool inside = px < W && py < H;
+    int m = 0;
+    uint32_t smin = 0u;
+    float T = 1.0f;
+    float wmin = inside ? -0.5f : INFINITY;   // the smallest kept weight; +inf once the pixel has stopped
+    auto visit = [&](int j, const float (&a)[4][1]) -> bool {
+        float w[4];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        bx0 = fminf(bx0, __shfl_xor_sync(FULL, bx0, o));
-        bx1 = fmaxf(bx1, __shfl_xor_sync(FULL, bx1, o));
-        by0 = fminf(by0, __shfl_xor_sync(FULL, by0, o));
-        by1 = fmaxf(by1, __shfl_xor_sync(FULL, by1, o));
-    }
-
-    int m = 0;          // kept entries
-    float D = 0.0f;     // normaliser
-    {
-        // ---- one dense walk keeping the K largest weights
-        float T = 1.0f, wmin = 0.0f;
-        int smin = 0;
-        bool done = !inside;
-        walk_list(rec_m, rec_w, rec_a, rec_h, isect_gid, range, st, ux, uy, bx0, bx1, by0, by1,
-                  alpha_min, alpha_max, done, [&](uint32_t pos, float a) -> bool {
-                      const float Tt = __fmul_rn(T, __fsub_rn(1.0f, a));
-                      if (T_min > 0.0f && Tt < T_min) return true;
-                      const float w = __fmul_rn(T, a);
-                      T = Tt;
-                      if (m < K) {
-                          my_key[m] = pos;
-                          my_w[m] = w;
-                          ++m;
-                          if (m < K) return false;
-                      } else if (w > wmin) {
-                          my_key[smin] = pos;
-                          my_w[smin] = w;
-                      } else {
-                          return __fmul_rn(T, alpha_max) <= wmin;
-                      }
-                      // the smallest kept weight, the latest entry among equal ones
-                      smin = 0;
-                      for (int j = 1; j < K; ++j)
-                          if (my_w[j] < my_w[smin] ||
-                              (my_w[j] == my_w[smin] && my_key[j] > my_key[smin]))
-                              smin = j;
-                      wmin = my_w[smin];
-                      return __fmul_rn(T, alpha_max) <= wmin;
-                  });
-        // depth order (list position), then the kept sum in that order
-        for (int i = 1; i < m; ++i) {
-            const uint32_t kk = my_key[i];
-            const float ww = my_w[i];
-            int j = i;
-            while (j > 0 && my_key[j - 1] > kk) {
-                my_key[j] = my_key[j - 1];
-                my_w[j] = my_w[j - 1];
-                --j;
-            }
-            my_key[j] = kk;
-            my_w[j] = ww;
+        for (int u = 0; u < 4; ++u) {   // as in topk_kernel
+            const float n = __fmul_rn(T, __fsub_rn(1.0f, a[u][0]));
+            w[u] = a[u][0] > 0.0f && !(n < T_min) ? __fmul_rn(T, a[u][0]) : -1.0f;
+            T = n;
         }
-        for (int j = 0; j < m; ++j) D = __fadd_rn(D, my_w[j]);
-        for (int j = 0; j < m; ++j) my_key[j] = isect_gid[my_key[j]];
-    }
-
-    // ---- outputs (a pixel outside the image writes nothing)
-    if (inside) {
-        const int64_t p = int64_t(py) * W + px;
-        for (int j = 0; j < K; ++j) {
-            const bool has = j < m;
-            ids[p * K + j] = has ? int32_t(my_key[j]) : -1;
-            wout[p * K + j] = has ? __fdiv_rn(my_w[j], D) : 0.0f;
+#pragma unroll 1
+        for (int u = 0; u < 4; ++u) {   // the insertion's code once
+            const float x = u == 0 ? w[0] : u == 1 ? w[1] : u == 2 ? w[2] : w[3];
+            if (x > wmin) slot_insert(s, K, st.g[j + u], x, m, smin, wmin);
         }
-        cnt[p] = uint8_t(m);
-    }
+        // no later entry can enter once fl(T alpha_max) is no larger than wmin
+        if (T < T_min || __fmul_rn(T, alpha_max) <= wmin) wmin = INFINITY;
+        return !__all_sync(FULL, wmin == INFINITY);
+    };
+    walk_block<true, 1>(rec_m, rec_w, rec_a, rec_h, isect_gid, ranges[at.tile], W, H, at.x0, at.y0,
+                        alpha_min, alpha_max, st, visit);
+    top_finish(m, K, isect_gid, s_key + lane, s_w + lane);
+    __syncwarp();
+    store_slots<1>(W, H, at.x0, at.y0, K, vec != 0, reinterpret_cast<const int32_t *>(s_key), ids);
+    store_slots<1>(W, H, at.x0, at.y0, K, vec != 0, (const float *)s_w, wout);
+    if (inside) cnt[int64_t(py) * W + px] = uint8_t(m);
 }
 
 // ------------------------------------------------------------------ Stratified-K
@@ -602,13 +553,13 @@ cudaError_t launch_select_rule(const qr_frame &f, int rule, int32_t *ids, float 
                           f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
                           f.params.alpha_max, f.params.T_min, ids, w, cnt, last...);
     };
-    // Top-K with registers / in the tile kernel (us): K = 8 room VGA 64 / 83, object
-    // 517 x 389 101 / 216; K = 16 room VGA 169 / 141, object of 30k at VGA 176 / 139,
-    // but where latency bounds the walk (few blocks, or long lists, for which
-    // the capacity per tile stands) room 160 x 120 36 / 62, room 320 x 240 79 / 99,
-    // object 517 x 389 191 / 325; K = 32 room 800 x 600 903 / 441, object VGA 806 /
-    // 714.
-    const bool latency = tiles * 4 <= kFewBlocks || f.max_isect >= kLongTopLists * tiles;
+    // Top-K of 9 .. 16 entries in registers / in slots (us, K = 9, 16) where a
+    // frame has few blocks: long lists, object 30k at 100 x 70 124, 131 / 157, 169,
+    // object 200k at 320 x 240 149, 178 / 170, 206, room 100k at 160 x 120 (326
+    // entries per tile) 46, 56 / 54, 66; short ones, room 100k at 320 x 240 (151) 60,
+    // 78 / 48, 58, room 20k at 160 x 120 (65) 30, 34 / 33, 25.  With more blocks slots
+    // are the faster ones throughout (topk_slots_kernel).
+    const bool latency = tiles * 4 <= kFewBlocks && f.max_isect >= kLongTopLists * tiles;
     cudaError_t e;
     if (rule == kStratified) {
         e = go(stratified_kernel, 4, size_t(kSelBlock) * 4 * 3 * K, tau, vec);
@@ -619,15 +570,7 @@ cudaError_t launch_select_rule(const qr_frame &f, int rule, int32_t *ids, float 
     } else if (K <= 16 && latency) {
         e = go(topk_kernel<16>, 8, 0, vec);
     } else {
-        const size_t dyn = size_t(K | 1) * kPix * 4 * 2;
-        e = cudaFuncSetAttribute(topk_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(dyn));
-        if (e != cudaSuccess) return e;
-        e = pdl_launch(topk_tile_kernel, dim3(unsigned(tiles)), dim3(kThreads), dyn, s,
-                       (const float4 *)slot<float4>(f, S_REC_M), (const float4 *)slot<float4>(f, S_REC_C),
-                       (const float *)slot<float>(f, S_REC_A), (const float *)slot<float>(f, S_REC_H),
-                       (const uint32_t *)slot<uint32_t>(f, S_IGID), (const uint2 *)slot<uint2>(f, S_RANGES),
-                       f.camera.width, f.camera.height, f.params.tile_w, f.tiles_x, K, f.params.alpha_min,
-                       f.params.alpha_max, f.params.T_min, ids, w, cnt);
+        e = go(topk_slots_kernel, 8, size_t(kTopPix) * 8 * (K + (K + 3) / 4), vec);
     }
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();

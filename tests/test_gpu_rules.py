@@ -190,3 +190,46 @@ def test_topk_kernels_agree(K):
     assert a["frame"].frame.max_isect == 500 * tiles and int(a["counts"].max()) == K
     for k in ("ids", "weights", "counts"):
         assert torch.equal(a[k], b[k]), k
+
+
+@pytest.mark.parametrize("size", [(113, 67), (330, 250)])
+@pytest.mark.parametrize("K", [9, 12, 16, 17, 29, 32])
+def test_topk_slots_deep_lists(K, size):
+    """Slot groups whole and cut (K % 4) and up to hundreds of members per
+    pixel, on images of few and of many blocks, both filled by the slab."""
+    rng = np.random.default_rng(12)
+    n, wide = 3000, size[0] / 113
+    mean = np.stack([rng.uniform(-0.3 * wide, 0.3 * wide, n), rng.uniform(-0.3 * wide, 0.3 * wide, n),
+                     rng.uniform(-1.5, 1.5, n)], 1).astype(np.float32)
+    g = scenes.Gaussians(mean, np.full((n, 3), np.log(wide) - 2.0, np.float32),
+                         np.tile(np.array([1, 0, 0, 0], np.float32), (n, 1)),
+                         rng.uniform(0.02, 0.4, n).astype(np.float32))
+    rep = _run(g, None, scenes.tiny_camera(*size), oracle.RULE_TOPK, K, max_tie_frac=0.06,
+               pixels=H.sample_pixels(*size, 200, seed=K), label=f"slots K={K} {size}")
+    assert rep["kept_mean"] > K / 2
+
+
+@pytest.mark.parametrize("K", [9, 13, 16])
+def test_topk_slots_and_registers_agree(K):
+    """An image of few blocks takes slots or, at a large capacity, sorted
+    registers: the same Gaussians with the same weights."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, f = H.small_room(n=20000, channels=16)
+    cam = scenes.room_camera(113, 67)
+    gdev, tiles = q.gaussians_to_device(g), 8 * 5
+    outs = []
+    for per_tile in (300, 2048):
+        fr = q.frame_create(g.n, cam, q.default_params(K), per_tile * tiles)
+        q.qr_project(fr, *gdev)
+        q.qr_sort(fr)
+        out = (torch.empty((fr.pixels, K), dtype=torch.int32, device="cuda"),
+               torch.empty((fr.pixels, K), dtype=torch.float32, device="cuda"),
+               torch.empty(fr.pixels, dtype=torch.uint8, device="cuda"))
+        q.qr_select_rule(fr, q.QR_RULE_TOPK, *out, None)
+        code, n_isect = q.qr_frame_status(fr)
+        assert code == q.QR_OK and n_isect > 0
+        outs.append(out)
+    assert int(outs[0][2].max()) == K
+    for a, b in zip(*outs):
+        assert torch.equal(a, b)
