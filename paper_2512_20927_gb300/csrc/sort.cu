@@ -24,10 +24,11 @@
 //      its tile's bucket at an atomically claimed position (counted per tile
 //      in shared memory first, one global atomic per touched tile, when the
 //      grid has at most 4096 tiles);
-//   5. tile_sort: one CTA per tile sorts a bucket of up to 2048 keys
-//      (bitonic network over the unique 64-bit keys in registers: register
-//      swaps, warp shuffles, shared memory only for the cross-warp strides)
-//      and writes the ids; a larger bucket goes to a list, which
+//   5. tile_sort: one CTA per tile sorts a bucket of up to 2048 keys by
+//      32-bit stand-ins for the unique 64-bit ones, or by those where depths
+//      tie ("per-tile sort" below): a bitonic network in registers (register
+//      swaps, warp shuffles, shared memory only for the cross-warp strides);
+//      it writes the ids.  A larger bucket goes to a list, which
 //      tile_sort_big's persistent CTAs of 1024 threads work through: up to
 //      8192 keys merge-sorted in shared memory (runs of 8 in registers, then
 //      merge-path rounds between two buffers), beyond that in 8192-key
@@ -306,60 +307,96 @@ expand_scatter(const uint32_t *__restrict__ koff, const uint32_t *__restrict__ k
 }
 
 // ------------------------------------------------------------------ per-tile sort
-// Buckets are sorted by 32-bit keys first: the leading bits of (depth - the
-// bucket's smallest depth) that 32 - IB bits hold, and the key's position in
-// the bucket (IB bits, below 2^IB keys).  The order of the 64-bit keys is
-// then right but for keys whose leading bits agree (about n^2 / 2^(33 - IB)
-// pairs of evenly spread depths), which exchange places with their
-// neighbours until every pair is in order; buckets that need more than
-// kFixRounds of that (many equal depths) are sorted again by the 64-bit keys.
-// The result is the order of the 64-bit keys in every case.  A 32-bit
-// compare-exchange takes one shuffle and three instructions, a 64-bit one two
-// and seven, and a shared-memory key half the bandwidth.
+// Buckets are sorted by 32-bit keys where they can be: the leading bits of
+// (depth - the bucket's smallest depth) that 32 - IB bits hold, and the key's
+// position in the bucket (IB bits, below 2^IB keys).  The order of the 64-bit
+// keys is then right but for runs of keys whose leading bits agree (about n^2 /
+// 2^(33 - IB) pairs of evenly spread depths), inside which every key is placed
+// by its rank; a bucket with a run longer than kRunLimit is sorted again by the
+// 64-bit keys.  A bucket of many equal depths (a plane that faces the camera) is
+// sorted by those at once: it is told by the equal ones among the first keys of
+// a few warps, kTies of them or more.  The result is the order of
+// the 64-bit keys in every case.  A 32-bit compare-exchange takes one
+// shuffle and three instructions, a 64-bit one two and seven, and a
+// shared-memory key half the bandwidth.
 // Projected frames (sort stage, 64-bit network and merges -> now): 1M room at
 // 1296 x 968 157 -> 135 us, object VGA with 710 buckets of 2k-5k keys 162 ->
 // 150 us, room VGA 38 -> 37 us, 2,000 Gaussians 14.3 -> 15.4 us (the two
-// barriers of the depth range and the check).
-constexpr int kFixRounds = 16;
+// barriers of the depth range and the check).  Equal depths (64-bit alone ->
+// neighbours exchanged up to 16 times after the 32-bit sort, then the 64-bit
+// one -> now), VGA: 300k Gaussians in one plane 60 -> 101 -> 60 us, 16 planes 58 ->
+// 79 -> 60, 64 planes 58 -> 60 -> 60, a plane of every tenth Gaussian 58 -> 89 -> 64;
+// 1.5M in one plane 239 -> 525 -> 247, in 256 planes 226 -> 232 -> 236, a plane of
+// every twentieth 228 -> 379 -> 245.
+constexpr int kRunLimit = 256;
+constexpr int kTies = 4;
 
-// CTA-wide smallest value and bit length of the spread of a thread's (lo, hi).
+// CTA-wide smallest value and bit length of the spread of a thread's (lo, hi);
+// first: a depth of the bucket, or a value that is none.  Returns how many
+// threads of the first kTieWarps warps have one that another lane of their
+// warp has too (asking all warps cost 1.6 us of a VGA room's 53, these 0.2).
 template <int NTH>
-__device__ __forceinline__ void depth_span(uint32_t lo, uint32_t hi, uint32_t *s_w, uint32_t &smallest,
-                                           int &bits) {
-    lo = __reduce_min_sync(0xffffffffu, lo);
-    hi = __reduce_max_sync(0xffffffffu, hi);
-    if ((threadIdx.x & 31) == 0) {
-        s_w[threadIdx.x >> 5] = lo;
-        s_w[32 + (threadIdx.x >> 5)] = hi;
+__device__ __forceinline__ int depth_span(uint32_t lo, uint32_t hi, uint32_t first, uint32_t *s_w,
+                                          uint32_t &smallest, int &bits) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int kTieWarps = NTH / 128;
+    unsigned tied = 0u;
+    if (warp < kTieWarps) {
+        const unsigned peers = __match_any_sync(FULL, first);
+        tied = __ballot_sync(FULL, (peers & (peers - 1u)) != 0u);
+    }
+    lo = __reduce_min_sync(FULL, lo);
+    hi = __reduce_max_sync(FULL, hi);
+    if (lane == 0) {
+        s_w[warp] = lo;
+        s_w[32 + warp] = hi;
+        if (warp < kTieWarps) s_w[64 + warp] = __popc(tied);
     }
     __syncthreads();
-    const int lane = threadIdx.x & 31;
-    lo = __reduce_min_sync(0xffffffffu, lane < NTH / 32 ? s_w[lane] : 0xFFFFFFFFu);
-    hi = __reduce_max_sync(0xffffffffu, lane < NTH / 32 ? s_w[32 + lane] : 0u);
+    lo = __reduce_min_sync(FULL, lane < NTH / 32 ? s_w[lane] : 0xFFFFFFFFu);
+    hi = __reduce_max_sync(FULL, lane < NTH / 32 ? s_w[32 + lane] : 0u);
     smallest = lo;
     bits = hi > lo ? 32 - __clz(hi - lo) : 0;
+    return int(__reduce_add_sync(FULL, lane < kTieWarps ? s_w[64 + lane] : 0u));
 }
 
-// Neighbours of the n keys in s exchange places until all are in order; false
-// if kFixRounds did not suffice.  Ends with a barrier.
+// Whether the n keys in s are in order.
 template <int NTH>
-__device__ __forceinline__ bool fix_order(unsigned long long *s, int n) {
-    for (int r = 0;; ++r) {
-        bool bad = false;
-        for (int i = threadIdx.x; i + 1 < n; i += NTH) bad |= s[i] > s[i + 1];
-        if (!__syncthreads_or(bad)) return true;
-        if (r == kFixRounds) return false;
-        for (int odd = 0; odd < 2; ++odd) {
-            for (int i = 2 * int(threadIdx.x) + odd; i + 1 < n; i += 2 * NTH) {
-                const unsigned long long x = s[i], y = s[i + 1];
-                if (x > y) {
-                    s[i] = y;
-                    s[i + 1] = x;
-                }
-            }
-            __syncthreads();
+__device__ __forceinline__ bool in_order(const unsigned long long *s, int n) {
+    bool bad = false;
+    for (int i = threadIdx.x; i + 1 < n; i += NTH) bad |= s[i] > s[i + 1];
+    return !__syncthreads_or(bad);
+}
+
+// The n keys in s are in order but for runs of equal leading bits: hands each
+// key with its place, found by its rank in its run, to put(place, key); false
+// if a run is longer than kRunLimit (not every key has then got its place).
+// Ends with a barrier.
+template <int NTH, typename Put>
+__device__ __forceinline__ bool order_runs(const unsigned long long *s, int n, uint32_t smallest, int sh,
+                                           Put put) {
+    auto leading = [&](unsigned long long k) { return (uint32_t(k >> 32) - smallest) >> sh; };
+    bool too_long = false;
+    for (int i = threadIdx.x; i < n; i += NTH) {
+        const unsigned long long k = s[i];
+        const uint32_t p = leading(k);
+        int place = i;
+        for (int j = i - 1; j >= 0; --j) {
+            const unsigned long long o = s[j];
+            if (leading(o) != p) break;
+            if (i - j > kRunLimit) { too_long = true; break; }
+            place -= o > k;
         }
+        for (int j = i + 1; j < n; ++j) {
+            const unsigned long long o = s[j];
+            if (leading(o) != p) break;
+            if (j - i > kRunLimit) { too_long = true; break; }
+            place += o < k;
+        }
+        put(place, k);
     }
+    return !__syncthreads_or(too_long);
 }
 
 // A bucket of up to T * E keys: E per thread in blocked order, sorted by the
@@ -371,46 +408,52 @@ __device__ void sort_registers(const unsigned long long *__restrict__ src, int n
     constexpr int IB = 8 + (E == 8 ? 3 : E == 4 ? 2 : E == 2 ? 1 : 0);   // log2(T E)
     const int base = threadIdx.x * E;
     uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+    uint32_t first = ~threadIdx.x;   // a lane past the bucket ties with none
 #pragma unroll
     for (int e = 0; e < E; ++e) {
         const int i = int(threadIdx.x) + e * T;
         if (i < n) {
             const unsigned long long k = src[i];
+            const uint32_t d = uint32_t(k >> 32);
             s[i] = k;
-            lo = min(lo, uint32_t(k >> 32));
-            hi = max(hi, uint32_t(k >> 32));
+            if (e == 0) first = d;
+            lo = min(lo, d);
+            hi = max(hi, d);
         }
     }
     uint32_t smallest;
     int bits;
-    depth_span<T>(lo, hi, s_w, smallest, bits);   // its barrier also publishes s
-    const int sh = max(0, bits - (32 - IB));
-    uint32_t v[E];
-#pragma unroll
-    for (int e = 0; e < E; ++e)
-        v[e] = base + e < n ? (((uint32_t(s[base + e] >> 32) - smallest) >> sh) << IB) | uint32_t(base + e)
-                            : 0xFFFFFFFFu;
-    bitonic_regs<E, T, uint32_t>(v, x);
+    const int ties = depth_span<T>(lo, hi, first, s_w, smallest, bits);   // its barrier also publishes s
     unsigned long long k[E];
+    if (ties < kTies) {
+        const int sh = max(0, bits - (32 - IB));
+        uint32_t v[E];
 #pragma unroll
-    for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[v[e] & ((1u << IB) - 1u)] : ~0ull;
-    __syncthreads();
+        for (int e = 0; e < E; ++e)
+            v[e] = base + e < n ? (((uint32_t(s[base + e] >> 32) - smallest) >> sh) << IB) | uint32_t(base + e)
+                                : 0xFFFFFFFFu;
+        bitonic_regs<E, T, uint32_t>(v, x);
 #pragma unroll
-    for (int e = 0; e < E; ++e)
-        if (base + e < n) s[base + e] = k[e];
-    __syncthreads();
-    if (!fix_order<T>(s, n)) {
-#pragma unroll
-        for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[base + e] : ~0ull;
-        __syncthreads();
-        bitonic_regs<E, T, unsigned long long>(k, s);
+        for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[v[e] & ((1u << IB) - 1u)] : ~0ull;
         __syncthreads();
 #pragma unroll
         for (int e = 0; e < E; ++e)
             if (base + e < n) s[base + e] = k[e];
         __syncthreads();
+        if (in_order<T>(s, n)) {
+            for (int i = threadIdx.x; i < n; i += T) dst[i] = uint32_t(s[i]);
+            return;
+        }
+        if (order_runs<T>(s, n, smallest, sh, [&](int i, unsigned long long key) { dst[i] = uint32_t(key); }))
+            return;
     }
-    for (int i = threadIdx.x; i < n; i += T) dst[i] = uint32_t(s[i]);
+#pragma unroll
+    for (int e = 0; e < E; ++e) k[e] = base + e < n ? s[base + e] : ~0ull;
+    __syncthreads();
+    bitonic_regs<E, T, unsigned long long>(k, s);
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        if (base + e < n) dst[base + e] = uint32_t(k[e]);
 }
 
 // Merge sorted A[0,na) and B[0,nb) into C with the whole CTA of NT threads
@@ -448,7 +491,7 @@ tile_sort(const uint2 *__restrict__ ranges, unsigned long long *__restrict__ key
     pdl_wait();   // the predecessor's outputs are complete and visible
     __shared__ unsigned long long s_k[8 * T];
     __shared__ uint32_t s_x[8 * T];
-    __shared__ uint32_t s_w[64];
+    __shared__ uint32_t s_w[72];
     const uint2 r = ranges[blockIdx.x];
     const int n = int(r.y - r.x);
     if (n > 8 * T) {
@@ -605,61 +648,92 @@ __device__ uint32_t *merge_words(uint32_t *s, uint32_t *t, int n) {
     return s;
 }
 
-// Sorts the n <= BIG_CAP keys in a (unpadded; a and b hold BIG_SLOTS 64-bit
-// slots each) and returns the buffer with the sorted keys (unpadded).
-template <int E>
-__device__ unsigned long long *sort_big_bucket(unsigned long long *a, unsigned long long *b, int n,
-                                               uint32_t *s_w) {
-    constexpr int IB = 13;   // BIG_CAP positions
-    uint32_t *x = reinterpret_cast<uint32_t *>(b), *y = x + BIG_CAP + BIG_CAP / 32;
-    uint32_t lo = 0xFFFFFFFFu, hi = 0u;
+// The n <= BIG_CAP keys of src into a (unpadded; the next barrier publishes
+// them), with the thread's smallest, largest and first depth.
+__device__ __forceinline__ void load_big(const unsigned long long *src, int n,
+                                         unsigned long long *a, uint32_t &lo, uint32_t &hi, uint32_t &first) {
+    lo = 0xFFFFFFFFu;
+    hi = 0u;
+    first = ~threadIdx.x;
     for (int i = threadIdx.x; i < n; i += TB) {
-        const uint32_t d = uint32_t(a[i] >> 32);
+        const unsigned long long k = src[i];
+        const uint32_t d = uint32_t(k >> 32);
+        a[i] = k;
+        if (i < TB) first = d;
         lo = min(lo, d);
         hi = max(hi, d);
     }
+}
+
+// Sorts the n <= BIG_CAP keys that load_big has put into a (a and b hold
+// BIG_SLOTS 64-bit slots each) and returns the buffer with the sorted keys
+// (unpadded).
+template <int E>
+__device__ unsigned long long *sort_big_bucket(unsigned long long *a, unsigned long long *b, int n,
+                                               uint32_t lo, uint32_t hi, uint32_t first, uint32_t *s_w) {
+    constexpr int IB = 13;   // BIG_CAP positions
+    uint32_t *x = reinterpret_cast<uint32_t *>(b), *y = x + BIG_CAP + BIG_CAP / 32;
     uint32_t smallest;
     int bits;
-    depth_span<TB>(lo, hi, s_w, smallest, bits);
-    const int sh = max(0, bits - (32 - IB));
-    for (int r0 = int(threadIdx.x) * 8; r0 < n; r0 += TB * 8) {
-        uint32_t v[8];
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            v[e] = r0 + e < n ? (((uint32_t(a[r0 + e] >> 32) - smallest) >> sh) << IB) | uint32_t(r0 + e)
-                              : 0xFFFFFFFFu;
-        sort8(v);
-#pragma unroll
-        for (int e = 0; e < 8; ++e)
-            if (r0 + e < n) x[pad32(r0 + e)] = v[e];
-    }
-    __syncthreads();
-    const uint32_t *o = merge_words<E>(x, y, n);
+    const int ties = depth_span<TB>(lo, hi, first, s_w, smallest, bits);
     unsigned long long k[E];
+    if (ties < kTies) {
+        const int sh = max(0, bits - (32 - IB));
+        for (int r0 = int(threadIdx.x) * 8; r0 < n; r0 += TB * 8) {
+            uint32_t v[8];
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = int(threadIdx.x) + e * TB;
-        k[e] = i < n ? a[o[pad32(i)] & ((1u << IB) - 1u)] : 0ull;
-    }
-    __syncthreads();
+            for (int e = 0; e < 8; ++e)
+                v[e] = r0 + e < n ? (((uint32_t(a[r0 + e] >> 32) - smallest) >> sh) << IB) | uint32_t(r0 + e)
+                                  : 0xFFFFFFFFu;
+            sort8(v);
 #pragma unroll
-    for (int e = 0; e < E; ++e) {
-        const int i = int(threadIdx.x) + e * TB;
-        if (i < n) b[i] = k[e];
+            for (int e = 0; e < 8; ++e)
+                if (r0 + e < n) x[pad32(r0 + e)] = v[e];
+        }
+        __syncthreads();
+        const uint32_t *o = merge_words<E>(x, y, n);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = int(threadIdx.x) + e * TB;
+            k[e] = i < n ? a[o[pad32(i)] & ((1u << IB) - 1u)] : 0ull;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = int(threadIdx.x) + e * TB;
+            if (i < n) b[i] = k[e];
+        }
+        __syncthreads();
+        if (in_order<TB>(b, n)) return b;
+        if (order_runs<TB>(b, n, smallest, sh, [&](int i, unsigned long long key) { a[i] = key; })) return a;
+        for (int i = threadIdx.x; i < n; i += TB) a[pad(i)] = b[i];
+    } else {
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = int(threadIdx.x) + e * TB;
+            k[e] = i < n ? a[i] : 0ull;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int i = int(threadIdx.x) + e * TB;
+            if (i < n) a[pad(i)] = k[e];
+        }
     }
-    __syncthreads();
-    if (fix_order<TB>(b, n)) return b;
-    for (int i = threadIdx.x; i < n; i += TB) a[pad(i)] = b[i];
     __syncthreads();
     unsigned long long *q = sort_smem<E>(a, b, n), *t = q == a ? b : a;
     for (int i = threadIdx.x; i < n; i += TB) t[i] = q[pad(i)];
     __syncthreads();
     return t;
 }
-__device__ __forceinline__ unsigned long long *sort_big_any(unsigned long long *a, unsigned long long *b,
+// load_big and sort_big_bucket.
+__device__ __forceinline__ unsigned long long *sort_big_any(const unsigned long long *src,
+                                                            unsigned long long *a, unsigned long long *b,
                                                             int n, uint32_t *s_w) {
-    if (n <= TB * 4) return sort_big_bucket<4>(a, b, n, s_w);
-    return sort_big_bucket<8>(a, b, n, s_w);
+    uint32_t lo, hi, first;
+    load_big(src, n, a, lo, hi, first);
+    if (n <= TB * 4) return sort_big_bucket<4>(a, b, n, lo, hi, first, s_w);
+    return sort_big_bucket<8>(a, b, n, lo, hi, first, s_w);
 }
 
 // The buckets of more than 8 T keys, listed by tile_sort: persistent CTAs of
@@ -674,7 +748,7 @@ tile_sort_big(const uint2 *__restrict__ ranges, unsigned long long *__restrict__
               const uint32_t *__restrict__ big, const uint32_t *__restrict__ counters) {
     pdl_wait();   // the predecessor's outputs are complete and visible
     extern __shared__ unsigned long long s_k[];   // 2 x BIG_SLOTS
-    __shared__ uint32_t s_w[64];
+    __shared__ uint32_t s_w[72];
     unsigned long long *s_t = s_k + BIG_SLOTS;
     const uint32_t nbig = counters[CNT_BIG];
     for (uint32_t bi = blockIdx.x; bi < nbig; bi += gridDim.x) {
@@ -682,18 +756,14 @@ tile_sort_big(const uint2 *__restrict__ ranges, unsigned long long *__restrict__
         const int n = int(r.y - r.x);
         unsigned long long *src = keys + r.x;
         if (n <= BIG_CAP) {
-            for (int i = threadIdx.x; i < n; i += TB) s_k[i] = src[i];
-            __syncthreads();
-            const unsigned long long *o = sort_big_any(s_k, s_t, n, s_w);
+            const unsigned long long *o = sort_big_any(src, s_k, s_t, n, s_w);
             for (int i = threadIdx.x; i < n; i += TB) igid[r.x + i] = uint32_t(o[i]);
             __syncthreads();
             continue;
         }
         for (int c0 = 0; c0 < n; c0 += BIG_CAP) {
             const int m = min(BIG_CAP, n - c0);
-            for (int i = threadIdx.x; i < m; i += TB) s_k[i] = src[c0 + i];
-            __syncthreads();
-            const unsigned long long *o = sort_big_any(s_k, s_t, m, s_w);
+            const unsigned long long *o = sort_big_any(src + c0, s_k, s_t, m, s_w);
             for (int i = threadIdx.x; i < m; i += TB) src[c0 + i] = o[i];
             __syncthreads();
         }

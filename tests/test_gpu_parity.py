@@ -248,6 +248,36 @@ def test_tile_sort_equal_and_narrow_depths(n, depths):
         assert len(set(gids[a:b].tolist())) == b - a
 
 
+@pytest.mark.parametrize("n", [300, 2048, 2049, 8192, 9000])
+@pytest.mark.parametrize("run", [2, 256, 257, 258])
+@pytest.mark.parametrize("ulps", [1, 16])
+def test_tile_sort_runs_of_close_depths(n, run, ulps):
+    """One run of keys whose leading bits agree, at the longest length that is
+    placed by rank and beside it, among distinct depths: equal depths, or 16
+    values that a far Gaussian leaves the 32-bit keys no bits for."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    g, _ = _slab_scene(n)
+    rng = np.random.default_rng(n + run)
+    z = rng.permutation(n) * (1.0 / n) + 0.25
+    at = rng.choice(n, run, replace=False)
+    z[at] = rng.integers(0, ulps, run) * 2.0 ** -21
+    if ulps > 1:
+        z[np.setdiff1d(np.arange(n), at)[0]] = -50.0
+    g.mean[:, 2] = z
+    fr = H.run_gpu(g, None, scenes.tiny_camera(48, 48), K=8, dense=False)["frame"]
+    v = q.qr_frame_view_get(fr)
+    tiles = fr.frame.tiles_x * fr.frame.tiles_y
+    rngs = _device_copy(v.tile_range, 2 * tiles, torch.int32).cpu().numpy().reshape(tiles, 2)
+    gkey = _device_copy(v.depth_key, n, torch.int32).cpu().numpy().view(np.float32)
+    gids = _device_copy(v.isect_gid, int(rngs[-1, 1]), torch.int32).cpu().numpy()
+    assert (rngs[:, 1] - rngs[:, 0]).max() >= 0.9 * n - 1
+    assert len(np.unique(gkey[at])) <= ulps
+    for a, b in rngs:
+        np.testing.assert_array_equal(np.lexsort((gids[a:b], gkey[gids[a:b]])), np.arange(b - a))
+        assert len(set(gids[a:b].tolist())) == b - a
+
+
 @pytest.mark.parametrize("C", [16, 64, 512])
 def test_blend_stage_matches_definition(C):
     import torch
