@@ -983,16 +983,23 @@ void launch_bwd_pixel(const qr_frame &f, const void *feat, const float *scale, i
             static_cast<const unsigned char *>(feat), scale, C, ids, w, cnt, g, P, f.params.K,
             f.camera.width, f.params.alpha_max, E, pl);
     };
-    // four pixels' rows of up to 16 channels per lane fit a warp's registers
+    // four pixels' rows of up to 16 channels per lane fit a warp's registers; a
+    // CTA takes a strip of 16 x 8 pixels, so images of fewer than two strips per
+    // SM keep the warp per pixel (the whole backward with groups / without, us:
+    // object 64 x 48, 24 strips, 256 BF16 channels 380 / 338, 512 FP32 567 / 525;
+    // object 160 x 120, 150 strips 278 / 259, 400 / 387; 200 x 150, 247 strips,
+    // object 263 / 252, 375 / 370, room 146 / 150, 208 / 217; 240 x 180, 345 strips,
+    // object 271 / 268, 393 / 394, room 168 / 169, 239 / 241; room 320 x 240 170 /
+    // 184, 235 / 253)
+    const unsigned strips = unsigned((f.camera.width + 15) / 16) * unsigned((f.camera.height + 7) / 8);
     auto group = [&](auto kern) {
-        const unsigned strips = unsigned((f.camera.width + 15) / 16) * unsigned((f.camera.height + 7) / 8);
         kern<<<strips, T, 0, s>>>(
             slot<float4>(f, S_REC_M), slot<float4>(f, S_REC_C), slot<float>(f, S_REC_A),
             static_cast<const unsigned char *>(feat), scale, C, ids, w, cnt, g, f.params.K,
             f.camera.width, f.camera.height, f.params.alpha_max, E);
     };
     constexpr int CPV = VecB<DT>::C;
-    if (!loss && f.params.K <= 8 && vpl > 0 && vpl * CPV <= 16) {
+    if (!loss && f.params.K <= 8 && vpl > 0 && vpl * CPV <= 16 && strips >= 2u * unsigned(sms_now())) {
         if (vpl == 1) group(bwd_group<DT, 1>);
         if constexpr (CPV <= 8)
             if (vpl == 2) group(bwd_group<DT, 2>);

@@ -161,6 +161,35 @@ def test_backward_pixel_groups(kind, C, K):
     _check_all(got, ref)
 
 
+@pytest.mark.parametrize("kind,C,K", [("f32", 128, 8), ("f32", 256, 1), ("f32", 512, 3), ("bf16", 256, 5),
+                                      ("bf16", 512, 8), ("fp8", 512, 7)])
+def test_backward_pixel_groups_larger_image(kind, C, K):
+    """As above on an odd image of more than two 16 x 8 strips per SM, which
+    take the pixel groups (smaller ones a warp per pixel)."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    cam = scenes.room_camera(289, 133)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert -(-cam.width // 16) * -(-cam.height // 8) >= 2 * sms
+    g, f = H.small_room(n=20000, channels=C)
+    fdev = torch.from_numpy(f).cuda()
+    table, scale, decoded = fdev, None, f
+    if kind == "bf16":
+        table, decoded = q.qr_quantize_bf16(fdev), oracle.bf16_decode(oracle.bf16_encode(f))
+    elif kind == "fp8":
+        (table, scale), decoded = q.qr_quantize_fp8(fdev), oracle.fp8_dequantize_rows(*oracle.fp8_quantize_rows(f))
+    res = q.render_frame(q.gaussians_to_device(g), None, cam, K=K)
+    pr, pix, ref = H.run_oracle(g, decoded, cam, K)
+    gout = np.random.default_rng(C + K).normal(size=(cam.width * cam.height, C)).astype(np.float32)
+    gout[(ref.tie & compare.Q_TIE_BITS) != 0] = 0.0
+    got = q.qr_backward(res["frame"], table, scale, res["ids"], res["weights"], res["counts"],
+                        torch.from_numpy(gout).cuda())
+    got = tuple(x.cpu().numpy() for x in got)
+    ref = oracle.backward(pr, decoded, K, pix, gout.astype(np.float64), alpha_min=oracle.ALPHA_MIN_F32,
+                          alpha_max=oracle.ALPHA_MAX_F32, with_scales=True)
+    _check_all(got, ref)
+
+
 @pytest.mark.parametrize("C,K", [(64, 16), (136, 8), (512, 8)])
 def test_backward_bf16_gradient_is_the_rounded_one(C, K):
     import torch
