@@ -310,10 +310,10 @@ qr_status qr_batch_prepare(const qr_view *views, int32_t n_views, void *ws, size
  * same per-channel sums as qr_blend with width > 0; ids/weights/counts are
  * also written).  dtype and C are shared by the batch (rows of 32, 64 or 128
  * sixteen-byte vectors: e.g. 512-D F32 / BF16 / FP8); group = pixels per
- * warp in the blend (4, 2 or 1; 0 = largest allowed by K); chunks = channel
- * slices per feature row for groups of 4, taken by different blend warps
- * (1, 2 or 4 dividing C / 128 and leaving at most 512 channels per slice;
- * 0 = the built-in choice);
+ * warp in the blend (4; 2 where K <= 16; 1; 0 = 4, as qr_blend); chunks =
+ * channel slices per feature row for K <= 8 and groups of 4, one after the
+ * other (1, 2 or 4 dividing C / 128 and leaving at most 512 channels per
+ * slice; 0 = the built-in choice);
  * blend_warps = blend warps per CTA beside the four selection warps (4 or 8;
  * 0 = 8); ctas_per_sm caps the resident CTAs per SM (0 = occupancy limit).
  * Results do not depend on group size or chunks beyond the summation order

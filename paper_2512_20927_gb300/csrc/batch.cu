@@ -12,12 +12,14 @@
 //      each warp walks an 8 x 8 block of the tile on its own; the kept ids and
 //      normalised weights go to one of two shared-memory buffers and are also
 //      written out (coalesced runs) for a backward pass;
-//   2. blend (8 warps, warp per 2x2 / 2x1 pixel group, one channel chunk of the
-//      rows after the other, like qr_blend): equal ids of the group are merged with __match_any_sync, the
-//      group's weights of each distinct row are gathered into a per-warp
-//      table, each distinct feature row (or its chunk) is read once with
-//      16-byte loads and accumulated into every pixel of the group, and the
-//      rows of the map are written with streaming stores.
+//   2. blend (8 warps, warp per 2x2 pixel group whatever K is, as in qr_blend, one
+//      channel chunk of the rows after the other): equal ids of the group are
+//      merged with __match_any_sync, the group's weights of each distinct row
+//      are gathered into a per-warp table, each distinct feature row (or its
+//      chunk) is read once with 16-byte loads and accumulated into every pixel
+//      of the group, and the rows of the map are written with streaming
+//      stores.  The same groups and the same order of rows make the map of 16 x
+//      16 tiles qr_blend's bit for bit.
 // Hand-over between the roles uses named barriers (below).  Per-view
 // descriptors live in device memory (qr_batch_prepare), the counter is
 // cleared by a memset on the stream, so the launch can sit in a CUDA graph.
@@ -25,6 +27,11 @@
 // of two rooms (5.0M pixels, 512 BF16 channels, 10.3 GB of maps) 2,025 us with
 // the group's table built for every channel chunk, 1,895 us with one table
 // for all of a group's chunks (0.80 of a plain copy's rate).
+// K > 8, two pixels (K <= 16) or one per group -> four, us, six views of a 200k
+// room, scores not asked for: 512 FP32 channels K = 9 2298 -> 2086, K = 16 2997 ->
+// 2812, K = 17 4643 -> 2958, K = 24 6395 -> 4760, K = 32 8837 -> 5761; 512 BF16 K =
+// 16 2596 -> 2447, K = 32 8279 -> 5377; 128 FP32 K = 16 1418 -> 1322, K = 24 2654 ->
+// 2605 (the larger tables leave one CTA per SM from K = 24 on), K = 32 3801 -> 3014.
 #include <type_traits>
 
 #include <cuda_bf16.h>
@@ -113,16 +120,21 @@ __device__ __forceinline__ int find_view(const BatchView *views, int n_views, ui
 }
 
 // Dynamic shared memory: ids [2][256][KSB] int32, weights [2][256][KSB] float.
-// QPL quads (4 channels) per lane per channel chunk, NCH chunks per row.
-template <int DT, int QPL, int G, int NCH>
+// QPL quads (4 channels) per lane per channel chunk, NCH chunks per row, EPL of
+// a pixel group's G K entries per lane (lane l holds entries l, l + 32, ...), as
+// in qr_blend's kernel.
+template <int DT, int QPL, int G, int NCH, int EPL>
 __global__ void __launch_bounds__(kBT, DT == QR_FP8E4M3 ? 1 : 2)
 batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_items,
              uint32_t *__restrict__ counter, int KSB) {
     __shared__ SelStage st[kSelThreads / 32];
     __shared__ float s_thr[kKMax + 1];
     __shared__ int s_item[2];
-    __shared__ __align__(16) float s_tw[kNBW][32][G];   // per blend warp: row-weight table
-    __shared__ int s_tid[kNBW][32];
+    // per blend warp: row-weight table.  92 rows, not 96, for three entries per
+    // lane: with K = 22 or 23 two CTAs share an SM's memory then
+    constexpr int ROWS = EPL == 3 ? 92 : 32 * EPL;
+    __shared__ __align__(16) float s_tw[kNBW][ROWS][G];
+    __shared__ int s_tid[kNBW][ROWS];
     extern __shared__ __align__(16) unsigned char s_dyn[];
     int32_t *s_ids0 = reinterpret_cast<int32_t *>(s_dyn);
     float *s_w0 = reinterpret_cast<float *>(s_dyn) + 2 * kSelPix * KSB;
@@ -197,37 +209,78 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
         const int tile_w = V.tile_w, tile_h = kSelPix / tile_w;
         const int half_w = tile_w / 2;
         const unsigned char *feat = V.feat;
-        const int mm = lane / K, j = lane - mm * K;
+        int mm[EPL], j[EPL];   // pixel of the group and entry that the lane holds
+#pragma unroll
+        for (int h = 0; h < EPL; ++h) {
+            mm[h] = (lane + 32 * h) / K;
+            j[h] = lane + 32 * h - mm[h] * K;
+        }
         for (int gi = bw; gi < kSelPix / G; gi += nbw) {
-            int lx, ly;
-            if (G == 4) { lx = 2 * (gi % half_w) + (mm & 1); ly = 2 * (gi / half_w) + (mm >> 1); }
-            else if (G == 2) { lx = 2 * (gi % half_w) + mm; ly = gi / half_w; }
-            else { lx = gi % tile_w; ly = gi / tile_w; }
-            const int loc = ly * tile_w + lx;
-            const int px = tx * tile_w + lx, py = ty * tile_h + ly;
-            int64_t p = -1;
-            if (mm < G && px < V.W && py < V.H) p = int64_t(py) * V.W + px;
-            int id = -1;
-            float w = 0.f;
-            if (p >= 0) {
-                id = s_ids[loc * KSB + j];
-                w = s_w[loc * KSB + j];
+            // pixel m of the group: place in the tile, number in the image (-1: none)
+            auto pixel = [&](int m, int &loc) -> int64_t {
+                int lx, ly;
+                if (G == 4) { lx = 2 * (gi % half_w) + (m & 1); ly = 2 * (gi / half_w) + (m >> 1); }
+                else if (G == 2) { lx = 2 * (gi % half_w) + m; ly = gi / half_w; }
+                else { lx = gi % tile_w; ly = gi / tile_w; }
+                loc = ly * tile_w + lx;
+                const int px = tx * tile_w + lx, py = ty * tile_h + ly;
+                int64_t p = -1;
+                if (m < G && px < V.W && py < V.H) p = int64_t(py) * V.W + px;
+                return p;
+            };
+            int64_t p = -1;   // pixel g in lane g K (one entry per lane) or g
+            int id[EPL];
+            float w[EPL];
+#pragma unroll
+            for (int h = 0; h < EPL; ++h) {
+                int loc;
+                const int64_t ph = pixel(mm[h], loc);
+                if (EPL == 1) p = ph;
+                id[h] = -1;
+                w[h] = 0.f;
+                if (ph >= 0) {
+                    id[h] = s_ids[loc * KSB + j[h]];
+                    w[h] = s_w[loc * KSB + j[h]];
+                }
             }
-            const unsigned peers = __match_any_sync(FULL, id);
-            const int leader = __ffs(peers) - 1;
-            const unsigned leaders = __ballot_sync(FULL, id >= 0 && lane == leader);
-            const int nrows = __popc(leaders);
+            if (EPL > 1) {
+                int loc;
+                p = pixel(lane, loc);
+            }
             // the G weights of each distinct row, gathered once (a pixel that
             // lists an id twice gets the sum)
+            unsigned peers = __match_any_sync(FULL, id[0]);
+            int leader = __ffs(peers) - 1;
+            unsigned fresh = __ballot_sync(FULL, id[0] >= 0 && lane == leader);
+            int nrows = __popc(fresh);
 #pragma unroll
-            for (int g = 0; g < G; ++g) s_tw[bw][lane][g] = 0.f;
+            for (int h = 0; h < EPL; ++h)
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    if (32 * h + 32 <= ROWS || lane + 32 * h < ROWS) s_tw[bw][lane + 32 * h][g] = 0.f;
             __syncwarp();
-            if (id >= 0) {
-                const int slot = __popc(leaders & ((1u << leader) - 1u));
-                atomicAdd(&s_tw[bw][slot][mm], w);
-                if (lane == leader) s_tid[bw][slot] = id;
+            if (id[0] >= 0) {
+                const int slot = __popc(fresh & ((1u << leader) - 1u));
+                atomicAdd(&s_tw[bw][slot][mm[0]], w[0]);
+                if (lane == leader) s_tid[bw][slot] = id[0];
             }
             __syncwarp();
+#pragma unroll
+            for (int h = 1; h < EPL; ++h) {   // further entries: among the rows so far, or new ones
+                int slot = -1;
+                for (int k = 0; k < nrows; ++k)
+                    if (s_tid[bw][k] == id[h]) slot = k;
+                peers = __match_any_sync(FULL, id[h]);
+                leader = __ffs(peers) - 1;
+                fresh = __ballot_sync(FULL, id[h] >= 0 && slot < 0 && lane == leader);
+                if (slot < 0) slot = nrows + __popc(fresh & ((1u << leader) - 1u));
+                if (id[h] >= 0) {
+                    atomicAdd(&s_tw[bw][slot][mm[h]], w[h]);
+                    if ((fresh >> lane) & 1u) s_tid[bw][slot] = id[h];
+                }
+                nrows += __popc(fresh);
+                __syncwarp();
+            }
 #pragma unroll 1
             for (int ch = 0; ch < NCH; ++ch) {   // the group's table serves every chunk
                 float acc[G][QPL][4];
@@ -274,7 +327,7 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
                 }
 #pragma unroll
                 for (int g = 0; g < G; ++g) {
-                    const int64_t pg = __shfl_sync(FULL, p, g * K < 32 ? g * K : 0);
+                    const int64_t pg = __shfl_sync(FULL, p, EPL == 1 ? (g * K < 32 ? g * K : 0) : g);
                     if (pg >= 0) {
                         float4 *o = reinterpret_cast<float4 *>(V.out) + pg * int64_t(ROWQ) + ch * CQ + lane;
 #pragma unroll
@@ -290,10 +343,10 @@ batch_kernel(const BatchView *__restrict__ views, int n_views, uint32_t total_it
     }
 }
 
-template <int DT, int QT, int G, int NCH>
+template <int DT, int QT, int G, int NCH, int EPL = 1>
 cudaError_t run_batch(const BatchView *dviews, int n_views, uint32_t total, uint32_t *counter,
                       int K, int nbw, int ctas_per_sm, cudaStream_t s) {
-    auto kern = batch_kernel<DT, QT / NCH, G, NCH>;
+    auto kern = batch_kernel<DT, QT / NCH, G, NCH, EPL>;
     const int KSB = K | 1;
     const int nt = kSelThreads + 32 * nbw;
     const size_t dyn = size_t(KSB) * kSelPix * 2 * 8;
@@ -321,15 +374,20 @@ constexpr int batch_default_chunks() {
 }
 
 // QT = C / 128 quads per lane over the whole row (1 .. 16).  group picks the
-// pixel-group size (0 = largest allowed by K), chunks the channel chunks per
-// row for groups of 4 (0 = default; 1, 2, 4 where they divide QT and leave at
-// most 4 quads per lane).
+// pixel-group size (0 = 4), chunks the channel chunks per row for groups of 4
+// and K <= 8 (0 = default; 1, 2, 4 where they divide QT and leave at most 4
+// quads per lane).
 template <int DT, int QT>
 cudaError_t pick(const BatchView *d, int n, uint32_t total, uint32_t *counter, int K, int group,
                  int chunks, int nbw, int ctas, cudaStream_t s) {
     constexpr int DEF = batch_default_chunks<QT>();
-    const int g = group > 0 ? group : (K <= 8 ? 4 : K <= 16 ? 2 : 1);
-    if (g == 4 && K <= 8) {
+    const int g = group > 0 ? group : 4;
+    if (g == 4 && K > 8) {
+        if (K <= 16) return run_batch<DT, QT, 4, DEF, 2>(d, n, total, counter, K, nbw, ctas, s);
+        if (K <= 23) return run_batch<DT, QT, 4, DEF, 3>(d, n, total, counter, K, nbw, ctas, s);
+        return run_batch<DT, QT, 4, DEF, 4>(d, n, total, counter, K, nbw, ctas, s);
+    }
+    if (g == 4) {
         const int c = chunks > 0 ? chunks : DEF;
         if constexpr (QT <= 4)
             if (c == 1) return run_batch<DT, QT, 4, 1>(d, n, total, counter, K, nbw, ctas, s);

@@ -155,3 +155,37 @@ def test_batch_chunks_and_blend_warps_bit_identical(dtype, channels):
         q.qr_blend(tab, None, ref[i]["ids"], ref[i]["weights"], ref[i]["counts"], tiled,
                    width=cam.width)
         assert torch.equal(tiled, ref[i]["out"]), i
+
+
+@pytest.mark.parametrize("dtype,channels", [("f32", 256), ("bf16", 512), ("fp8", 512)])
+@pytest.mark.parametrize("K", [9, 12, 16, 17, 23, 24, 32])
+def test_batch_of_many_entries_equals_the_tiled_blend(dtype, channels, K):
+    """More than 32 entries per 2 x 2 pixels: the groups, and so the sums, are
+    qr_blend's over 16 x 16 tiles, bit for bit; two pixels or one per group
+    change the order of a pixel's rows only."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    from paper_2512_20927_gb300.batch import Batch, Scene
+    g, f = scenes.room_scene(seed=2, n=40000, channels=channels)
+    g.opacity *= 0.3                       # more members per pixel
+    fdev = torch.from_numpy(f).cuda()
+    tab = {"f32": lambda x: x, "bf16": q.qr_quantize_bf16, "fp8": q.qr_quantize_fp8}[dtype](fdev)
+    feat, scale = tab if isinstance(tab, tuple) else (tab, None)
+    views = [(0, scenes.room_camera(150, 110)), (0, scenes.room_camera(33, 17, yaw=2.5))]
+    sc = [Scene(q.gaussians_to_device(g), tab)]
+    b, two, one = (Batch(sc, views, K=K, group=n) for n in (0, 2, 1))
+    for x in (b, two, one):
+        x.step()
+    torch.cuda.synchronize()
+    assert all(c == q.QR_OK for c in b.status()[0])
+    for i, (_, cam) in enumerate(views):
+        got = b.view_slice(i)
+        tiled = torch.empty_like(got["out"])
+        q.qr_blend(feat, scale, got["ids"], got["weights"], got["counts"], tiled, width=cam.width)
+        assert torch.equal(got["out"], tiled), i
+        for x in (two, one):
+            other = x.view_slice(i)
+            for k in ("ids", "weights", "counts"):
+                assert torch.equal(got[k], other[k]), k
+            torch.testing.assert_close(other["out"], got["out"], rtol=1e-5, atol=1e-6)
+    assert int(b.view_slice(0)["counts"].max()) > 6
