@@ -27,13 +27,18 @@
 // (64 registers) instead of 24 cost up to 13 %.
 // Where latency bounds it, a warp takes half a block (8 x 4 pixels, one per
 // lane): each step of its chain is shorter, the list is culled twice as often.
-// That is so for images of few blocks and where lists are long, for which the
-// capacity of the lists per tile stands (the host does not know their lengths;
-// a caller sizes it by the frame's intersections).  Whole blocks / halves, K =
-// 8 unless stated: 2,000 Gaussians at 128 x 128 25 / 17 us, room at 320 x 240 23 /
-// 19, at 480 x 360 23 / 25, at 640 x 480 31 / 33, 1M room at 1296 x 968 85 / 109;
-// object (2,500 entries per tile at VGA) at 320 x 240 167 / 117, at 640 x 480
-// 130 / 115 (K = 16: 165 / 134, K = 32: 206 / 189), at 1000 x 700 127 / 122.
+// That is so for images of few blocks, and where walks are long: an object's
+// silhouette, not a room, whose walks end at its surfaces.  The host knows
+// neither; it takes a capacity of 2,048 entries per tile for long lists, but for
+// K <= 8 on images so large that whole blocks fill the chip many times over.
+// Whole blocks / halves, us, K = 8 and 16: 2,000 Gaussians at 128 x 128 25 / 17;
+// VGA, object of 50k Gaussians (227 entries per tile) 52 / 49, 68 / 60, 200k (912)
+// 87 / 75, 113 / 91, 500k (2,279) 135 / 122, 176 / 142; VGA, room of 500k (456) 39 / 41,
+// 54 / 50, 2M (1,782) 42 / 46, 54 / 55; 1000 x 700, object of 500k 134 / 130, 176 / 156;
+// 1296 x 968, room of 1M 92 / 116, 141 / 150, 3M 101 / 129, 154 / 168, object of 1M 201 /
+// 216, 301 / 277.  So a guess that is wrong, as for a room with capacity to
+// spare (render_frame's default of 8 entries per Gaussian), costs up to a
+// tenth up to VGA.
 // Halving only the blocks of long lists (the second halves' CTAs leave early
 // elsewhere) cost 2-9 us wherever lists are short.
 #include "select_tile.cuh"
@@ -41,8 +46,10 @@
 namespace qr {
 namespace {
 
-// 8 x 8 blocks up to which, and capacity per tile from which, blocks are halved
+// 8 x 8 blocks up to which blocks are halved; capacity per tile from which they
+// are too, for K <= 8 up to kManyBlocks of them
 constexpr int kSmallBlocks = 152 * 8;
+constexpr int kManyBlocks = 152 * 100;
 constexpr int64_t kLongLists = 2048;
 
 // One CTA of one warp per 8 x (4 PX) pixels.
@@ -109,7 +116,8 @@ cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cn
                           f.params.alpha_max, ids, w, cnt, vec);
     };
     cudaError_t e;
-    if (tiles * 4 <= kSmallBlocks || f.max_isect >= kLongLists * tiles)
+    const bool many = K <= 8 && tiles * 4 > kManyBlocks;
+    if (tiles * 4 <= kSmallBlocks || (!many && f.max_isect >= kLongLists * tiles))
         e = riemann ? go(select_kernel<true, 1>, 1) : go(select_kernel<false, 1>, 1);
     else
         e = riemann ? go(select_kernel<true, 2>, 2) : go(select_kernel<false, 2>, 2);

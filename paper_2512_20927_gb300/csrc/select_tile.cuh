@@ -13,9 +13,9 @@
 //   stop once T_test < 1/(K+1) = tau_{K-1}, i.e. when k reaches K; otherwise
 //   T = T_test.
 //
-// What bounds it: instruction issue where every SM has 32 warps (a VGA frame
-// is one wave), and the latency of the longest lists' chain of steps where it
-// has not (a thumbnail, a silhouette tile).  Hence:
+// What bounds it: instruction issue where every SM has its 24 warps (a VGA frame
+// is little more than one wave), and the latency of the longest lists' chain
+// of steps where it has not (a thumbnail, a silhouette tile).  Hence:
 //   * A warp works alone: it owns an 8 x 8 block (two vertically adjacent
 //     pixels per lane), stages the tile's list for itself and stops when its
 //     own 64 pixels have stopped; no CTA barrier ties it to the other warps
