@@ -521,12 +521,14 @@ uint64_t qr_launch_count(void);
 /* Test hook for the device-side error path.  The relevance kernels
  * (qr_relevance's TMA kernel, qr_blend_relevance) and qr_dense's block kernel
  * bound each of their waits on another role or the tensor cores to a number
- * of polls (2^26 by default, seconds); when one runs out the CTA stops every
- * role, waits (with the default bound) for its own copies and MMAs in flight,
- * frees its tensor memory and writes QR_ERR_DEVICE_TIMEOUT to the call's
- * status word (qr_dense: the frame's).  qr_set_wait_limit(polls) sets that bound for the launches
- * that follow (0 restores the default), so a test can make a wait run out
- * without anything hanging.  Not for production use; not thread-safe. */
+ * of polls (2^26 by default, seconds; qr_dense rounds it down to a multiple
+ * of 1,024, so that below it every wait gives up); when one runs out the CTA
+ * stops every role, waits (with the default bound) for its own copies and
+ * MMAs in flight, frees its tensor memory and writes QR_ERR_DEVICE_TIMEOUT to
+ * the call's status word (qr_dense: the frame's).  qr_set_wait_limit(polls)
+ * sets that bound for the launches that follow (0 restores the default), so a
+ * test can make a wait run out without anything hanging.  Not for production
+ * use; not thread-safe. */
 void qr_set_wait_limit(uint32_t polls);
 
 /* Tuning: the blend of 512-D rows (any dtype) with K <= 8 splits each

@@ -270,12 +270,14 @@ constexpr size_t kDenseShared = (sizeof(DenseShared) + 127) / 128 * 128;
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(tma_smem_addr(bar)) : "memory");
 }
-// Wait bounded to `limit` polls (wait_limit(): at most 2^31, so that i does not
-// wrap); false when it ran out or another role has given up.
+// Wait bounded to `rounds` rounds of polls; false when it ran out or another role
+// has given up.  (A round of a length known only at run time cost the kernel
+// 5-15 us: the room below 557 -> 571.)
+constexpr unsigned kPolls = 1024;
 __device__ __forceinline__ bool dense_wait(uint64_t *bar, uint32_t parity, volatile int *abort,
-                                           unsigned limit) {
-    for (unsigned i = 0; i < limit; i += 1024) {
-        if (tma_mbar_wait(bar, parity, min(limit - i, 1024u))) return true;
+                                           unsigned rounds) {
+    for (unsigned i = 0; i < rounds; ++i) {
+        if (tma_mbar_wait(bar, parity, kPolls)) return true;
         if (*abort) return false;
     }
     *abort = 1;
@@ -330,7 +332,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                    int H, int tile_w, int tiles_x, float alpha_min, float alpha_max, float T_min,
                    float *__restrict__ out, float *__restrict__ T_final,
                    unsigned long long *__restrict__ stats, uint32_t *__restrict__ counters,
-                   unsigned limit) {
+                   unsigned rounds) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int QB = Quad<DT>::B;
     constexpr int WPG = dense_wpg(C), QPT = dense_qpt(C);
@@ -378,7 +380,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
         for (uint32_t it = 0;; ++it) {
             const uint32_t r = it % kRows, ph = (it / kRows) & 1u;
             // one verdict per warp: its lanes meet again below
-            if (!__all_sync(FULL, dense_wait(&sh.r_full[r], ph, abort, limit))) break;
+            if (!__all_sync(FULL, dense_wait(&sh.r_full[r], ph, abort, rounds))) break;
             const DenseRow &R = sh.row[r];
             const int block = R.block, last = R.last, at = R.slot;
             if (block == kItemEnd) break;
@@ -441,7 +443,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
         bool ok = true;
         auto open = [&]() {
             if (e >= 0) return;
-            ok = ok && dense_wait(&sh.w_empty[p][sc % kSlots], ((sc / kSlots) & 1u) ^ 1u, abort, limit);
+            ok = ok && dense_wait(&sh.w_empty[p][sc % kSlots], ((sc / kSlots) & 1u) ^ 1u, abort, rounds);
             ok = __all_sync(FULL, ok);
             e = 0;
             gmask = 0;
@@ -460,7 +462,7 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
             e = -1;
         };
         for (uint32_t j = 0; ok; ++j) {
-            ok = __all_sync(FULL, dense_wait(&sh.mail_full[p], j & 1u, abort, limit));
+            ok = __all_sync(FULL, dense_wait(&sh.mail_full[p], j & 1u, abort, rounds));
             if (!ok) break;
             const int block = sh.mail[p];
             __syncwarp();
@@ -474,11 +476,11 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                     tma_expect_tx(&sh.clc, 16);
                     try_cancel(&sh.response, &sh.clc);
-                    ok = dense_wait(&sh.clc, i & 1u, abort, limit);
+                    ok = dense_wait(&sh.clc, i & 1u, abort, rounds);
                     if (ok) next = cancelled_cta(&sh.response);
                     else tma_mbar_wait(&sh.clc, i & 1u, kDenseSpin);   // it lands before the CTA exits
                 }
-                ok = ok && dense_wait(&sh.mail_empty[p1], (((i + 1) / kProd) & 1u) ^ 1u, abort, limit);
+                ok = ok && dense_wait(&sh.mail_empty[p1], (((i + 1) / kProd) & 1u) ^ 1u, abort, rounds);
                 if (ok) {
                     sh.mail[p1] = next;
                     mbar_arrive(&sh.mail_full[p1]);
@@ -549,8 +551,8 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
             for (int p = 0; p < kProd; ++p) {
                 for (bool last = false; ok && !end && !last;) {
                     const uint32_t s = sc[p] % kSlots, r = rc % kRows;
-                    ok = __all_sync(FULL, dense_wait(&sh.w_full[p][s], (sc[p] / kSlots) & 1u, abort, limit));
-                    if (ok) ok = __all_sync(FULL, dense_wait(&sh.r_empty[r], ((rc / kRows) & 1u) ^ 1u, abort, limit));
+                    ok = __all_sync(FULL, dense_wait(&sh.w_full[p][s], (sc[p] / kSlots) & 1u, abort, rounds));
+                    if (ok) ok = __all_sync(FULL, dense_wait(&sh.r_empty[r], ((rc / kRows) & 1u) ^ 1u, abort, rounds));
                     if (!ok) break;
                     ++sc[p];
                     ++rc;
@@ -597,7 +599,7 @@ cudaError_t run_block(const qr_frame &f, const void *feat, const float *scale, f
         slot<float>(f, S_REC_H), slot<uint32_t>(f, S_IGID), slot<uint2>(f, S_RANGES),
         static_cast<const unsigned char *>(feat), scale, f.camera.width, f.camera.height,
         f.params.tile_w, f.tiles_x, f.params.alpha_min, f.params.alpha_max, f.params.T_min, out,
-        T_final, stats, slot<uint32_t>(f, S_COUNTERS), wait_limit());
+        T_final, stats, slot<uint32_t>(f, S_COUNTERS), wait_limit() / kPolls);
     count_launch();
     return cudaGetLastError();
 }

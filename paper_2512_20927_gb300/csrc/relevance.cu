@@ -894,7 +894,7 @@ cudaError_t run(const float *map, const uint16_t *q, int64_t P, int C, float *ou
 }  // namespace
 
 void set_wait_limit(unsigned polls) { g_wait_limit = polls ? polls : kSpinLimit; }
-unsigned wait_limit() { return g_wait_limit < 1u << 31 ? g_wait_limit : 1u << 31; }
+unsigned wait_limit() { return g_wait_limit; }
 
 bool blend_relevance_supported(qr_dtype dt, int Q, int C, int K) {
     if (C < FB_CHUNK || C % FB_CHUNK || K < 1 || K > 8) return false;

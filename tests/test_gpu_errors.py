@@ -87,6 +87,14 @@ def test_dense_wait_that_runs_out_reports_timeout_and_recovers(channels, dtype):
         with pytest.raises(q.QRError) as e:
             q.render_frame(gdev, feat, cam, K=8, dense=True)
         assert e.value.code == q.QR_ERR_DEVICE_TIMEOUT
+        # one round of polls: a wait or another may run out, far into the work or
+        # nowhere; the kernel returns either way
+        q.qr_set_wait_limit(1024)
+        for _ in range(3):
+            q.qr_project(fr, *gdev)
+            q.qr_sort(fr)
+            q.qr_dense(fr, table, scale, out, T)
+            assert q.qr_frame_status(fr)[0] in (q.QR_OK, q.QR_ERR_DEVICE_TIMEOUT)
     finally:
         q.qr_set_wait_limit(0)
     q.qr_project(fr, *gdev)
