@@ -497,6 +497,52 @@ def test_dense_subtile_kernel(C, kind, tile):
           f"(oracle {want}), executed/useful FMA {executed / max(blended * C, 1):.2f}")
 
 
+@pytest.mark.parametrize("C,kind,tile", [(64, "f32", (8, 32)), (64, "bf16", (16, 16)), (64, "fp8", (32, 8)),
+                                         (128, "f32", (16, 16)), (128, "fp8", (16, 16)),
+                                         (256, "bf16", (32, 8)), (256, "fp8", (8, 32)),
+                                         (512, "bf16", (16, 16))])
+def test_dense_block_kernel_other_widths(C, kind, tile):
+    """The widths and formats of the block kernel that the test above leaves out."""
+    test_dense_subtile_kernel(C, kind, tile)
+
+
+@pytest.mark.parametrize("kind", ["f32", "bf16", "fp8"])
+@pytest.mark.parametrize("scene", ["deep", "room"])
+def test_dense_kernels_agree_bit_for_bit(kind, scene):
+    """Rows of 64, 128, 256 and 512 channels on the block kernel and of 192 on
+    the slice kernel: the same sums and transmittances for the channels they
+    share, on lists of thousands of entries too, and no timeout."""
+    import torch
+    from paper_2512_20927_gb300 import qrender as q
+    if scene == "deep":
+        g, _ = _slab_scene(6000)
+        cam = scenes.tiny_camera(53, 47)
+    else:
+        g, _ = H.small_room(n=20000, channels=16)
+        cam = scenes.room_camera(150, 110)
+    x = torch.randn((g.n, 512), device="cuda", generator=torch.Generator("cuda").manual_seed(5))
+    table, scale = x, None
+    if kind == "bf16":
+        table = q.qr_quantize_bf16(x)
+    elif kind == "fp8":
+        table, scale = q.qr_quantize_fp8(x)
+    fr = q.render_frame(q.gaussians_to_device(g), None, cam, K=8)["frame"]
+
+    def dense(C):
+        out = torch.full((fr.pixels, C), float("nan"), device="cuda")
+        T = torch.full((fr.pixels,), float("nan"), device="cuda")
+        q.qr_dense(fr, table[:, :C].contiguous(), scale, out, T)
+        assert q.qr_frame_status(fr)[0] == q.QR_OK
+        return out, T
+    want, T = dense(192)
+    assert bool((T < 0.5).any()) and bool(torch.isfinite(want).all())
+    for C in (64, 128, 256, 512):
+        got, Tc = dense(C)
+        n = min(C, 192)
+        assert torch.equal(got[:, :n], want[:, :n]), C
+        assert torch.equal(Tc, T) and bool(torch.isfinite(got).all()), C
+
+
 @pytest.mark.parametrize("dtype,C", [("f32", 512), ("bf16", 512), ("bf16", 1024), ("fp8", 1024),
                                      ("fp8", 512)])
 def test_blend_channel_chunks_bit_identical(dtype, C):
