@@ -82,8 +82,8 @@ cudaError_t launch_project(const qr_frame &f, const float *mean, const float *lo
 cudaError_t launch_sort(const qr_frame &f, cudaStream_t s);
 cudaError_t launch_select(const qr_frame &f, int32_t *ids, float *w, uint8_t *cnt, bool riemann,
                           cudaStream_t s);
-// stats (nullable, wide rows only): [0] += blended (pixel, Gaussian) pairs,
-// [1] += executed (8-pixel group, entry) pairs of the accumulation
+// stats (nullable, rows of the block kernel only): [0] += blended (pixel,
+// Gaussian) pairs, [1] += executed multiply-adds
 cudaError_t launch_dense(const qr_frame &f, const void *feat, const float *scale, qr_dtype dt,
                          int C, float *out, float *T_final, cudaStream_t s,
                          unsigned long long *stats = nullptr);
@@ -206,23 +206,6 @@ __device__ __forceinline__ uint32_t block_inclusive_scan(uint32_t v, uint32_t *s
     total = s_w[nw - 1];
     __syncthreads();
     return r;
-}
-
-// Exclusive scan of `total` u32 in place by one CTA: coalesced chunks of
-// blockDim.x elements with a running carry.  Returns the grand total to
-// thread 0 through *sum_out (nullable).
-__device__ __forceinline__ void cta_exclusive_scan(uint32_t *data, int total, uint32_t *sum_out) {
-    __shared__ uint32_t s_w[32];
-    uint32_t carry = 0;
-    for (int base = 0; base < total; base += blockDim.x) {
-        const int i = base + threadIdx.x;
-        const uint32_t v = i < total ? data[i] : 0u;
-        uint32_t chunk;
-        const uint32_t inc = block_inclusive_scan(v, s_w, chunk);
-        if (i < total) data[i] = carry + inc - v;
-        carry += chunk;
-    }
-    if (sum_out && threadIdx.x == 0) *sum_out = carry;
 }
 
 // Two independent inclusive scans in one pass (x and y of one uint2 per
