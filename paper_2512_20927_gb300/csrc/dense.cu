@@ -379,14 +379,13 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
         unsigned long long n_exec = 0;
         for (uint32_t it = 0;; ++it) {
             const uint32_t r = it % kRows, ph = (it / kRows) & 1u;
-            // one verdict per warp: its lanes meet again below
-            if (!__all_sync(FULL, dense_wait(&sh.r_full[r], ph, abort, rounds))) break;
+            bool ok = dense_wait(&sh.r_full[r], ph, abort, rounds);
             const DenseRow &R = sh.row[r];
-            const int block = R.block, last = R.last, at = R.slot;
-            if (block == kItemEnd) break;
+            const int block = ok ? R.block : kItemEnd, last = R.last, at = ok ? R.slot : 0;
+            ok = block != kItemEnd;
             const DenseSlot &S = sh.slot[0][at];
             const unsigned char *rows = s_rows + size_t(r) * kEnt * ROW + size_t(q0) * QB;
-            uint32_t mask = S.mask[g];
+            uint32_t mask = ok ? S.mask[g] : 0u;
             n_exec += __popc(mask);
             while (mask) {
                 const int e = __ffs(mask) - 1;
@@ -411,7 +410,8 @@ dense_block_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ 
                     }
                 }
             }
-            __syncwarp();
+            // one verdict per warp: its lanes go on, or leave, together
+            if (!__all_sync(FULL, ok)) break;
             if (lane == 0) {
                 mbar_arrive(&sh.r_empty[r]);
                 mbar_arrive(&sh.w_empty[0][at]);

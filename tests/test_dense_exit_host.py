@@ -28,9 +28,9 @@ def _calls(text, name):
 
 
 def test_every_wait_is_voted_by_its_warp():
-    """A wait of all lanes is the argument of a vote, or of the `ok` that the
-    next statement votes on; the waits of lane 0 alone are voted on after its
-    branch."""
+    """A wait is the argument of a vote, or sets the `ok` that is voted on before
+    the lanes part: in the consumers in place of the barrier that ends a slot,
+    in the producers after lane 0's branch."""
     for role, text in _roles().items():
         voted = [c for _, c in _calls(text, "__all_sync")]
         waits = list(_calls(text, "dense_wait"))
@@ -39,7 +39,10 @@ def test_every_wait_is_voted_by_its_warp():
             if any(call in v for v in voted):
                 continue
             assert re.search(r"ok = (ok && )?$", text[:at]), (role, call)
-            assert "ok = __all_sync(FULL, ok);" in text[at:], (role, call)
+            assert "__all_sync(FULL, ok)" in text[at:], (role, call)
+    consumers = _roles()["consumers"]
+    wait, vote = consumers.index("dense_wait("), consumers.index("if (!__all_sync(FULL, ok)) break;")
+    assert not re.search(r"\b(break|continue|return|__syncwarp)\b", consumers[wait:vote])
 
 
 def test_nothing_in_flight_outlives_the_cta():
