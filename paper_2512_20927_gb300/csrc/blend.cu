@@ -3,24 +3,23 @@
 //     out[p] = sum_{j < cnt[p]} w[p][j] * f[ids[p][j]]
 // with the 1/(1 - T^Q) normalisation already folded into w by the selection.
 //
-// GB300 design: this is the bandwidth-bound stage (about zero flops per byte),
-// so the kernel is built around 16-byte vector traffic:
-//   - one warp per pixel (for rows of 512 B or more; narrower rows pack
-//     several pixels into a warp), each lane owning a fixed set of 16-byte
-//     column vectors of the row, so every warp-wide load or store moves 512
-//     contiguous bytes;
-//   - the pixel's ids and weights are read at one address by all of its
-//     lanes (a single L1 broadcast per entry);
-//   - all row loads of a pixel are issued before the FMAs (unrolled by 4
-//     rows) to keep enough bytes in flight per SM;
+// GB300 design: this is the bandwidth-bound stage (about zero flops per byte):
+//   - rows of 512 bytes to 2 KB whose vectors divide evenly (blend_group_kernel):
+//     a warp per group of four pixels, 2 x 2 on screen or consecutive, which reads
+//     each distinct row of their entries once, in quads of 4 channels per lane,
+//     and accumulates it into every pixel that lists it;
+//   - narrower rows (several pixels per warp) and rows of 4 KB (a warp per pixel):
+//     blend_kernel, each lane owning 16-byte vectors of the row, four rows in
+//     flight, a pixel's ids and weights read at one address by all its lanes;
 //   - BF16 rows are widened with bit shifts, FP8 E4M3 rows with the hardware
 //     conversion instructions; FP8 rows fold their per-Gaussian scale into
 //     the weight;
-//   - the map is written with streaming (evict-first) 16-byte stores so it
-//     does not displace the feature rows that neighbouring pixels share in L2;
-//   - one CTA renders one 16x16 screen tile, its warps interleaved over the
-//     tile's pixels, so rows shared by a tile's pixels are re-read from the
-//     SM's L1 instead of L2.
+//   - the map is written with streaming (evict-first) 16-byte stores, 512
+//     contiguous bytes per warp, so it does not displace the feature rows that
+//     neighbouring pixels share in L2;
+//   - one CTA takes one 16x16 screen tile (or 256 consecutive pixels), its warps
+//     interleaved over it, so rows shared by its pixels are re-read from the SM's
+//     L1 instead of L2.
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
 

@@ -416,7 +416,7 @@ eq2_mma(const float *__restrict__ F, const float *__restrict__ tn, int M, int C,
             }
         }
         __syncwarp();
-        // ---------------- 3. gradient rows, 16 pixels x 8 channels at a time
+        // ---------------- 3. gradient rows, 16 pixels x 16 channels at a time
 #pragma unroll
         for (int m2 = 0; m2 < NT / 2; ++m2) {
             const int n0 = 2 * m2, n1 = 2 * m2 + 1;     // n-tiles of rows g and g + 8
