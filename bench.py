@@ -575,7 +575,7 @@ def run_fused_relevance(ctx, hbm_peak, steps=20):
             "fused_frac_of_hbm": round(fused_bytes / fused / 1e6 / hbm_peak, 4),
             "map_bytes_not_written": int(P * C * 4),
             "note": "fused: the blend of each 16x8 pixel block goes to shared memory and "
-                    "through tcgen05 kind::tf32; the 512-D map never reaches HBM"}
+                    "through tcgen05 kind::f16 (BF16); the 512-D map never reaches HBM"}
 
 
 def run_object(local, hbm_peak, steps=20):

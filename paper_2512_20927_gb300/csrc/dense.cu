@@ -228,7 +228,7 @@ dense_kernel(const float4 *__restrict__ rec_m, const float4 *__restrict__ rec_w,
 // Room VGA, 500k Gaussians, 512 FP32 channels (21.5 GFLOP useful, 1.1 times
 // that executed): 1379 us with one CTA per 16 x 4 pixels that walked, staged
 // rows and accumulated 32 list entries (9 survivors) at a time behind named
-// barriers; 566 us now.  The roles alone: consumers 320 us at the FP32 peak,
+// barriers; 556 us now.  The roles alone: consumers 320 us at the FP32 peak,
 // walk and copies without the multiply-adds 326 us.  Five warps per scheduler
 // (20 in all) leave a consumer 96 registers; a 21st warp cost 80 and spills
 // (1096 us), two producers 585 us.  Other rows (slices of 64 channels that walk
@@ -622,7 +622,11 @@ template <int DT>
 cudaError_t dispatch(const qr_frame &f, const void *feat, const float *scale, int C, float *out,
                      float *T_final, unsigned long long *stats, cudaStream_t s) {
     constexpr int cpv = Cpv<DT>::v;
-    // wide rows: one walk per pixel, culled and skipped entries
+    // the block kernel: one walk per pixel, culled and skipped entries.  It wants
+    // C / 4 quads that fill the 32 or 64 lanes of a pixel group's warps (64
+    // channels: half of them) and 64 rows in shared memory, so 64 to 512
+    // channels; widths in between are not instantiated and walk every pixel once
+    // per slice below (room 500k at 100 x 70: 192 channels 468 us, 256 120 us)
     if (C == 512) return run_block<DT, 512>(f, feat, scale, out, T_final, stats, s);
     if (C == 256) return run_block<DT, 256>(f, feat, scale, out, T_final, stats, s);
     if (C == 128) return run_block<DT, 128>(f, feat, scale, out, T_final, stats, s);
